@@ -28,13 +28,16 @@
 // The backward, given the blend masks, runs every 8x4 warp block as its own
 // one-warp CTA: it visits the entries one of its pixels blended, takes each
 // lane's decision from the lane's own mask bit, walks the fragments in
-// reverse recovering T_k by division (Eq. 5), and merges the per-pixel
-// gradients of each Gaussian across the warp with a reduce-scatter
-// butterfly (each level halves the fields a lane carries) before one global
-// atomic per (Gaussian, warp, field).  Without masks a CTA per tile stages
-// the list, visits the entries whose pixel box meets each warp's block and
-// sums the warps in shared memory first.  This replaces the paper's Gradient
+// reverse recovering T_k by division (Eq. 5), and sums the per-pixel terms
+// of each Gaussian over the warp on the tensor cores, four entries at a
+// time, before one global atomic per (Gaussian, warp, field).  Without masks
+// a CTA per tile stages the list, visits the entries whose pixel box meets
+// each warp's block, merges the per-pixel gradients with a reduce-scatter
+// butterfly (each level halves the fields a lane carries) and sums the warps
+// in shared memory first.  This replaces the paper's Gradient
 // Merging Unit (Sec. 5.3).
+#include <stddef.h>
+
 #include <algorithm>
 
 #include "gs_internal.cuh"
@@ -163,6 +166,13 @@ __device__ __forceinline__ Quad quad_form(float ca, float cb, float cc, float dx
 __device__ __forceinline__ float exp2_sfu(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 1 / x with the SFU's rcp instruction (x well inside the normal range).
+__device__ __forceinline__ float rcp_sfu(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -903,114 +913,162 @@ __device__ __forceinline__ x2f x2_fma(x2f a, x2f b, x2f c) {  // a b + c
     return r;
 }
 
-// One warp's staged run for the masked backward: the blended entries'
-// fields, one array per field (slot k: the run's k-th blended entry from the
-// top), so that slots k and k + 1 load as one packed pair.
-struct __align__(16) RunStage {
-    float x[32], y[32], ca[32], cb[32], cc[32], lop[32], dep[32], cr[32], cg[32], cl[32];
-    uint32_t id[32];
+__device__ __forceinline__ x2f x2_dup(float v) { return x2_pack(v, v); }
+
+// The masked backward's working set of one warp: a ring of 64 staged entries
+// (slot s: pair s / 2, half s & 1, so that two consecutive slots load as
+// packed pairs, two fields per 16-byte load) and the (h, w) columns of the
+// step being merged, one row of 32 pixels each.
+struct __align__(16) PwRing {
+    float4 xy[32];     // x0 x1 y0 y1
+    float4 ab[32];     // conic a, b
+    float4 cl[32];     // conic c, log2(opacity)
+    float4 dr[32];     // depth, red
+    float4 gb[32];     // green, blue
+    uint32_t id[64];
+    uint32_t pm[64];   // pixels that blended the entry
+    float op[64];      // opacity (mapping)
+    float col[8][36];  // h0 w0 h1 w1 h2 w2 h3 w3 over the pixels (36: the rows start in different banks)
 };
 
-__device__ __forceinline__ x2f x2_ld(const float* p) { return *reinterpret_cast<const x2f*>(p); }
+__device__ __forceinline__ void x2_ld2(const float4* p, x2f& lo, x2f& hi) {  // one 16-byte load: two packed pairs
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+    lo = v.x;
+    hi = v.y;
+}
 
-// Two consecutive fragments of a warp's run, back to front (slot k + 1 is
-// the earlier entry of the list, so slot k goes first): the geometry and the
-// gradient products of both in packed pairs, with the forward's arithmetic
-// in every half (the same alpha); the transmittance and suffix recursions
-// (Eq. 5) run fragment by fragment as in back_frag.  c0, c1: whether the
-// forward blended them.  Writes each fragment's merged fields to f0, f1.
-template <int MODE>
-__device__ __forceinline__ void back_pair(BackState& S, const RunStage& R, int k, bool c0, bool c1, x2f PXC, x2f PYC,
-                                          const gs_config& cfg, float* f0, float* f1) {
-    const x2f DX = x2_sub(PXC, x2_ld(R.x + k)), DY = x2_sub(PYC, x2_ld(R.y + k));
-    const x2f CA = x2_ld(R.ca + k), CB = x2_ld(R.cb + k), CC = x2_ld(R.cc + k);
+// 32 x 32 bit transpose over the warp: bit p of lane e's result is bit e of
+// lane p's word (five butterfly exchanges; at distance s the partners swap
+// the half words of s-bit groups that belong to the other).
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const uint32_t keep_lo = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu
+                                 : s == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+        const bool up = (lane & s) != 0;
+        const uint32_t keep = up ? ~keep_lo : keep_lo;
+        const uint32_t z = __funnelshift_l(y, y, up ? 32 - s : s);  // the partner's half into place
+        x = (x & keep) | (z & ~keep);
+    }
+    return x;
+}
+
+// d += a b on the tensor cores: a 16 x 8 (row i, column k), b 8 x 8 in tf32,
+// accumulated in float32.  Lane 4 r + c holds a(r, c), a(r + 8, c),
+// a(r, c + 4), a(r + 8, c + 4); b(c, r), b(c + 4, r); d(r, 2 c), d(r, 2 c + 1),
+// d(r + 8, 2 c), d(r + 8, 2 c + 1).
+// FIRST: d = a b.
+template <bool FIRST>
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    if (FIRST)
+        asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+            "{%10, %10, %10, %10};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+    else
+        asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+            "{%0, %1, %2, %3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// v = hi + lo with hi the nearest float of 11 significand bits (a tf32 value;
+// ties away from zero) and lo the exact rest, of which the tensor cores use
+// the first 11 bits: 23 of v's 24 bits in the worst case.
+__device__ __forceinline__ void tf32_split(float v, uint32_t& hi, uint32_t& lo) {
+    hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(v - __uint_as_float(hi));
+}
+
+// Two consecutive fragments of a warp's ring, back to front (slot s first):
+// the geometry of both in packed pairs with the forward's arithmetic in every
+// half (the same alpha), the transmittance and suffix recursions (Eq. 5)
+// fragment by fragment.  c0, c1: whether the forward blended them into this
+// pixel; a fragment that was not keeps the state (alpha 0: T / 1, s + 0).
+// Returns per fragment w = T alpha and h = alpha dL/dalpha = w (c . g - s),
+// the gradient of the exponent (0 where alpha was clamped).
+__device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pair, bool c0, bool c1, x2f PXC, x2f PYC,
+                                          float alpha_max, float& h0, float& w0, float& h1, float& w1) {
+    x2f X, Y, CA, CB, CC, LOP, DEP, CR, CG, CL;
+    x2_ld2(R.xy + pair, X, Y);
+    x2_ld2(R.ab + pair, CA, CB);
+    x2_ld2(R.cl + pair, CC, LOP);
+    x2_ld2(R.dr + pair, DEP, CR);
+    x2_ld2(R.gb + pair, CG, CL);
+    const x2f DX = x2_sub(PXC, X), DY = x2_sub(PYC, Y);
     const x2f A = x2_fma(CB, DY, x2_mul(CA, DX));  // Q d, as quad_form
     const x2f B = x2_fma(CC, DY, x2_mul(CB, DX));
     const x2f Q = x2_fma(DX, A, x2_mul(DY, B));
-    float e0, e1;
-    x2_unpack(x2_fma(Q, x2_pack(R_NEG_HALF_LOG2E, R_NEG_HALF_LOG2E), x2_ld(R.lop + k)), e0, e1);
+    float e0, e1, cg0, cg1;
+    x2_unpack(x2_fma(Q, x2_dup(R_NEG_HALF_LOG2E), LOP), e0, e1);
     const float raw0 = exp2_sfu(e0), raw1 = exp2_sfu(e1);
-    const float al0 = fminf(cfg.alpha_max, raw0), al1 = fminf(cfg.alpha_max, raw1);
-    float d0, d1, r0, r1, g0, g1, b0, b1;
-    x2_unpack(x2_ld(R.dep + k), d0, d1);
-    x2_unpack(x2_ld(R.cr + k), r0, r1);
-    x2_unpack(x2_ld(R.cg + k), g0, g1);
-    x2_unpack(x2_ld(R.cl + k), b0, b1);
-    const float cg0 = __fmaf_rn(d0, S.gD, __fmaf_rn(b0, S.gC2, __fmaf_rn(g0, S.gC1, r0 * S.gC0)));
-    const float cg1 = __fmaf_rn(d1, S.gD, __fmaf_rn(b1, S.gC2, __fmaf_rn(g1, S.gC1, r1 * S.gC0)));
-    S.T = c0 ? __fdividef(S.T, 1.f - al0) : S.T;
-    const float T0 = S.T;
-    const float w0 = c0 ? al0 * S.T : 0.f;
-    const float dif0 = cg0 - S.sg;
-    S.sg = c0 ? __fmaf_rn(al0, dif0, S.sg) : S.sg;
-    S.T = c1 ? __fdividef(S.T, 1.f - al1) : S.T;
-    const float T1 = S.T;
-    const float w1 = c1 ? al1 * S.T : 0.f;
-    const float dif1 = cg1 - S.sg;
-    S.sg = c1 ? __fmaf_rn(al1, dif1, S.sg) : S.sg;
+    x2_unpack(x2_fma(DEP, x2_dup(S.gD),
+                     x2_fma(CL, x2_dup(S.gC2), x2_fma(CG, x2_dup(S.gC1), x2_mul(CR, x2_dup(S.gC0))))),
+              cg0, cg1);
+    const float al0 = c0 ? fminf(alpha_max, raw0) : 0.f, al1 = c1 ? fminf(alpha_max, raw1) : 0.f;
+    // T / (1 - alpha) by the reciprocal instruction (at most 1 ulp) and a
+    // product, as the fast division of back_frag
+    S.T *= rcp_sfu(1.f - al0);
+    w0 = al0 * S.T;
+    const float dif0 = c0 ? cg0 - S.sg : 0.f;
+    S.sg = __fmaf_rn(al0, dif0, S.sg);
+    S.T *= rcp_sfu(1.f - al1);
+    w1 = al1 * S.T;
+    const float dif1 = c1 ? cg1 - S.sg : 0.f;
+    S.sg = __fmaf_rn(al1, dif1, S.sg);
     // the clamp passes no gradient to opacity or shape
-    const bool cl0 = raw0 > cfg.alpha_max, cl1 = raw1 > cfg.alpha_max;
-    const x2f H = x2_mul(x2_pack(cl0 ? 0.f : -0.5f * w0, cl1 ? 0.f : -0.5f * w1), x2_pack(dif0, dif1));
-    const x2f U = x2_mul(H, DX), V = x2_mul(H, DY);
-    x2_unpack(x2_mul(A, H), f0[0], f1[0]);
-    x2_unpack(x2_mul(B, H), f0[1], f1[1]);
-    x2_unpack(x2_mul(U, DX), f0[2], f1[2]);
-    x2_unpack(x2_mul(U, DY), f0[3], f1[3]);
-    x2_unpack(x2_mul(V, DY), f0[4], f1[4]);
-    if (MODE == GS_MAP) {
-        float q0, q1;
-        x2_unpack(Q, q0, q1);
-        f0[5] = (c0 && !cl0) ? exp2_sfu(__fmul_rn(q0, R_NEG_HALF_LOG2E)) * (T0 * dif0) : 0.f;
-        f1[5] = (c1 && !cl1) ? exp2_sfu(__fmul_rn(q1, R_NEG_HALF_LOG2E)) * (T1 * dif1) : 0.f;
-        f0[6] = w0 * S.gD;
-        f0[7] = w0 * S.gC0;
-        f0[8] = w0 * S.gC1;
-        f0[9] = w0 * S.gC2;
-        f1[6] = w1 * S.gD;
-        f1[7] = w1 * S.gC0;
-        f1[8] = w1 * S.gC1;
-        f1[9] = w1 * S.gC2;
-    } else {
-        f0[5] = w0 * S.gD;
-        f1[5] = w1 * S.gD;
-    }
+    h0 = raw0 > alpha_max ? 0.f : w0 * dif0;
+    h1 = raw1 > alpha_max ? 0.f : w1 * dif1;
 }
 
 // Backward compositing of one warp's block of a tile from the forward's
 // per-pixel blend masks (warp w of the tile's).  Pixel-parallel tiles (EP
-// false): the warp's 8x4 block, the masks in the run-major layout.
+// false): the warp's 8x4 (or 4x8) block, the masks in the run-major layout.
 // Entry-parallel tiles of strided frames (EP true): the tile's sampled
 // pixels 32 w .. 32 w + 31 in row-major order, the masks in the
 // entry-parallel forward's pixel-major layout, whose words past a pixel's
 // stopping batch were never written: each lane keeps only the bits before
-// its own last blended position.  The warp walks its runs of 32 list
-// entries from the last one holding an entry one of its pixels blended back
-// to the first.  Per run it stages only those
-// entries, one lane each (the record alone: no box, which the masks make
-// unnecessary), the last first, then evaluates them back to front, 2 NP at
-// a time in packed pairs; a lane's fragment counts when its own mask bit
-// says the forward blended it, so both passes take identical decisions by
+// its own last blended position.
+//
+// The warp walks its runs of 32 list entries from the last one holding an
+// entry one of its pixels blended back to the first.  Per run it stages only
+// those entries, one lane each (the record alone: no box, which the masks
+// make unnecessary), the last first, into a ring, with the pixels that
+// blended each (the run's mask words transposed over the warp).  Steps of
+// four entries leave the ring whenever it holds them, across run borders
+// (only the last step of a warp is padded); a lane's fragment counts when the
+// forward blended it, so both passes take identical decisions by
 // construction, and the alpha it recomputes is the forward's (same staged
-// values, same arithmetic).  The merged fields go straight to grad2d, one
-// atomic per (entry, field, warp): the warps of a tile share nothing and run
-// as one-warp CTAs that the hardware schedules as they free up, heavy tiles
-// first.
-template <int DT, int MODE, int NP, bool EP>
+// values, same arithmetic).
+//
+// The sums over the pixels are a contraction on the tensor cores.  With h and
+// w as in back_pair and pixel p at lattice offset (u, v) from the block's
+// centre (u, v half-integers up to 3.5, so 1, u, v, u u, u v, v v are exact in
+// tf32), every gradient of an entry is a combination of the moments
+// sum_p h {1, u, v, u u, u v, v v} and of sum_p w g, g the pixel's image
+// gradient (depth and colour): rows 0-5 of the left matrix hold the moments'
+// factors, rows 8-11 g's leading tf32 part and rows 12-15 its remainder, and
+// the right matrix holds four entries' (h, w) columns, split into tf32 pairs
+// (tf32_split; the products of two such parts are exact in the float32
+// accumulator).  Against 64-bit sums the split is as close as the float32
+// butterfly it replaced.  That butterfly took 94 instructions for four
+// entries' 24 pose-only fields (82 for two entries' 20 mapping fields) and
+// 13 per entry to form them; the columns, splits, 8 tensor instructions and
+// the moments' recombination take about 85 for four entries in either mode.
+//
+// The recombined gradients go straight to grad2d, one atomic per (entry,
+// field, warp): the warps of a tile share nothing and run as one-warp CTAs
+// that the hardware schedules as they free up, heavy tiles first.
+template <int DT, int MODE, bool EP>
 __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
                                        const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
                                        const float* __restrict__ d_rgb, const float* __restrict__ d_depth,
                                        float* __restrict__ grad2d, const uint32_t* __restrict__ bmask, int tile,
-                                       int w, RunStage& R) {
-    constexpr int NF = Fields<MODE>::N;
-    constexpr int BSTEP = 2 * NP;  // entries per step, merged together
-    static_assert(BSTEP * NF <= 32, "one lane per merged value");
+                                       int w, PwRing& R) {
     const int lane = threadIdx.x & 31;
-    // slots past a run's entries are read by the last step's unused halves:
-    // they must hold finite values (zeros, or an earlier run's records)
-#pragma unroll
-    for (int q = 0; q < (int)(sizeof(RunStage) / 4 / 32); ++q) (&R.x[0])[q * 32 + lane] = 0.f;
-    __syncwarp();
     const int lt = w * 32 + lane;
     PixelMap m;
     if (EP) {
@@ -1026,13 +1084,8 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
     BackState S;
     const uint32_t own = min(back_start(cfg, g, m, t_final, last_idx, d_rgb, d_depth, S), end - start);
-    uint32_t last = own;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+    const uint32_t last = __reduce_max_sync(0xffffffffu, own);
     if (last == 0u) return;  // (warp-uniform) no pixel of the block blended anything
-    const float pxc = (float)m.px + 0.5f, pyc = (float)m.py + 0.5f;
-    const x2f PXC = x2_pack(pxc, pxc), PYC = x2_pack(pyc, pyc);
-    const int owner = merge_owner<BSTEP * NF>();
     // this pixel's word of run r at bm[r rs]
     const uint32_t* bm = EP ? bmask + blend_mask_base_ep(tile, start) + (size_t)lt * ((end - start + 31) >> 5)
                             : bmask + blend_mask_base(tile, start) + lt;
@@ -1044,6 +1097,116 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
                          ? __ldg(vals + start + (uint32_t)r_top * 32u + (uint32_t)lane)
                          : 0u;
     uint32_t bm_nx = __ldg(bm + (size_t)r_top * rs);
+    const float pxc = (float)m.px + 0.5f, pyc = (float)m.py + 0.5f;
+    const x2f PXC = x2_dup(pxc), PYC = x2_dup(pyc);
+    // the left matrix: lane 4 j + c holds row j (moment j) and row j + 8
+    // (image gradient channel j & 3: leading part, j >= 4: remainder) at
+    // pixels 8 c + s and 8 c + 4 + s of step s
+    const int c = lane & 3, j = lane >> 2;
+    const int bw = g.tw < 8 ? 4 : 8;  // the block's width in pixels
+    const float sx = (float)g.sx, sy = (float)g.sy;
+    const float X0 = __shfl_sync(0xffffffffu, pxc, 0) + 0.5f * (float)(bw - 1) * sx;  // the block's centre
+    const float Y0 = __shfl_sync(0xffffffffu, pyc, 0) + 0.5f * (float)(32 / bw - 1) * sy;
+    uint32_t am[4][4];
+    R.col[0][lane] = S.gD;
+    R.col[1][lane] = MODE == GS_MAP ? S.gC0 : 0.f;
+    R.col[2][lane] = MODE == GS_MAP ? S.gC1 : 0.f;
+    R.col[3][lane] = MODE == GS_MAP ? S.gC2 : 0.f;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int q = 8 * c + 4 * b + s;
+            const float u = (float)(q & (bw - 1)) - 0.5f * (float)(bw - 1);
+            const float v = (float)(bw == 8 ? q >> 3 : q >> 2) - 0.5f * (float)(32 / bw - 1);
+            const float f1 = j == 0 ? 1.f : (j == 1 || j == 3 || j == 4) ? u : j < 6 ? v : 0.f;
+            const float f2 = j == 3 ? u : (j == 4 || j == 5) ? v : 1.f;
+            uint32_t hi, lo;
+            tf32_split(R.col[j & 3][q], hi, lo);
+            am[s][2 * b] = __float_as_uint(f1 * f2);
+            am[s][2 * b + 1] = j < 4 ? hi : lo;
+        }
+    __syncwarp();
+    // recombination (see the step): the factor of the lane's own moment
+    const float own_f = j == 3 ? -0.5f * sx * sx : j == 4 ? -sx * sy : j == 5 ? -0.5f * sy * sy : 0.f;
+    // its two coefficients: k1 = ca, cb, -ox / 2, -oy, -oy / 2 and k2 = cb, cc,
+    // 0, -ox, 0 for j = 1..5, (ox, oy) = (X0, Y0) - (x, y)
+    constexpr int AB = offsetof(PwRing, ab) / 4, CL = offsetof(PwRing, cl) / 4;
+    const int slot_off = (c >> 1) * 4 + (c & 1);
+    const int k1o = j == 1 ? AB : j == 2 ? AB + 2 : j == 3 ? 0 : 2;
+    const int k2o = j == 1 ? AB + 2 : j == 2 ? CL : 0;
+    const float k1s = j == 3 || j == 5 ? 0.5f : 1.f, k2s = j == 1 || j == 2 || j == 4 ? 1.f : 0.f;
+    const float k1c = j == 3 ? -0.5f * X0 : j == 4 ? -Y0 : j == 5 ? -0.5f * Y0 : 0.f;
+    const float k2c = j == 4 ? -X0 : 0.f;
+    const float v1f = j == 3 || j == 5 ? 1.f : 0.f;
+
+    // One step: slots g0 .. g0 + 3 of the ring (g0 a multiple of 4), the
+    // first nv of them entries.
+    auto step = [&](int g0, int nv) {
+        const uint4 pm = *reinterpret_cast<const uint4*>(R.pm + g0);
+        const uint32_t bit = 1u << lane;
+        float h[4], wt[4];
+        back_pair(S, R, g0 >> 1, (pm.x & bit) != 0u, (pm.y & bit) != 0u, PXC, PYC, cfg.alpha_max, h[0], wt[0], h[1],
+                  wt[1]);
+        back_pair(S, R, (g0 >> 1) + 1, (pm.z & bit) != 0u, (pm.w & bit) != 0u, PXC, PYC, cfg.alpha_max, h[2], wt[2],
+                  h[3], wt[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {  // (after all of the step's loads)
+            R.col[2 * e][lane] = h[e];
+            R.col[2 * e + 1][lane] = wt[e];
+        }
+        __syncwarp();
+        const float4 va = *reinterpret_cast<const float4*>(&R.col[j][8 * c]);
+        const float4 vb = *reinterpret_cast<const float4*>(&R.col[j][8 * c + 4]);
+        __syncwarp();  // the next step reuses the columns
+        float d[4], dl[4];  // two chains of 4 instead of one of 8
+        const float fa[4] = {va.x, va.y, va.z, va.w}, fb[4] = {vb.x, vb.y, vb.z, vb.w};
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            uint32_t ah, al, bh, bl;
+            tf32_split(fa[s], ah, al);
+            tf32_split(fb[s], bh, bl);
+            if (s == 0) {
+                mma_tf32<true>(d, am[s], ah, bh);
+                mma_tf32<true>(dl, am[s], al, bl);
+            } else {
+                mma_tf32<false>(d, am[s], ah, bh);
+                mma_tf32<false>(dl, am[s], al, bl);
+            }
+        }
+        // lane 4 j + e (e = c): moment j of entry e's h, and sum w g of
+        // channel j & 3 (its two parts on lanes 16 apart)
+        const float mo = d[0] + dl[0];
+        float wg = d[3] + dl[3];
+        wg += __shfl_xor_sync(0xffffffffu, wg, 16);
+        const float M1 = __shfl_sync(0xffffffffu, mo, c);
+        const float MX = sx * __shfl_sync(0xffffffffu, mo, 4 + c);
+        const float MY = sy * __shfl_sync(0xffffffffu, mo, 8 + c);
+        // sums of h dx and h dy about the Gaussian's mean, (dx, dy) = (ox +
+        // sx u, oy + sy v), and the lane's field k1 v1 + k2 v2 + own_f mo:
+        // j = 1, 2 dL/dmean = Q sum h d; j = 3..5 dL/dconic = -(1/2, 1, 1/2)
+        // sum h (dx dx, dx dy, dy dy), with sum h dx dx = sx^2 m_uu + ox (MX +
+        // SX) and likewise; j = 0 dL/ddepth (pose only) or dL/dopacity
+        // (mapping).  k1 and k2 are one staged field each, scaled and shifted.
+        const int slot = g0 + c;
+        const float* fld = reinterpret_cast<const float*>(R.xy + (g0 >> 1)) + slot_off;
+        const float SX = __fmaf_rn(X0 - fld[0], M1, MX), SY = __fmaf_rn(Y0 - fld[2], M1, MY);
+        const float k1 = __fmaf_rn(k1s, fld[k1o], k1c), k2 = __fmaf_rn(k2s, fld[k2o], k2c);
+        const float v1 = __fmaf_rn(v1f, j == 5 ? MY : MX, j == 5 ? SY : SX);
+        const float v2 = j == 4 ? MY : SY;
+        float f = __fmaf_rn(k1, v1, __fmaf_rn(k2, v2, own_f * mo));
+        if (MODE == GS_TRACK && j == 0) f = wg;
+        if (MODE == GS_MAP && j == 0) f = __fdividef(mo, R.op[slot]);  // alpha = opacity e^(-q/2)
+        if (c < nv) {
+            float* dst = grad2d + (size_t)R.id[slot] * GS_GRAD2D_STRIDE;
+            // columns: du dv dA dB dC dop dd . dr dg db
+            if (j < 6 && f != 0.f) atomicAdd(dst + (j == 0 ? (MODE == GS_MAP ? 5 : 6) : j - 1), f);
+            if (MODE == GS_MAP && j < 4 && wg != 0.f) atomicAdd(dst + (j == 0 ? 6 : j + 7), wg);
+        }
+    };
+
+    int head = 0, tail = 0;  // entries stepped over, entries staged
 #pragma unroll 1
     for (int r = r_top; r >= 0; --r) {
         // only bits before the pixel's own last blended position count
@@ -1056,84 +1219,70 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
             id_nx = __ldg(vals + start + (uint32_t)(r - 1) * 32u + (uint32_t)lane);
             bm_nx = __ldg(bm + (size_t)(r - 1) * rs);
         }
-        const unsigned mw = __reduce_or_sync(0xffffffffu, mine);
+        // pixels that blended entry 32 r + lane
+        const uint32_t pix = warp_transpose(mine);
+        const unsigned mw = __ballot_sync(0xffffffffu, pix != 0u);
         if (mw == 0u) continue;
-        // stage the run's blended entries: entry 32 r + lane into slot (its
-        // rank from the top among the run's set bits)
-        if ((mw >> lane) & 1u) {
-            const int slot = __popc(mw & ~((2u << lane) - 1u));
+        // stage the run's blended entries, the last first
+        if (pix != 0u) {
+            const int slot = (tail + __popc(mw & ~((2u << lane) - 1u))) & 63;
             const Splat v = load_splat<DT>(splats, id);
-            R.x[slot] = v.x;
-            R.y[slot] = v.y;
-            R.ca[slot] = v.ca;
-            R.cb[slot] = v.cb;
-            R.cc[slot] = v.cc;
-            R.lop[slot] = log2_opacity(v.op);
-            R.dep[slot] = v.depth;
-            R.cr[slot] = v.r;
-            R.cg[slot] = v.g;
-            R.cl[slot] = v.b;
+            float* const xy = reinterpret_cast<float*>(R.xy + (slot >> 1)) + (slot & 1);
+            float* const ab = reinterpret_cast<float*>(R.ab + (slot >> 1)) + (slot & 1);
+            float* const cl = reinterpret_cast<float*>(R.cl + (slot >> 1)) + (slot & 1);
+            float* const dr = reinterpret_cast<float*>(R.dr + (slot >> 1)) + (slot & 1);
+            float* const gb = reinterpret_cast<float*>(R.gb + (slot >> 1)) + (slot & 1);
+            xy[0] = v.x;
+            xy[2] = v.y;
+            ab[0] = v.ca;
+            ab[2] = v.cb;
+            cl[0] = v.cc;
+            cl[2] = log2_opacity(v.op);
+            dr[0] = v.depth;
+            dr[2] = v.r;
+            gb[0] = v.g;
+            gb[2] = v.b;
             R.id[slot] = id;
+            R.pm[slot] = pix;
+            if (MODE == GS_MAP) R.op[slot] = v.op;
         }
+        tail += __popc(mw);
         __syncwarp();
-        unsigned mq = mw;
-        for (int k = 0; mq; k += BSTEP) {
-            bool cu[BSTEP], has[BSTEP];  // slot k + u: blended here, holds an entry
-#pragma unroll
-            for (int u = 0; u < BSTEP; ++u) {
-                const int bit = mq ? 31 - __clz(mq) : -1;
-                has[u] = bit >= 0;
-                cu[u] = has[u] && ((mine >> (bit & 31)) & 1u);
-                if (has[u]) mq &= ~(1u << bit);
-            }
-            float f[BSTEP * NF];
-#pragma unroll
-            for (int p = 0; p < NP; ++p)
-                back_pair<MODE>(S, R, k + 2 * p, cu[2 * p], cu[2 * p + 1], PXC, PYC, cfg, f + 2 * p * NF,
-                                f + (2 * p + 1) * NF);
-            const float v = warp_merge<BSTEP * NF>(f);
-            if (owner >= 0) {
-                const int u = owner / NF, fl = owner - u * NF;
-                bool valid = has[0];
-#pragma unroll
-                for (int x = 1; x < BSTEP; ++x) valid = u == x ? has[x] : valid;
-                if (valid && v != 0.f)
-                    atomicAdd(grad2d + (size_t)R.id[k + u] * GS_GRAD2D_STRIDE + field_col<MODE>(fl),
-                              v * field_scale(fl));
-            }
-        }
-        __syncwarp();  // the next run reuses the slots
+        // at most 3 entries stay behind, so the next run's 32 find room; the
+        // slots it overwrites were read before the last step's barriers
+#pragma unroll 1
+        for (; tail - head >= 4; head += 4) step(head & 63, 4);
+    }
+    if (tail > head) {  // the last, padded step: no pixel blended the pads
+        if (lane < 4 && lane >= tail - head) R.pm[(head & 63) + lane] = 0u;
+        __syncwarp();
+        step(head & 63, tail - head);
     }
 }
 
-// Pairs per step of the masked backward: two for the pose-only fields (24
-// merged values; 98.0-98.7 us against 99.0 with one pair, and 99.0 for three
-// unpacked entries), one when mapping (20).
-template <int MODE>
-struct PwPairs {
-    static constexpr int N = MODE == GS_TRACK ? 2 : 1;
-};
+// One-warp CTAs of the masked backward per SM: 24 at 80 registers (tracking
+// 640x480 / 200k: 71.7 us, mapping 1200x680 / 1M: 153 us; 32 at 64 registers
+// spill: 88 and 164 us; 28: 75 and 159; 20: 71.9 and 161).  The float32
+// butterfly kernel it replaced took 87 and 210 us.
+#define PW_CTAS 24
 
-// One-warp CTAs: 32 per SM at 64 registers for the pose-only fields; 24 when
-// mapping.
 // Warps per tile of the masked backward.
 __host__ __device__ inline int pw_warps(const Grid& g, bool ep) {
     return ep ? (g.tw * g.th + 31) >> 5 : tile_threads(g) >> 5;
 }
 
 template <int DT, int MODE, bool EP>
-__global__ void __launch_bounds__(32, MODE == GS_TRACK ? 32 : 24)
+__global__ void __launch_bounds__(32, PW_CTAS)
     k_render_bwd_pw(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
                     const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order,
                     const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
                     const float* __restrict__ d_rgb, const float* __restrict__ d_depth, float* __restrict__ grad2d,
                     const uint32_t* __restrict__ bmask) {
-    __shared__ RunStage R;
+    __shared__ PwRing R;
     const int wpt = pw_warps(g, EP);
     const int t = (int)blockIdx.x / wpt, w = (int)blockIdx.x % wpt;
     const int tile = order ? (int)__ldg(order + t) : t;
-    bwd_pw<DT, MODE, PwPairs<MODE>::N, EP>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth,
-                                           grad2d, bmask, tile, w, R);
+    bwd_pw<DT, MODE, EP>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, w, R);
 }
 
 // ---------------------------------------------------------------------------
@@ -1674,17 +1823,17 @@ __global__ void __launch_bounds__(R_THREADS, KST == 1 ? 4 : 2)
 
 // Jobs with blend masks: one-warp CTAs over (job, tile, warp).
 template <bool EP>
-__global__ void __launch_bounds__(32, 32) k_wave_render_bwd_pw(const gs_config cfg,
+__global__ void __launch_bounds__(32, PW_CTAS) k_wave_render_bwd_pw(const gs_config cfg,
                                                                 const __grid_constant__ Wave<WaveBwdJob> W) {
-    __shared__ RunStage R;
+    __shared__ PwRing R;
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveBwdJob& J = W.job[j];
     const int blk = (int)blockIdx.x - W.start[j];
     const int wpt = pw_warps(J.g, EP);
     const int t = blk / wpt, w = blk % wpt;
     const int tile = J.order ? (int)__ldg(J.order + t) : t;
-    bwd_pw<GS_F32, GS_TRACK, PwPairs<GS_TRACK>::N, EP>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx,
-                                                        J.d_rgb, J.d_depth, J.grad2d, J.bmask, tile, w, R);
+    bwd_pw<GS_F32, GS_TRACK, EP>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb, J.d_depth,
+                                 J.grad2d, J.bmask, tile, w, R);
 }
 
 template <int NW>
