@@ -21,13 +21,13 @@
 //                   with shared-memory atomics: no global atomics)
 //   k_tile_sort     bucket sort, heavy first: the remainder keys are unique,
 //                   so any correct sort of them gives the same result.
-//                   One launch: buckets of up to 512 keys take one warp
-//                   each, a merge sort with the keys in registers; up to
-//                   4096 keys one CTA, each warp merge-sorting 256 (8 per
-//                   lane) before the warps merge their runs, up to 8192 the
-//                   same with 512 per warp; longer buckets sort
-//                   8192-key runs in shared memory and merge them by rank
-//                   in global memory.  The sort writes tile_id << 32 |
+//                   One launch, a distribution sort by depth in shared
+//                   memory: a warp a bucket of up to 256 keys, 128 threads
+//                   up to 1024, 256 up to 2048, a CTA of 512 above, in slabs
+//                   of at most 4096 keys where the bucket is longer.  Buckets
+//                   whose depths crowd into one bin are merge sorted instead
+//                   (in registers and shared memory; above 65536 keys also in
+//                   global memory).  The sort writes tile_id << 32 |
 //                   depth_bits and the id.
 // The scatter order inside a bucket depends on atomics, the output does not.
 // Everything stays on the device: the key count is never read by the host.
@@ -39,8 +39,8 @@ namespace gs {
 
 #define BIN_THREADS 256
 #define TS_THREADS 512
-#define TS_SMEM_KEYS 8192
-#define SW_MAX 512               // buckets up to this length sort with one warp
+#define TS_KEYS 4096             // keys a CTA sorts in shared memory at a time
+#define TS_DIST_KEYS 65536       // longer buckets merge sorted runs in global memory
 
 typedef unsigned long long u64;
 
@@ -271,9 +271,9 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
 // alone (the compositing kernels may treat the first tiles of the order
 // differently, and their results must not depend on scheduling).  Finer than
 // whole octaves, it launches the compositing CTAs closer to longest first
-// (tracking step 231.6 -> 226.4 us against octaves).  n_big receives the
-// number of tiles longer than SW_MAX keys, which are exactly the first n_big
-// of the order (SW_MAX + 1 starts a group).
+// (tracking step 231.6 -> 226.4 us against octaves).  n_big[0..3] receive
+// the numbers of tiles longer than 4096, 2048, 1024 and 256 keys, which are
+// exactly the first ones of the order (those lengths end groups).
 #define OG_N 133  // order groups: quarter octaves of the length, then length 1, then empty
 __device__ __forceinline__ int order_group(uint32_t len) {
     if (len == 0) return OG_N - 1;
@@ -297,7 +297,10 @@ __device__ __forceinline__ void tile_order_body(const uint32_t* __restrict__ ran
     if (threadIdx.x == 0) {
         uint32_t run = 0;
         for (int b = 0; b < OG_N; ++b) {
-            if (b == order_group(SW_MAX + 1)) *n_big = run + cnt[b];
+            if (b == order_group(4097)) n_big[0] = run + cnt[b];
+            if (b == order_group(2049)) n_big[1] = run + cnt[b];
+            if (b == order_group(1025)) n_big[2] = run + cnt[b];
+            if (b == order_group(257)) n_big[3] = run + cnt[b];
             cur[b] = run;
             run += cnt[b];
         }
@@ -441,25 +444,6 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter(gs_camera cam, flo
         }
 }
 
-// Bitonic sort of m (power of two) keys in shared memory, ascending.
-__device__ __forceinline__ void bitonic_smem(u64* s, int m) {
-    for (int k = 2; k <= m; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < (m >> 1); i += blockDim.x) {
-                const int lo = 2 * i - (i & (j - 1));
-                const int hi = lo + j;
-                const u64 a = s[lo], b = s[hi];
-                const bool asc = (lo & k) == 0;
-                if ((a > b) == asc) {
-                    s[lo] = b;
-                    s[hi] = a;
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 // Number of keys in sorted run r[0, len) that are < x (lower bound).
 __device__ __forceinline__ int rank_in(const u64* r, int len, u64 x) {
     int lo = 0, hi = len;
@@ -501,21 +485,23 @@ __device__ __forceinline__ void sort_regs(u64 (&v)[KPT]) {
             }
 }
 
-__device__ __forceinline__ void named_bar(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+// Barrier of a sorting group: one warp, or nthreads threads on named
+// barrier `id`.
+__device__ __forceinline__ void group_bar(int id, int nthreads) {
+    if (nthreads == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 // Merge rounds from sorted runs of `run` keys up to one run of nthr * KPT
 // keys.  t: the thread's index in the group; buf: the group's buffer
-// (pad16 of nthr * KPT keys); the group synchronises with __syncwarp when
-// it is one warp, else with named barrier 1 over nthr threads.
+// (pad16 of nthr * KPT keys); bar: the group's barrier.
 template <int KPT>
-__device__ __forceinline__ void merge_rounds(u64 (&v)[KPT], u64* buf, int t, int nthr, int run) {
+__device__ __forceinline__ void merge_rounds(u64 (&v)[KPT], u64* buf, int t, int nthr, int run, int bar) {
     const int M = nthr * KPT;
     for (; run < M; run <<= 1) {
 #pragma unroll
         for (int k = 0; k < KPT; ++k) buf[pad16(t * KPT + k)] = v[k];
-        if (nthr == 32) __syncwarp(); else named_bar(1, nthr);
+        group_bar(bar, nthr);
         const int pair0 = (t * KPT) & ~(2 * run - 1);
         const int diag = t * KPT - pair0;
         const int a0 = pair0, b0 = pair0 + run;
@@ -540,125 +526,304 @@ __device__ __forceinline__ void merge_rounds(u64 (&v)[KPT], u64* buf, int t, int
                 y = j < run ? buf[pad16(b0 + j)] : ~0ull;
             }
         }
-        if (nthr == 32) __syncwarp(); else named_bar(1, nthr);
+        group_bar(bar, nthr);
     }
 }
 
 // Loads a bucket of n <= nthr * KPT keys into the blocked layout (coalesced
 // through buf), padding with ~0.
 template <int KPT>
-__device__ __forceinline__ void load_blocked(const u64* key, int n, u64 (&v)[KPT], u64* buf, int t, int nthr) {
+__device__ __forceinline__ void load_blocked(const u64* key, int n, u64 (&v)[KPT], u64* buf, int t, int nthr, int bar) {
     // all KPT global loads are issued before the first shared store
 #pragma unroll
     for (int r = 0; r < KPT; ++r) v[r] = t + r * nthr < n ? __ldcg(key + t + r * nthr) : ~0ull;
 #pragma unroll
     for (int r = 0; r < KPT; ++r) buf[pad16(t + r * nthr)] = v[r];
-    if (nthr == 32) __syncwarp(); else named_bar(1, nthr);
+    group_bar(bar, nthr);
 #pragma unroll
     for (int k = 0; k < KPT; ++k) v[k] = buf[pad16(t * KPT + k)];
-    if (nthr == 32) __syncwarp(); else named_bar(1, nthr);
+    group_bar(bar, nthr);
 }
 
 // Writes the sorted bucket (coalesced through buf): tile_id << 32 |
-// depth_bits and the id.
+// depth_bits and the id, or with val NULL the remainder keys as they are.
 template <int KPT>
 __device__ __forceinline__ void store_sorted(u64* key, uint32_t* val, int n, u64 hi, const u64 (&v)[KPT], u64* buf,
-                                             int t, int nthr) {
+                                             int t, int nthr, int bar) {
 #pragma unroll
     for (int k = 0; k < KPT; ++k) buf[pad16(t * KPT + k)] = v[k];
-    if (nthr == 32) __syncwarp(); else named_bar(1, nthr);
+    group_bar(bar, nthr);
     for (int x = t; x < n; x += nthr) {
         const u64 w = buf[pad16(x)];
-        key[x] = hi | (w >> 32);
-        val[x] = (uint32_t)w;
+        key[x] = val ? hi | (w >> 32) : w;
+        if (val) val[x] = (uint32_t)w;
     }
 }
 
-template <int KPT>
-__device__ __forceinline__ void warp_sort_bucket(u64* key, uint32_t* val, int n, u64 hi, u64* buf) {
-    const int lane = threadIdx.x & 31;
-    u64 v[KPT];
-    load_blocked<KPT>(key, n, v, buf, lane, 32);
-    sort_regs<KPT>(v);
-    merge_rounds<KPT>(v, buf, lane, 32, KPT);
-    store_sorted<KPT>(key, val, n, hi, v, buf, lane, 32);
+// Merge sort of n <= nthr * 8 keys from src to (key, val) by a group: each
+// warp sorts a run of 256, then the group merges the runs.
+__device__ __noinline__ void merge_sort_group(const u64* src, u64* key, uint32_t* val, int n, u64 hi, u64* buf, int t,
+                                              int nthr, int bar) {
+    u64 v[8];
+    load_blocked<8>(src, n, v, buf, t, nthr, bar);
+    sort_regs<8>(v);
+    merge_rounds<8>(v, buf + pad16((t >> 5) * 256), t & 31, 32, 8, bar);
+    if (nthr > 32) {
+        group_bar(bar, nthr);
+        merge_rounds<8>(v, buf, t, nthr, 256, bar);
+    }
+    store_sorted<8>(key, val, n, hi, v, buf, t, nthr, bar);
 }
 
+// ---------------------------------------------------------------------------
+// Distribution sort of a bucket of n <= 8 TPG keys by a group of TPG threads.
+// The bucket's depth range is cut into at most 8 TPG equal bins (a shift of
+// the depth bits' offset from the smallest: monotone, whatever the bits
+// mean); the keys are counted per bin, the counts scanned, the keys placed
+// bin by bin in shared memory, and each key's place inside its bin is the
+// number of smaller keys there (neighbouring threads hold neighbouring
+// places, so they read the same few keys).  Surfaces cluster the depths:
+// about 8 keys share a bin on the tracking frame, 15 at 3M / 1920x1080.
+// A bin of more than DS_MAX_BIN keys (equal depths, a far outlier) sends the
+// bucket to the merge sort.  About 10 instructions a key and pass instead of
+// 25 dependent shared-memory loads a key and merge round (8 to 12 rounds):
+// 640x480 / 200k (496 k keys) 34.5 -> 13.2 us, 1200x680 / 1M (4.2 M keys)
+// 145 -> 54 us, 1920x1080 / 3M (23.4 M keys) 896 -> 332 us (two CTAs per SM;
+// 15.4, 74 and 465 us with one, 14.4, 54 and 357 with three, which spill;
+// 1024 threads of 4 keys each: 14.4, 62 and 389).
+// src may be key (every key is in registers before the first write).
+// buf: 8 TPG keys, bin: 8 TPG counters, red: 2 words a warp of the group.
+// ---------------------------------------------------------------------------
+#define DS_MAX_BIN 256
 
-// One launch for all buckets.  CTAs below n_big take the long buckets
-// (first in the order), one each; every later CTA takes 16 short buckets,
-// one per warp (both kinds run at once).
+template <int TPG>
+__device__ __forceinline__ void dist_sort_group(const u64* src, u64* key, uint32_t* val, int n, u64 hi, u64* buf,
+                                                uint32_t* bin, uint32_t* red, int t, int bar) {
+    constexpr int KPT = 8, M = TPG * KPT, W = TPG / 32;
+    constexpr int LOGM = TPG == 32 ? 8 : TPG == 128 ? 10 : TPG == 256 ? 11 : 12;
+    static_assert(1 << LOGM == M, "bins per group");
+    const int lane = t & 31, w = t >> 5;
+    u64 v[KPT];
+    uint32_t lo = ~0u, up = 0u;
+#pragma unroll
+    for (int r = 0; r < KPT; ++r)
+        if (t + r * TPG < n) v[r] = __ldcg(src + t + r * TPG);
+#pragma unroll
+    for (int r = 0; r < KPT / 4; ++r) reinterpret_cast<uint4*>(bin)[t + r * TPG] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int r = 0; r < KPT; ++r)
+        if (t + r * TPG < n) {
+            lo = min(lo, (uint32_t)(v[r] >> 32));
+            up = max(up, (uint32_t)(v[r] >> 32));
+        }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    up = __reduce_max_sync(0xffffffffu, up);
+    if (W > 1) {
+        if (lane == 0) {
+            red[w] = lo;
+            red[W + w] = up;
+        }
+        group_bar(bar, TPG);
+        lo = __reduce_min_sync(0xffffffffu, lane < W ? red[lane] : ~0u);
+        up = __reduce_max_sync(0xffffffffu, lane < W ? red[W + lane] : 0u);
+    } else {
+        __syncwarp();
+    }
+    const int sh = max(0, 32 - __clz(up - lo) - LOGM);  // (up - lo) >> sh < M
+#pragma unroll
+    for (int r = 0; r < KPT; ++r)
+        if (t + r * TPG < n) atomicAdd(bin + (((uint32_t)(v[r] >> 32) - lo) >> sh), 1u);
+    group_bar(bar, TPG);
+    // exclusive scan of the counts, 8 consecutive bins a thread
+    uint4 b0 = reinterpret_cast<const uint4*>(bin)[2 * t], b1 = reinterpret_cast<const uint4*>(bin)[2 * t + 1];
+    const uint32_t big = max(max(max(b0.x, b0.y), max(b0.z, b0.w)), max(max(b1.x, b1.y), max(b1.z, b1.w)));
+    const uint32_t sum = b0.x + b0.y + b0.z + b0.w + b1.x + b1.y + b1.z + b1.w;
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    uint32_t run = inc - sum, most = __reduce_max_sync(0xffffffffu, big);
+    if (W > 1) {
+        if (lane == 31) red[w] = inc;  // (every thread has read the range)
+        if (lane == 0) red[W + w] = most;
+        group_bar(bar, TPG);
+        const uint32_t x = lane < W ? red[lane] : 0u;
+        run += __reduce_add_sync(0xffffffffu, lane < w ? x : 0u);
+        most = __reduce_max_sync(0xffffffffu, lane < W ? red[W + lane] : 0u);
+    }
+    if (most > DS_MAX_BIN) {  // (group-uniform)
+        group_bar(bar, TPG);
+        merge_sort_group(src, key, val, n, hi, buf, t, TPG, bar);
+        return;
+    }
+    {
+        uint4 e0, e1;
+        e0.x = run; e0.y = e0.x + b0.x; e0.z = e0.y + b0.y; e0.w = e0.z + b0.z;
+        e1.x = e0.w + b0.w; e1.y = e1.x + b1.x; e1.z = e1.y + b1.y; e1.w = e1.z + b1.z;
+        reinterpret_cast<uint4*>(bin)[2 * t] = e0;
+        reinterpret_cast<uint4*>(bin)[2 * t + 1] = e1;
+    }
+    group_bar(bar, TPG);
+#pragma unroll
+    for (int r = 0; r < KPT; ++r)
+        if (t + r * TPG < n) buf[atomicAdd(bin + (((uint32_t)(v[r] >> 32) - lo) >> sh), 1u)] = v[r];
+    group_bar(bar, TPG);
+    // bin[c] now ends bin c, so bin c starts at bin[c - 1]
+    for (int p = t; p < n; p += TPG) {
+        const u64 k = buf[p];
+        const uint32_t c = ((uint32_t)(k >> 32) - lo) >> sh;
+        const int q0 = c ? (int)bin[c - 1] : 0, q1 = (int)bin[c];
+        int pos = q0;
+        for (int q = q0; q < q1; ++q) pos += buf[q] < k ? 1 : 0;
+        key[pos] = hi | (k >> 32);
+        val[pos] = (uint32_t)k;
+    }
+}
+
+// Shared memory of a sorting CTA: TS_KEYS keys and TS_KEYS counters (the
+// merge sort's padding, one key per 16, lies over the counters).
+#define TS_SMEM (TS_KEYS * (int)(sizeof(u64) + sizeof(uint32_t)))
+
+// Class sizes of the order (heavy first): n_big[0..3] tiles are longer than
+// 4096, 2048, 1024 and 256 keys.
+#define N_CLASS 4
+
+// One launch for all buckets, heavy first: a CTA of 512 threads takes one
+// bucket of more than 2048 keys, two of more than 1024, four of more than 256
+// (128 threads each) or 16 shorter ones (a warp each).
 __device__ __forceinline__ void tile_sort_body(const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order,
-                                               const uint32_t* __restrict__ n_big_p, int ntiles,
+                                               const uint32_t* __restrict__ n_big, int ntiles,
                                                u64* __restrict__ keys, uint32_t* __restrict__ vals,
                                                u64* __restrict__ tmp, int blk) {
     extern __shared__ __align__(16) u64 s[];
-    const int n_big = (int)*n_big_p;
-    if (blk >= n_big) {
-        const int warp = threadIdx.x >> 5;
-        const int idx = n_big + (blk - n_big) * (TS_THREADS / 32) + warp;
-        if (idx >= ntiles) return;
-        const int t = (int)order[idx];
-        const uint32_t b = ranges[2 * t], e = ranges[2 * t + 1];
-        const int n = (int)(e - b);
-        if (n <= 0 || n > SW_MAX) return;
-        const u64 hi = (u64)(uint32_t)t << 32;
-        u64* buf = s + pad16(warp * SW_MAX);
-        if (n <= 32) warp_sort_bucket<1>(keys + b, vals + b, n, hi, buf);
-        else if (n <= 64) warp_sort_bucket<2>(keys + b, vals + b, n, hi, buf);
-        else if (n <= 128) warp_sort_bucket<4>(keys + b, vals + b, n, hi, buf);
-        else if (n <= 256) warp_sort_bucket<8>(keys + b, vals + b, n, hi, buf);
-        else warp_sort_bucket<16>(keys + b, vals + b, n, hi, buf);
-        return;
+    __shared__ uint32_t s_red[2 * TS_THREADS / 32], s_cut[TS_DIST_KEYS / 2048 + 2];
+    uint32_t* const bins = reinterpret_cast<uint32_t*>(s + TS_KEYS);
+    const int tid = (int)threadIdx.x;
+    // the class of this CTA and its first tile in the order
+    int lim = 0, first = 0, per = 1;
+#pragma unroll
+    for (int cl = 0; cl <= N_CLASS; ++cl) {
+        const int end = cl < N_CLASS ? (int)n_big[cl] : ntiles;
+        per = cl < 2 ? 1 : cl == 2 ? 2 : cl == 3 ? 4 : 16;
+        const int blocks = (end - first + per - 1) / per;
+        if (blk < blocks) {
+            lim = end;
+            break;
+        }
+        blk -= blocks;
+        first = end;
     }
-    const int t = (int)order[blk];
-    const uint32_t b = ranges[2 * t], e = ranges[2 * t + 1];
+    if (lim == 0) return;
+    const int TPG = TS_THREADS / per, g = tid / TPG, t = tid % TPG;
+    const int idx = first + blk * per + g;
+    if (idx >= lim) return;
+    const int tile = (int)order[idx];
+    const uint32_t b = ranges[2 * tile], e = ranges[2 * tile + 1];
     const int n = (int)(e - b);
+    if (n <= 0) return;
+    const u64 hi = (u64)(uint32_t)tile << 32;
     u64* key = keys + b;
-    if (n <= 4096) {
-        // m / 256 warps, 8 keys per thread in registers: each warp sorts a
-        // run of 256, then the group merges the runs (half the serial merge
-        // steps per round of 16 keys per thread)
-        int m = 1024;
-        while (m < n) m <<= 1;
-        const int W = m / 256;
-        if ((int)(threadIdx.x >> 5) >= W) return;
-        u64 v[8];
-        load_blocked<8>(key, n, v, s, (int)threadIdx.x, W * 32);
-        sort_regs<8>(v);
-        merge_rounds<8>(v, s + pad16((threadIdx.x >> 5) * 256), (int)(threadIdx.x & 31), 32, 8);
-        merge_rounds<8>(v, s, (int)threadIdx.x, W * 32, 256);
-        store_sorted<8>(key, vals + b, n, (u64)(uint32_t)t << 32, v, s, (int)threadIdx.x, W * 32);
-        return;
-    }
-    if (n <= TS_SMEM_KEYS) {
-        // m / 512 warps, 16 keys per thread in registers: each warp sorts a
-        // run of 512, then the group merges the runs
-        int m = 2 * SW_MAX;
-        while (m < n) m <<= 1;
-        const int W = m / SW_MAX;
-        if ((int)(threadIdx.x >> 5) >= W) return;
-        u64 v[16];
-        load_blocked<16>(key, n, v, s, (int)threadIdx.x, W * 32);
-        sort_regs<16>(v);
-        merge_rounds<16>(v, s + pad16((threadIdx.x >> 5) * SW_MAX), (int)(threadIdx.x & 31), 32, 16);
-        merge_rounds<16>(v, s, (int)threadIdx.x, W * 32, SW_MAX);
-        store_sorted<16>(key, vals + b, n, (u64)(uint32_t)t << 32, v, s, (int)threadIdx.x, W * 32);
-        return;
-    }
-    // long bucket: sorted runs of TS_SMEM_KEYS, then merge by rank
-    for (int c = 0; c < n; c += TS_SMEM_KEYS) {
-        const int len = min(TS_SMEM_KEYS, n - c);
-        for (int i = threadIdx.x; i < TS_SMEM_KEYS; i += blockDim.x) s[i] = i < len ? key[c + i] : ~0ull;
+    uint32_t* val = vals + b;
+    // the group's slice of the shared memory: 8 TPG keys, then as many counters
+    u64* buf = s + (size_t)g * (TS_KEYS / per * 3 / 2);
+    uint32_t* bin = reinterpret_cast<uint32_t*>(buf + TS_KEYS / per);
+    uint32_t* red = s_red + g * (2 * TPG / 32);
+    if (per == 16) return dist_sort_group<32>(key, key, val, n, hi, buf, bin, red, t, 0);
+    if (per == 4) return dist_sort_group<128>(key, key, val, n, hi, buf, bin, red, t, 1 + g);
+    if (per == 2) return dist_sort_group<256>(key, key, val, n, hi, buf, bin, red, t, 1 + g);
+    if (n <= TS_KEYS) return dist_sort_group<512>(key, key, val, n, hi, buf, bin, red, t, 1);
+    // Longer buckets: the keys are first placed bin by bin in tmp (4096 bins
+    // over the depth range), then slabs of whole bins, each starting in its
+    // own 2048 places (so at most 2048 keys and one bin), are sorted alone.
+    if (n <= TS_DIST_KEYS) {
+        uint32_t lo = ~0u, up = 0u;
+        for (int i = tid; i < TS_KEYS; i += TS_THREADS) bins[i] = 0u;
+        for (int i = tid; i < n; i += TS_THREADS) {
+            const uint32_t d = (uint32_t)(__ldcg(key + i) >> 32);
+            lo = min(lo, d);
+            up = max(up, d);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        up = __reduce_max_sync(0xffffffffu, up);
+        constexpr int W = TS_THREADS / 32;
+        const int lane = tid & 31, w = tid >> 5;
+        if (lane == 0) {
+            s_red[w] = lo;
+            s_red[W + w] = up;
+        }
         __syncthreads();
-        bitonic_smem(s, TS_SMEM_KEYS);
-        for (int i = threadIdx.x; i < len; i += blockDim.x) key[c + i] = s[i];
+        lo = __reduce_min_sync(0xffffffffu, lane < W ? s_red[lane] : ~0u);
+        up = __reduce_max_sync(0xffffffffu, lane < W ? s_red[W + lane] : 0u);
+        const int sh = max(0, 32 - __clz(up - lo) - 12);
+        for (int i = tid; i < n; i += TS_THREADS)
+            atomicAdd(bins + (((uint32_t)(__ldcg(key + i) >> 32) - lo) >> sh), 1u);
+        __syncthreads();
+        uint32_t c[8], sum = 0u, big = 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            c[k] = bins[8 * tid + k];
+            sum += c[k];
+            big = max(big, c[k]);
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        uint32_t run = inc - sum, most = __reduce_max_sync(0xffffffffu, big);
+        if (lane == 31) s_red[w] = inc;
+        if (lane == 0) s_red[W + w] = most;
+        __syncthreads();
+        run += __reduce_add_sync(0xffffffffu, lane < w ? s_red[lane] : 0u);
+        most = __reduce_max_sync(0xffffffffu, lane < W ? s_red[W + lane] : 0u);
+        if (most <= 2048u) {  // (CTA-uniform)
+            // slab q starts at the first bin that starts at or after place
+            // 2048 q: the bin before it crosses that place
+            uint32_t at = run;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                bins[8 * tid + k] = at;
+                const uint32_t nx = at + c[k];
+                // places 2048 q in (at, nx]: at most one (a bin holds at most 2048)
+                if ((nx >> 11) != (at >> 11)) s_cut[nx >> 11] = nx;
+                at = nx;
+            }
+            const int slabs = (n + 2047) >> 11;
+            __syncthreads();
+            if (tid == 0) {
+                s_cut[0] = 0u;
+                s_cut[slabs] = (uint32_t)n;
+            }
+            u64* const place = tmp + b;
+            for (int i = tid; i < n; i += TS_THREADS) {
+                const u64 k = __ldcg(key + i);
+                place[atomicAdd(bins + (((uint32_t)(k >> 32) - lo) >> sh), 1u)] = k;
+            }
+            __threadfence_block();
+            __syncthreads();
+            for (int q = 0; q < slabs; ++q) {
+                const uint32_t p0 = s_cut[q], p1 = s_cut[q + 1];
+                if (p1 > p0)
+                    dist_sort_group<512>(place + p0, key + p0, val + p0, (int)(p1 - p0), hi, buf, bin, red, t, 1);
+                __syncthreads();
+            }
+            return;
+        }
+        __syncthreads();
+    }
+    // the longest buckets, and those with a depth shared by more than 2048
+    // keys: sorted runs of TS_KEYS, then merged by rank
+    for (int c = 0; c < n; c += TS_KEYS) {
+        merge_sort_group(key + c, key + c, nullptr, min(TS_KEYS, n - c), hi, s, tid, TS_THREADS, 1);
         __syncthreads();
     }
     __threadfence_block();
     u64* src = key;
     u64* dst = tmp + b;
-    for (int run = TS_SMEM_KEYS; run < n; run <<= 1) {
+    for (int run = TS_KEYS; run < n; run <<= 1) {
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const int pair = i & ~(2 * run - 1);  // run: a power of two
             const int a0 = pair, a1 = min(pair + run, n), b1 = min(pair + 2 * run, n);
@@ -674,7 +839,6 @@ __device__ __forceinline__ void tile_sort_body(const uint32_t* __restrict__ rang
         src = dst;
         dst = w;
     }
-    const u64 hi = (u64)(uint32_t)t << 32;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const u64 v = __ldcg(src + i);
         vals[b + i] = (uint32_t)v;
@@ -685,12 +849,12 @@ __device__ __forceinline__ void tile_sort_body(const uint32_t* __restrict__ rang
         for (int i = threadIdx.x; i < n; i += blockDim.x) key[i] = hi | (key[i] >> 32);
 }
 
-__global__ void __launch_bounds__(TS_THREADS) k_tile_sort(const uint32_t* __restrict__ ranges,
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_sort(const uint32_t* __restrict__ ranges,
                                                           const uint32_t* __restrict__ order,
-                                                          const uint32_t* __restrict__ n_big_p, int ntiles,
+                                                          const uint32_t* __restrict__ n_big, int ntiles,
                                                           u64* __restrict__ keys, uint32_t* __restrict__ vals,
                                                           u64* __restrict__ tmp) {
-    tile_sort_body(ranges, order, n_big_p, ntiles, keys, vals, tmp, (int)blockIdx.x);
+    tile_sort_body(ranges, order, n_big, ntiles, keys, vals, tmp, (int)blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -744,7 +908,7 @@ struct WaveSortJob {
     u64* tmp;
 };
 
-__global__ void __launch_bounds__(TS_THREADS) k_wave_tile_sort(const __grid_constant__ Wave<WaveSortJob> W) {
+__global__ void __launch_bounds__(TS_THREADS, 2) k_wave_tile_sort(const __grid_constant__ Wave<WaveSortJob> W) {
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveSortJob& J = W.job[j];
     tile_sort_body(J.ranges, J.order, J.n_big, J.ntiles, J.keys, J.vals, J.tmp, (int)blockIdx.x - W.start[j]);
@@ -781,7 +945,7 @@ static BinLayout bin_layout(int64_t n, int64_t cap, int ntiles) {
     L.zero_bytes = o;
     L.off_start = o; o = align256(o + sizeof(uint32_t) * (size_t)ntiles);
     L.off_order = o; o = align256(o + sizeof(uint32_t) * (size_t)ntiles);
-    L.off_nbig = o; o = align256(o + sizeof(uint32_t));
+    L.off_nbig = o; o = align256(o + N_CLASS * sizeof(uint32_t));
     L.off_hist = o;
     if (ntiles <= AGG_MAX_TILES) o = align256(o + sizeof(uint32_t) * (size_t)ntiles * (size_t)rows);
     L.off_tmp = o; o = align256(o + sizeof(u64) * (size_t)(cap > 0 ? cap : 1));
@@ -837,11 +1001,11 @@ static gs_status launch_tile_sort(int ntiles, const uint32_t* tile_ranges, const
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
         if (cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((TS_SMEM_KEYS + TS_SMEM_KEYS / 16) * sizeof(u64))) != cudaSuccess)
+                                 TS_SMEM) != cudaSuccess)
             return set_error(GS_ERR_CUDA, "cudaFuncSetAttribute(k_tile_sort)");
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
-    k_tile_sort<<<(unsigned)ntiles, TS_THREADS, (TS_SMEM_KEYS + TS_SMEM_KEYS / 16) * sizeof(u64), st>>>(
+    k_tile_sort<<<(unsigned)ntiles, TS_THREADS, TS_SMEM, st>>>(
         tile_ranges, order, n_big, ntiles, (u64*)keys_out, vals_out, tmp);
     return check_launch("k_tile_sort");
 }
@@ -1135,7 +1299,7 @@ gs_status wave_bin_sort(const gs_track_job* jobs, const WaveBin* bins, int n, cu
         static bool attr_done[64] = {false};
         int dev = 0;
         cudaGetDevice(&dev);
-        const int sm = (int)((TS_SMEM_KEYS + TS_SMEM_KEYS / 16) * sizeof(u64));
+        const int sm = TS_SMEM;
         if (dev < 0 || dev >= 64 || !attr_done[dev]) {
             if (cudaFuncSetAttribute(k_wave_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) != cudaSuccess)
                 return set_error(GS_ERR_CUDA, "cudaFuncSetAttribute(k_wave_tile_sort)");
