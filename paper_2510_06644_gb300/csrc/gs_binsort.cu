@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(1024) k_col_scan(uint32_t* __restrict__ hist, 
 }
 
 // Heavy-first tile order (defined below with the tile scan).
+template <int NW>
 __device__ __forceinline__ void tile_order_body(const uint32_t* __restrict__ ranges, int ntiles,
                                                 uint32_t* __restrict__ order, uint32_t* __restrict__ n_big);
 
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter_rows(gs_camera cam
                                                                    uint32_t* __restrict__ order,
                                                                    uint32_t* __restrict__ n_big) {
     if (blockIdx.x == gridDim.x - 1) {  // the heavy-first order, beside the scatter
-        tile_order_body(ranges, ntiles, order, n_big);
+        tile_order_body<BIN_THREADS / 32>(ranges, ntiles, order, n_big);
         return;
     }
     extern __shared__ uint32_t h[];
@@ -284,30 +285,45 @@ __device__ __forceinline__ int order_group(uint32_t len) {
     return (31 - msb) * 4 + (3 - sub);
 }
 
+template <int NW>  // warps of the CTA
 __device__ __forceinline__ void tile_order_body(const uint32_t* __restrict__ ranges, int ntiles,
                                                 uint32_t* __restrict__ order, uint32_t* __restrict__ n_big) {
     __shared__ uint32_t cnt[OG_N], cur[OG_N];
-    __shared__ uint32_t wcnt[32][OG_N];  // per warp and group, within a 1024-tile chunk
+    __shared__ uint32_t wcnt[NW][OG_N];  // per warp and group, within a chunk of 32 NW tiles
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int b = threadIdx.x; b < OG_N; b += blockDim.x) cnt[b] = 0;
     __syncthreads();
     for (int t = threadIdx.x; t < ntiles; t += blockDim.x)
         atomicAdd(&cnt[order_group(__ldcg(ranges + 2 * t + 1) - __ldcg(ranges + 2 * t))], 1u);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int b = 0; b < OG_N; ++b) {
-            if (b == order_group(4097)) n_big[0] = run + cnt[b];
-            if (b == order_group(2049)) n_big[1] = run + cnt[b];
-            if (b == order_group(1025)) n_big[2] = run + cnt[b];
-            if (b == order_group(257)) n_big[3] = run + cnt[b];
-            cur[b] = run;
-            run += cnt[b];
+    if (warp == 0) {  // exclusive scan of the groups, OG_L a lane
+        constexpr int OG_L = (OG_N + 31) / 32;
+        uint32_t c[OG_L], sum = 0;
+#pragma unroll
+        for (int k = 0; k < OG_L; ++k) {
+            c[k] = OG_L * lane + k < OG_N ? cnt[OG_L * lane + k] : 0u;
+            sum += c[k];
+        }
+        uint32_t run = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += y;
+        }
+        run -= sum;
+#pragma unroll
+        for (int k = 0; k < OG_L; ++k) {
+            const int b = OG_L * lane + k;
+            if (b < OG_N) cur[b] = run;
+            run += c[k];
+            if (b == order_group(4097)) n_big[0] = run;
+            if (b == order_group(2049)) n_big[1] = run;
+            if (b == order_group(1025)) n_big[2] = run;
+            if (b == order_group(257)) n_big[3] = run;
         }
     }
-    const int nw = (int)(blockDim.x >> 5);
-    for (int base = 0; base < ntiles; base += (int)blockDim.x) {
-        for (int q = threadIdx.x; q < 32 * OG_N; q += blockDim.x) (&wcnt[0][0])[q] = 0;
+    for (int base = 0; base < ntiles; base += 32 * NW) {
+        for (int q = threadIdx.x; q < NW * OG_N; q += blockDim.x) (&wcnt[0][0])[q] = 0;
         __syncthreads();
         const int t = base + (int)threadIdx.x;
         const int grp = t < ntiles ? order_group(__ldcg(ranges + 2 * t + 1) - __ldcg(ranges + 2 * t)) : OG_N;
@@ -317,7 +333,7 @@ __device__ __forceinline__ void tile_order_body(const uint32_t* __restrict__ ran
         __syncthreads();
         for (int b = threadIdx.x; b < OG_N; b += blockDim.x) {  // exclusive scan over the warps, per group
             uint32_t run = cur[b];
-            for (int w = 0; w < nw; ++w) {
+            for (int w = 0; w < NW; ++w) {
                 const uint32_t v = wcnt[w][b];
                 wcnt[w][b] = run;
                 run += v;
@@ -332,7 +348,7 @@ __device__ __forceinline__ void tile_order_body(const uint32_t* __restrict__ ran
 
 __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict__ ranges, int ntiles,
                                                      uint32_t* __restrict__ order, uint32_t* __restrict__ n_big) {
-    tile_order_body(ranges, ntiles, order, n_big);
+    tile_order_body<32>(ranges, ntiles, order, n_big);
 }
 
 // The column scan followed, in the CTA that finishes last (ticket; every
@@ -362,7 +378,7 @@ __device__ __forceinline__ void col_scan_tail_body(uint32_t* __restrict__ hist, 
     __threadfence();
     tile_scan_body(total, ntiles, T.cap, T.start, T.ranges, T.n_keys, T.status);
     __syncthreads();
-    if (T.order) tile_order_body(T.ranges, ntiles, T.order, T.n_big);  // else the scatter's extra CTA
+    if (T.order) tile_order_body<32>(T.ranges, ntiles, T.order, T.n_big);  // else the scatter's extra CTA
     if (threadIdx.x == 0) *T.ticket = 0u;
 }
 
@@ -373,55 +389,78 @@ __global__ void __launch_bounds__(1024) k_col_scan_tail(uint32_t* __restrict__ h
 
 // k_tile_scatter_rows with the rects the fused projection kept (no
 // geometry re-read, no tile-rect arithmetic): only the depth is loaded.
+// Block 0 computes the heavy-first order beside the scatter.  The others
+// cover `nrow` groups of per_cta Gaussians for each of the bands of `band`
+// tile rows, one band after the other: the keys' 8-byte writes land all over
+// their band's buckets, so a band is what L2 holds at once (written as one
+// region of 188 MB, the 23.4 M keys of 1920x1080 / 3M took 582 us, 340 MB of
+// it reads of partly written lines).
+struct ScatterArgs {
+    int TX;
+    const void* splats;
+    int64_t n, per_cta;
+    int nrow, ntiles, band;  // groups of Gaussians; tiles; tile rows per band
+    const uint32_t* start;
+    const uint32_t* hist;
+    const uint2* rects;
+    int64_t cap;
+    u64* keys;
+    const uint32_t* ranges;
+    uint32_t* order;
+    uint32_t* n_big;
+};
+
 template <int DT>
-__device__ __forceinline__ void scatter_rects_body(int TX, const void* __restrict__ splats, int64_t n,
-                                                   int64_t per_cta, int ntiles, const uint32_t* __restrict__ start,
-                                                   const uint32_t* __restrict__ hist,
-                                                   const uint2* __restrict__ rects, int64_t cap,
-                                                   u64* __restrict__ keys, const uint32_t* __restrict__ ranges,
-                                                   uint32_t* __restrict__ order, uint32_t* __restrict__ n_big,
-                                                   int blk, int nblk) {
-    if (blk == nblk - 1) {  // the heavy-first order, beside the scatter
-        tile_order_body(ranges, ntiles, order, n_big);
+__device__ __forceinline__ void scatter_rects_body(const ScatterArgs& A, int blk) {
+    if (blk == 0) {
+        tile_order_body<BIN_THREADS / 32>(A.ranges, A.ntiles, A.order, A.n_big);
         return;
     }
-    extern __shared__ uint32_t h[];
-    uint32_t* base = h + ntiles;
-    const uint32_t* row = hist + (size_t)blk * ntiles;
-    for (int t = threadIdx.x; t < ntiles; t += blockDim.x) {
-        h[t] = 0;
-        base[t] = start[t] + row[t];
-    }
+    extern __shared__ uint32_t h[];  // next free place of each of the band's tiles
+    const int grp = (blk - 1) % A.nrow, yb = (blk - 1) / A.nrow * A.band;
+    const int t0 = yb * A.TX, nt = min(A.ntiles - t0, A.band * A.TX);
+    const uint32_t* row = A.hist + (size_t)grp * A.ntiles + t0;
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) h[t] = A.start[t0 + t] + row[t];
     __syncthreads();
-    const int64_t k0 = (int64_t)blk * per_cta, k1 = min(n, k0 + per_cta);
-    for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-        const uint2 r = __ldg(rects + k);
-        const int x0 = (int)(r.x & 0xffffu), x1 = (int)(r.x >> 16), y0 = (int)(r.y & 0xffffu), y1 = (int)(r.y >> 16);
-        if (x1 <= x0) continue;
-        const float depth = DT == GS_F32 ? __ldg(reinterpret_cast<const float*>(splats) + 12 * (size_t)k + 6)
-                                         : __ldg(reinterpret_cast<const float*>(splats) + 8 * (size_t)k + 2);
-        const u64 rem = ((u64)__float_as_uint(depth) << 32) | (u64)(uint32_t)k;
-        for (int ty = y0; ty < y1; ++ty)
-            for (int tx = x0; tx < x1; ++tx) {
-                const int t = ty * TX + tx;
-                const u64 pos = (u64)base[t] + atomicAdd(h + t, 1u);
-                if ((int64_t)pos < cap) keys[pos] = rem;
-            }
+    const int64_t k0 = (int64_t)grp * A.per_cta, k1 = min(A.n, k0 + A.per_cta);
+    for (int64_t kb = k0; kb < k1; kb += blockDim.x) {
+        const int64_t k = kb + threadIdx.x;
+        int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
+        float depth = 0.f;
+        if (k < k1) {
+            const uint2 r = __ldg(A.rects + k);
+            x0 = (int)(r.x & 0xffffu);
+            x1 = (int)(r.x >> 16);
+            y0 = max((int)(r.y & 0xffffu), yb);
+            y1 = max(min((int)(r.y >> 16), yb + A.band), y0);
+            if (x1 > x0 && y1 > y0)
+                depth = DT == GS_F32 ? __ldg(reinterpret_cast<const float*>(A.splats) + 12 * (size_t)k + 6)
+                                     : __ldg(reinterpret_cast<const float*>(A.splats) + 8 * (size_t)k + 2);
+        }
+        const uint32_t kw = (uint32_t)(kb + (threadIdx.x & ~31u));  // the id: lane o's Gaussian is kw + o
+        warp_rect_tiles(x0, y0 - yb, x1 - x0, y1 - y0, __float_as_uint(depth), [&](int tx, int ty, uint32_t d, uint32_t o) {
+            const u64 pos = (u64)atomicAdd(h + ty * A.TX + tx, 1u);
+            if ((int64_t)pos < A.cap) A.keys[pos] = ((u64)d << 32) | (u64)(kw + o);
+        });
     }
 }
 
 template <int DT>
-__global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter_rects(int TX, const void* __restrict__ splats, int64_t n,
-                                                                    int64_t per_cta, int ntiles,
-                                                                    const uint32_t* __restrict__ start,
-                                                                    const uint32_t* __restrict__ hist,
-                                                                    const uint2* __restrict__ rects, int64_t cap,
-                                                                    u64* __restrict__ keys,
-                                                                    const uint32_t* __restrict__ ranges,
-                                                                    uint32_t* __restrict__ order,
-                                                                    uint32_t* __restrict__ n_big) {
-    scatter_rects_body<DT>(TX, splats, n, per_cta, ntiles, start, hist, rects, cap, keys, ranges, order, n_big,
-                           (int)blockIdx.x, (int)gridDim.x);
+__global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter_rects(const ScatterArgs A) {
+    scatter_rects_body<DT>(A, (int)blockIdx.x);
+}
+
+// Tile rows per band of the scatter (see ScatterArgs): one band for every 20
+// MB of keys the capacity allows, at most 6 (every band reads the rects
+// again).  Scatter times by number of bands: 1200x680 / 1M (capacity 51 MB) 1
+// band 55 us, 2 43.7, 4 47, 7 60; 1296x968 / 750k (48 MB) 49, 2 40, 3 37, 6 44;
+// 1200x680 / 458k at stride 2 (22 MB) 21.7, 2 19.6; 1920x1080 / 3M (384 MB) 3
+// bands 307, 6 263, 12 277, 24 392.
+static int scatter_band(const Grid& g, int64_t cap) {
+    const int64_t per = 20 << 20;
+    const int64_t want = (cap * (int64_t)sizeof(u64) + per - 1) / per;
+    const int64_t bands = std::min<int64_t>(std::max<int64_t>(std::min<int64_t>(want, 6), 1), g.TY);
+    return (int)((g.TY + bands - 1) / bands);
 }
 
 template <int DT>
@@ -875,27 +914,9 @@ __global__ void __launch_bounds__(1024) k_wave_col_scan_tail(const __grid_consta
                        W.start[j + 1] - W.start[j]);
 }
 
-struct WaveScatterJob {
-    int TX;
-    const void* splats;
-    int64_t n, per;
-    int ntiles;
-    const uint32_t* start;
-    const uint32_t* hist;
-    const uint2* rects;
-    int64_t cap;
-    u64* keys;
-    const uint32_t* ranges;
-    uint32_t* order;
-    uint32_t* n_big;
-};
-
-__global__ void __launch_bounds__(BIN_THREADS) k_wave_scatter_rects(const __grid_constant__ Wave<WaveScatterJob> W) {
+__global__ void __launch_bounds__(BIN_THREADS) k_wave_scatter_rects(const __grid_constant__ Wave<ScatterArgs> W) {
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
-    const WaveScatterJob& J = W.job[j];
-    scatter_rects_body<GS_F32>(J.TX, J.splats, J.n, J.per, J.ntiles, J.start, J.hist, J.rects, J.cap, J.keys,
-                               J.ranges, J.order, J.n_big, (int)blockIdx.x - W.start[j],
-                               W.start[j + 1] - W.start[j]);
+    scatter_rects_body<GS_F32>(W.job[j], (int)blockIdx.x - W.start[j]);
 }
 
 struct WaveSortJob {
@@ -983,9 +1004,10 @@ static gs_status set_agg_smem_attrs() {
     bool ok = cudaFuncSetAttribute(k_tile_scatter_rows<GS_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
               cudaFuncSetAttribute(k_tile_scatter_rows<GS_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
               cudaFuncSetAttribute(k_tile_scatter_rows<GS_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-              cudaFuncSetAttribute(k_tile_scatter_rects<GS_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-              cudaFuncSetAttribute(k_tile_scatter_rects<GS_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-              cudaFuncSetAttribute(k_tile_scatter_rects<GS_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+              cudaFuncSetAttribute(k_tile_scatter_rects<GS_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes / 2) == cudaSuccess &&
+              cudaFuncSetAttribute(k_tile_scatter_rects<GS_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes / 2) == cudaSuccess &&
+              cudaFuncSetAttribute(k_tile_scatter_rects<GS_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes / 2) == cudaSuccess &&
+              cudaFuncSetAttribute(k_wave_scatter_rects, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes / 2) == cudaSuccess;
     if (!ok) return set_error(GS_ERR_CUDA, "cudaFuncSetAttribute(k_tile_scatter_rows)");
     if (dev >= 0 && dev < 64) done[dev] = true;
     return GS_OK;
@@ -1199,20 +1221,14 @@ extern "C" gs_status gs_project_bin_sort(const gs_config* cfg, const gs_camera* 
     if ((s = check_launch("k_col_scan_tail")) != GS_OK) return s;
     if (keys_capacity == 0) return GS_OK;
     if ((s = set_agg_smem_attrs()) != GS_OK) return s;
-    const size_t sm = 2 * sizeof(uint32_t) * (size_t)ntiles;
-    const uint2* r = (const uint2*)rects;
-    if (rec_dtype == GS_F32)
-        k_tile_scatter_rects<GS_F32><<<nb + 1, BIN_THREADS, sm, st>>>(grid.TX, splats, n, per, ntiles, start, hist, r,
-                                                                     keys_capacity, (u64*)keys_out, tile_ranges,
-                                                                     order, n_big);
-    else if (rec_dtype == GS_BF16)
-        k_tile_scatter_rects<GS_BF16><<<nb + 1, BIN_THREADS, sm, st>>>(grid.TX, splats, n, per, ntiles, start, hist, r,
-                                                                      keys_capacity, (u64*)keys_out, tile_ranges,
-                                                                      order, n_big);
-    else
-        k_tile_scatter_rects<GS_F16><<<nb + 1, BIN_THREADS, sm, st>>>(grid.TX, splats, n, per, ntiles, start, hist, r,
-                                                                     keys_capacity, (u64*)keys_out, tile_ranges,
-                                                                     order, n_big);
+    const int band = scatter_band(grid, keys_capacity);
+    const ScatterArgs A = {grid.TX, splats, n, per, (int)nb, ntiles, band, start, hist, (const uint2*)rects, keys_capacity,
+                           (u64*)keys_out, tile_ranges, order, n_big};
+    const unsigned blocks = 1u + nb * (unsigned)((grid.TY + band - 1) / band);
+    const size_t sm = sizeof(uint32_t) * (size_t)grid.TX * (size_t)band;
+    if (rec_dtype == GS_F32) k_tile_scatter_rects<GS_F32><<<blocks, BIN_THREADS, sm, st>>>(A);
+    else if (rec_dtype == GS_BF16) k_tile_scatter_rects<GS_BF16><<<blocks, BIN_THREADS, sm, st>>>(A);
+    else k_tile_scatter_rects<GS_F16><<<blocks, BIN_THREADS, sm, st>>>(A);
     if ((s = check_launch("k_tile_scatter_rects")) != GS_OK) return s;
     return launch_tile_sort(ntiles, tile_ranges, order, n_big, keys_out, vals_out, tmp, st);
 }
@@ -1269,30 +1285,24 @@ gs_status wave_bin_sort(const gs_track_job* jobs, const WaveBin* bins, int n, cu
         if ((s = check_launch("k_wave_col_scan_tail")) != GS_OK) return s;
     }
     {
-        static bool attr_done[64] = {false};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-            if (cudaFuncSetAttribute(k_wave_scatter_rects, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(2 * AGG_MAX_TILES * sizeof(uint32_t))) != cudaSuccess)
-                return set_error(GS_ERR_CUDA, "cudaFuncSetAttribute(k_wave_scatter_rects)");
-            if (dev >= 0 && dev < 64) attr_done[dev] = true;
-        }
-        Wave<WaveScatterJob> W;
+        if ((s = set_agg_smem_attrs()) != GS_OK) return s;
+        Wave<ScatterArgs> W;
         W.n = n;
         int blocks = 0, smax = 1;
         for (int j = 0; j < n; ++j) {
             const gs_track_job& t = jobs[j];
             const WaveBin& b = bins[j];
+            const Grid g = make_grid(t.cam);
+            const int band = scatter_band(g, t.keys_capacity);
             W.start[j] = blocks;
-            blocks += (int)b.nb + 1;  // + the CTA that computes the heavy-first order
-            smax = std::max(smax, b.ntiles);
-            W.job[j] = WaveScatterJob{make_grid(t.cam).TX, t.splats, t.g.n, b.per, b.ntiles, b.start, b.hist,
-                                      (const uint2*)b.rects, t.keys_capacity, (u64*)t.keys, t.tile_ranges,
-                                      t.tile_order, b.n_big};
+            blocks += 1 + (int)b.nb * ((g.TY + band - 1) / band);
+            smax = std::max(smax, g.TX * band);
+            W.job[j] = ScatterArgs{g.TX, t.splats, t.g.n, b.per, (int)b.nb, b.ntiles, band, b.start, b.hist,
+                                   (const uint2*)b.rects, t.keys_capacity, (u64*)t.keys, t.tile_ranges, t.tile_order,
+                                   b.n_big};
         }
         W.start[n] = blocks;
-        k_wave_scatter_rects<<<(unsigned)blocks, BIN_THREADS, 2 * sizeof(uint32_t) * (size_t)smax, st>>>(W);
+        k_wave_scatter_rects<<<(unsigned)blocks, BIN_THREADS, sizeof(uint32_t) * (size_t)smax, st>>>(W);
         if ((s = check_launch("k_wave_scatter_rects")) != GS_OK) return s;
     }
     {

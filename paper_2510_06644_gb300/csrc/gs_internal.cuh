@@ -310,6 +310,43 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// Calls f(x, y, pay, o) for every tile (x, y) of every lane's rect of w x h
+// tiles at (x0, y0), pay being the value of the rect's lane o: the warp's tiles are
+// numbered through and dealt to the lanes 32 at a time (a lane finds its
+// tile's rect by a binary search of the running counts), so a rect of many
+// tiles does not hold up 31 idle lanes.  The whole warp calls it; w h = 0 for
+// a lane without a rect.
+template <typename F>
+__device__ __forceinline__ void warp_rect_tiles(int x0, int y0, int w, int h, uint32_t pay, F f) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t area = (uint32_t)(w * h);
+    uint32_t inc = area;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= (uint32_t)o) inc += y;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, inc, 31), exc = inc - area;
+    const uint32_t org = (uint32_t)x0 | ((uint32_t)y0 << 16);
+    for (uint32_t j0 = 0; j0 < total; j0 += 32u) {
+        const uint32_t j = j0 + lane;
+        uint32_t o = 0;  // lanes whose tiles end at or before j
+#pragma unroll
+        for (uint32_t s = 16; s > 0; s >>= 1)
+            if (__shfl_sync(0xffffffffu, inc, (int)(o + s - 1u)) <= j) o += s;
+        const uint32_t ow = __shfl_sync(0xffffffffu, (uint32_t)w, (int)o);
+        const uint32_t og = __shfl_sync(0xffffffffu, org, (int)o);
+        const uint32_t r = j - __shfl_sync(0xffffffffu, exc, (int)o);
+        const uint32_t op = __shfl_sync(0xffffffffu, pay, (int)o);
+        if (j < total) {
+            // r / ow: (r + 1/2) / ow is at least 1 / (2 ow) away from an
+            // integer, far more than its float32 rounding (r < 2^13 tiles)
+            const uint32_t row = ow == 1u ? r : (uint32_t)(((float)r + 0.5f) * __frcp_rn((float)ow));
+            f((int)((og & 0xffffu) + r - row * ow), (int)((og >> 16) + row), op, o);
+        }
+    }
+}
+
 // Warp sum of NF values, scattered over the lanes: at each butterfly level
 // (lane offsets 16, 8, ..., 1) the C values a lane still carries are paired,
 // the lower lanes keeping the first C/2 and the upper lanes the second C/2
