@@ -1045,7 +1045,7 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 //
 // The sums over the pixels are a contraction on the tensor cores.  With h and
 // w as in back_pair and pixel p at lattice offset (u, v) from the block's
-// centre (u, v half-integers up to 3.5, so 1, u, v, u u, u v, v v are exact in
+// centre (u, v half-integers up to 7.5, so 1, u, v, u u, u v, v v are exact in
 // tf32), every gradient of an entry is a combination of the moments
 // sum_p h {1, u, v, u u, u v, v v} and of sum_p w g, g the pixel's image
 // gradient (depth and colour): rows 0-5 of the left matrix hold the moments'
@@ -1103,7 +1103,8 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     // (image gradient channel j & 3: leading part, j >= 4: remainder) at
     // pixels 8 c + s and 8 c + 4 + s of step s
     const int c = lane & 3, j = lane >> 2;
-    const int bw = g.tw < 8 ? 4 : 8;  // the block's width in pixels
+    // the block's width in pixels: the lanes run row by row through it
+    const int bw = EP ? g.tw : (g.tw < 8 ? 4 : 8), lbw = bw == 16 ? 4 : bw == 8 ? 3 : 2;
     const float sx = (float)g.sx, sy = (float)g.sy;
     const float X0 = __shfl_sync(0xffffffffu, pxc, 0) + 0.5f * (float)(bw - 1) * sx;  // the block's centre
     const float Y0 = __shfl_sync(0xffffffffu, pyc, 0) + 0.5f * (float)(32 / bw - 1) * sy;
@@ -1119,7 +1120,7 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
         for (int b = 0; b < 2; ++b) {
             const int q = 8 * c + 4 * b + s;
             const float u = (float)(q & (bw - 1)) - 0.5f * (float)(bw - 1);
-            const float v = (float)(bw == 8 ? q >> 3 : q >> 2) - 0.5f * (float)(32 / bw - 1);
+            const float v = (float)(q >> lbw) - 0.5f * (float)(32 / bw - 1);
             const float f1 = j == 0 ? 1.f : (j == 1 || j == 3 || j == 4) ? u : j < 6 ? v : 0.f;
             const float f2 = j == 3 ? u : (j == 4 || j == 5) ? v : 1.f;
             uint32_t hi, lo;

@@ -29,7 +29,7 @@ def G():
 
 
 @pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 31, 32, 33, 63, 64, 65, 67, 130, 257])
-@pytest.mark.parametrize("sx,sy", [(1, 1), (2, 2), (4, 1)])
+@pytest.mark.parametrize("sx,sy", [(1, 1), (2, 2), (4, 1), (1, 4), (1, 2), (2, 1)])
 @pytest.mark.parametrize("mode", ["track", "map"])
 def test_masked_backward_equals_unmasked_at_step_edges(G, n, sx, sy, mode):
     W, H = 30 * sx, 21 * sy
