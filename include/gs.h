@@ -95,14 +95,15 @@ typedef struct {
     int32_t k_max;      /* largest interval */
     float w_rgb;        /* photometric weight of the loss (Eq. 6) */
     float w_depth;      /* geometric weight of the loss (Eq. 6) */
-    int32_t balance;    /* 1: in downsampled frames (both strides >= 2)
-                           gs_render_fwd reads last_idx on entry as the
+    int32_t balance;    /* 1: in downsampled frames (tiles of at most 64
+                           sampled pixels) gs_render_fwd reads last_idx on entry as the
                            previous iteration's per-pixel list positions and
                            pairs heavy with light pixels on the warps of a
                            tile (the workload scheduling of Sec. 5.2); any
                            content is valid and only changes scheduling,
                            never results.  0: no pairing in the forward.
-                           gs_render_bwd always pairs by its last_idx. */
+                           gs_render_bwd pairs by its last_idx where it
+                           composites such frames tile by tile. */
 } gs_config;
 
 /* 3D Gaussians (Sec. 2.1, Eq. 1), structure of arrays, float32:
@@ -513,8 +514,8 @@ typedef struct {
  * counts, the column scan with the tile scan and order, the key scatter, the
  * bucket sort, the forward compositing with the loss, the backward
  * compositing and the backward projection with the pose step -- one launch
- * each (the compositing ones once per kernel form present: full-resolution
- * tiles, strided tiles of up to 32 or 64 sampled pixels).  Each CTA finds its
+ * each (the backward compositing once per kernel form present; the forward
+ * in one launch whatever the jobs' resolutions and strides).  Each CTA finds its
  * job and its block inside the job from the wave's descriptor table, which
  * travels in the launch's parameter space (no device allocation, no copy).
  * jobs: host array of n_jobs (1..GS_WAVE_MAX) descriptors; the jobs' buffers

@@ -2,28 +2,24 @@
 // (Sec. 4.1, Eq. 6) and A-7 backward compositing (Sec. 2.2, Step 4: Eq. 4,
 // Eq. 5) on sm_103a.
 //
-// Two forms of the compositing, chosen per frame:
+// Two forms of the compositing, chosen per frame (fwd_entry_parallel,
+// bwd_entry_parallel):
 //
-// Pixel-parallel (full resolution, or a stride of 1 in one axis): one pixel
-// per thread; a full 16x16 tile takes a CTA of 256 threads, the smaller
-// tiles of a downsampled frame take groups of 64 or 128 threads of such a
-// CTA, each group with its own named barrier and slice of the staging
-// buffer.  Groups are issued in the heavy-first tile order produced by the
-// binning, so the longest lists start first (the GPU counterpart of the
-// paper's subtile streaming, Sec. 5.2).  Warps cover 8x4 pixel blocks.  The
-// forward stages a tile's sorted list through shared memory in batches of
-// 768 records (4 CTAs per SM; one dummy slot per 32 records); the thread
-// that stages an entry also marks the warp blocks its alpha >= alpha_min
-// ellipse meets (block bits), each warp builds from those bits a mask of the
-// entries it may blend and visits only them, three at a time (their alphas
-// are independent; the blends then run in order without branches; a slot
-// past the word's last entry reads the word's dummy).  The alpha of a
-// fragment is one FMA and one ex2: op e^(-q/2) = 2^(log2 op - q log2(e)/2),
-// with q = d.(Q d) and log2 op staged per entry.  The forward also records,
-// per pixel and run of 32 list entries, the entries it blended (the blend
-// masks).
+// Pixel-parallel: one pixel per thread; a full 16x16 tile takes a CTA of 256
+// threads, the smaller tiles of a downsampled frame share one.  Tiles are
+// issued in the heavy-first order produced by the binning, so the longest
+// lists start first (the GPU counterpart of the paper's subtile streaming,
+// Sec. 5.2).  Warps cover 8x4 pixel blocks.  The forward stages a tile's
+// sorted list in batches, an entry a thread, with a mask per warp of the
+// pixels that can blend the entry; each warp compacts the entries it may
+// blend and composites them in pairs (their geometry in packed f32x2
+// operations), four a step.  The alpha of a fragment is one FMA and one ex2:
+// op e^(-q/2) = 2^(log2 op - q log2(e)/2), with q = d.(Q d) and log2 op staged
+// per entry.  The forward also records, per pixel and run of 32 list entries,
+// the entries it blended (the blend masks).
 //
-// Entry-parallel (both strides >= 2): see the section of that name below.
+// Entry-parallel (tiles of at most 64 sampled pixels): see the section of
+// that name below.
 //
 // The backward, given the blend masks, runs every 8x4 warp block as its own
 // one-warp CTA: it visits the entries one of its pixels blended, takes each
@@ -39,6 +35,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "gs_internal.cuh"
 
@@ -47,9 +44,10 @@ namespace gs {
 #define R_THREADS 256            // largest CTA (16x16 tile)
 #define R_BATCH 1024             // largest batch of entries a tile stages at a time
 #define R_MASKW (R_BATCH / 32)   // mask words of a batch (at most 32: lane q holds word q)
-#define R_FWD_SMEM (48 * 1024)          // forward staging budget per CTA (768 entries: 4 CTAs per SM)
 #define R_BWD_SMEM (70 * 1024)          // backward staging budget per CTA (512 entries: 51 KB, 4 CTAs per SM)
-#define R_STEP 3                 // list entries evaluated side by side in the forward walk
+
+#define EP_B 256     // entries an entry-parallel tile stages per batch (64-pixel
+                     // tiles 512: fewer CTA barriers per list)
 
 struct StagedSplat {
     float4 a;   // x, y, conic_a, conic_b
@@ -192,6 +190,44 @@ __device__ __forceinline__ float raw_alpha(float q, float log2_op) {
     return exp2_sfu(__fmaf_rn(q, R_NEG_HALF_LOG2E, log2_op));
 }
 
+// Two float32 values in one 64-bit register for the packed f32x2
+// instructions (add, sub, mul, fma with round-to-nearest: one instruction for
+// both halves, each half rounded exactly as the scalar operation).
+typedef unsigned long long x2f;
+
+__device__ __forceinline__ x2f x2_pack(float lo, float hi) {
+    x2f r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void x2_unpack(x2f v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ x2f x2_sub(x2f a, x2f b) {
+    x2f r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ x2f x2_mul(x2f a, x2f b) {
+    x2f r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ x2f x2_fma(x2f a, x2f b, x2f c) {  // a b + c
+    x2f r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ x2f x2_dup(float v) { return x2_pack(v, v); }
+
+__device__ __forceinline__ x2f x2_ld(const float* p) { return *reinterpret_cast<const x2f*>(p); }
+__device__ __forceinline__ void x2_ld2(const float4* p, x2f& lo, x2f& hi) {  // one 16-byte load: two packed pairs
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+    lo = v.x;
+    hi = v.y;
+}
+
 // Pixel box of a staged Gaussian: its integer 3-sigma box (the definition of
 // which pixels see it), shrunk to the pixels whose centre lies in the
 // axis-aligned bounding box of the ellipse where alpha can reach alpha_min,
@@ -225,91 +261,8 @@ __device__ __forceinline__ int4 pixel_box(const Splat& v, float alpha_min, float
     return box;
 }
 
-// The warp blocks of a group's tile in full-resolution pixels: warp w's
-// block (strip w / wx, column w % wx) spans columns x0 + (w % wx) sxb ..
-// + bw and rows y0 + (w / wx) syb .. + bh (the extents map_pixel gives).
-struct TileBlocks {
-    int x0, y0, bw, bh, sxb, syb, wx, ns;
-};
-
-// (KST == 1: a full-resolution 16x16 tile of 8 warps, compile-time extents)
-template <int KST>
-__device__ __forceinline__ TileBlocks tile_blocks(const Grid& g, int tile, int TT) {
-    const int tx = tile % g.TX, ty = tile / g.TX;
-    TileBlocks b;
-    if (KST == 1) {
-        b.x0 = tx * 16;
-        b.y0 = ty * 16;
-        b.bw = 7;
-        b.bh = 3;
-        b.sxb = 8;
-        b.syb = 4;
-        b.wx = 2;
-        b.ns = 4;
-        return b;
-    }
-    const int BW = g.tw < 8 ? g.tw : 8, BH = 32 / BW, WX = g.tw / BW;
-    b.x0 = tx * g.tw * g.sx;
-    b.y0 = ty * g.th * g.sy;
-    b.bw = (BW - 1) * g.sx;
-    b.bh = (BH - 1) * g.sy;
-    b.sxb = BW * g.sx;
-    b.syb = BH * g.sy;
-    b.wx = WX;
-    b.ns = (TT >> 5) / WX;
-    return b;
-}
-
-// Warp blocks of the tile in which a Gaussian can be blended: bit w when
-// some pixel of warp w's block lies in the Gaussian's box (bx, staged form)
-// and in the region d^T Q d <= t (t = t2 widened by 1 %; t2 < 0: the box
-// alone decides).  Per strip of blocks (a band of rows) the ellipse's x
-// extent over the band follows from its chord [(-cb dy -+ sqrt(t ca - det
-// dy^2)) / ca] at the band's rows closest to the rightmost point (dy = -cb
-// ex / cc) and the leftmost point (dy = cb ex / cc): the chord's right end
-// is concave in dy and its left end convex.  The extent is widened by 1e-2
-// ex + 0.05 px, well beyond the float32 rounding of the fragment test, so
-// the bits never drop a fragment the compositing loop would blend.
-__device__ __forceinline__ unsigned block_bits(const Splat& v, const int4& bx, float t2, const TileBlocks& tb) {
-    const bool ell = t2 > 0.f;
-    const float det = v.ca * v.cc - v.cb * v.cb;
-    float tA = 0.f, ey = 0.f, yr = 0.f, ia = 0.f, sl = 0.f;
-    if (ell) {
-        const float t = t2 * 1.01f;
-        const float ex = sqrtf(t * v.cc / det);
-        tA = t * v.ca;
-        ey = sqrtf(tA / det);
-        yr = -v.cb * ex / v.cc;
-        ia = 1.f / v.ca;
-        sl = 1e-2f * ex + 0.05f;
-    }
-    unsigned bits = 0u;
-#pragma unroll 1
-    for (int s = 0; s < tb.ns; ++s) {
-        const int ry = tb.y0 + s * tb.syb;
-        const int r0 = max(ry, bx.z), r1 = min(ry + tb.bh, bx.z + bx.w);
-        if (r0 > r1) continue;
-        int c0 = bx.x, c1 = bx.x + bx.y;
-        if (ell) {
-            const float ylo = fminf(fmaxf((float)r0 + 0.5f - v.y, -ey), ey);
-            const float yhi = fminf(fmaxf((float)r1 + 0.5f - v.y, -ey), ey);
-            const float dr = fminf(fmaxf(yr, ylo), yhi), dl = fminf(fmaxf(-yr, ylo), yhi);
-            const float xr = (sqrtf(fmaxf(tA - det * dr * dr, 0.f)) - v.cb * dr) * ia;
-            const float xl = (-sqrtf(fmaxf(tA - det * dl * dl, 0.f)) - v.cb * dl) * ia;
-            c0 = max(c0, (int)ceilf(v.x + xl - sl - 0.5f));
-            c1 = min(c1, (int)floorf(v.x + xr + sl - 0.5f));
-        }
-        for (int c = 0; c < tb.wx; ++c) {
-            const int x = tb.x0 + c * tb.sxb;
-            if (c0 <= x + tb.bw && c1 >= x) bits |= 1u << (s * tb.wx + c);
-        }
-    }
-    return bits;
-}
-
-// Stages a Gaussian; with tb (the forward) c.w holds its block bits.
-__device__ __forceinline__ void fill_staged(const Splat& v, float alpha_min, StagedSplat& s,
-                                            const TileBlocks* tb = nullptr) {
+// Stages a Gaussian for the unmasked backward.
+__device__ __forceinline__ void fill_staged(const Splat& v, float alpha_min, StagedSplat& s) {
     s.a = make_float4(v.x, v.y, v.ca, v.cb);
     s.b = make_float4(v.cc, v.op, v.depth, log2_opacity(v.op));
     // the box as (x0, x1 - x0, y0, y1 - y0), clamped far outside any image;
@@ -319,7 +272,7 @@ __device__ __forceinline__ void fill_staged(const Splat& v, float alpha_min, Sta
     const int lo = -(1 << 28), hi = 1 << 28;
     const int x0 = max(bx.x, lo), x1 = min(bx.y, hi), y0 = max(bx.z, lo), y1 = min(bx.w, hi);
     s.box = x1 < x0 || y1 < y0 ? make_int4(hi, 0, hi, 0) : make_int4(x0, x1 - x0, y0, y1 - y0);
-    s.c = make_float4(v.r, v.g, v.b, tb ? __uint_as_float(block_bits(v, s.box, t2, *tb)) : 0.f);
+    s.c = make_float4(v.r, v.g, v.b, 0.f);
 }
 
 // Stages list entries [0, n_in) of `ids` into sp[] (and their ids into sid[]
@@ -327,16 +280,10 @@ __device__ __forceinline__ void fill_staged(const Splat& v, float alpha_min, Sta
 // before it converts any, so KST dependent id -> record loads are in flight
 // per thread (KST = 4 for the small groups of downsampled frames, which
 // stage several entries per thread; 1 for full-resolution tiles).
-// Forward layout of a staged batch: slot 33 q of each run of 32 entries is
-// a dummy that never blends (an empty box), entry e sits at slot il_slot(e):
-// a step slot with no entry left in its word reads the word's dummy instead
-// of testing for one.
-__device__ __forceinline__ int il_slot(int e) { return (e >> 5) * 33 + (e & 31) + 1; }
-
-template <int DT, int KST, bool IL = false>
+template <int DT, int KST>
 __device__ __forceinline__ void stage_batch(const void* __restrict__ splats, const uint32_t* __restrict__ ids,
                                             int n_in, int lt, int TT, float alpha_min, StagedSplat* sp,
-                                            uint32_t* sid, const TileBlocks* tb = nullptr) {
+                                            uint32_t* sid) {
     for (int e0 = lt; e0 < n_in; e0 += KST * TT) {
         uint32_t id[KST];
 #pragma unroll
@@ -348,8 +295,8 @@ __device__ __forceinline__ void stage_batch(const void* __restrict__ splats, con
 #pragma unroll
         for (int k = 0; k < KST; ++k)
             if (e0 + k * TT < n_in) {
-                fill_staged(v[k], alpha_min, sp[IL ? il_slot(e0 + k * TT) : e0 + k * TT], tb);
-                if (sid) sid[e0 + k * TT] = id[k];
+                fill_staged(v[k], alpha_min, sp[e0 + k * TT]);
+                sid[e0 + k * TT] = id[k];
             }
     }
 }
@@ -376,36 +323,6 @@ __device__ __forceinline__ unsigned warp_masks(const StagedSplat* sp, int limit,
         if (lane == q) mine = w;
     }
     return mine;
-}
-
-// The same masks from the block bits of a forward batch (warp wg of its
-// group): entries whose alpha region misses the block are left out too.
-__device__ __forceinline__ unsigned warp_masks_bits(const StagedSplat* sp, int limit, int words, int wg) {
-    const int lane = threadIdx.x & 31;
-    unsigned mine = 0u;
-    const int nq = min(words, (limit + 31) >> 5);  // the words holding entries
-#pragma unroll 4
-    for (int q = 0; q < nq; ++q) {
-        const int e = q * 32 + lane;
-        const bool hit = e < limit && ((__float_as_uint(sp[il_slot(e)].c.w) >> wg) & 1u);
-        const unsigned w = __ballot_sync(0xffffffffu, hit);
-        if (lane == q) mine = w;
-    }
-    return mine;
-}
-
-// Alpha of a staged Gaussian at the pixel (Eq. 2), or -1 when the pixel is
-// outside its box or the exponent is positive (the fragment is skipped).
-__device__ __forceinline__ float frag_alpha(const StagedSplat& s, const PixelMap& m, float pxc, float pyc,
-                                           float alpha_max) {
-    const int4 box = s.box;
-    const float4 A = s.a;
-    const float cc = s.b.x, lop = s.b.w;
-    const Quad Qd = quad_form(A.z, A.w, cc, pxc - A.x, pyc - A.y);
-    const float alpha = fminf(alpha_max, raw_alpha(Qd.q, lop));
-    const bool in = (unsigned)(m.px - box.x) <= (unsigned)box.y && (unsigned)(m.py - box.z) <= (unsigned)box.w &&
-                    !(Qd.q < 0.f);
-    return in ? alpha : -1.f;
 }
 
 // Forward outputs (gs_render_fwd) and, when trgb is given, the fused loss
@@ -435,9 +352,8 @@ __host__ __device__ inline size_t blend_mask_base(int tile, uint32_t start) {
     return (size_t)256 * ((size_t)(start >> 5) + (size_t)tile);
 }
 
-// Entry-parallel tiles (at most 64 sampled pixels) keep one run per pixel
-// instead of one per warp: pixel q of tile t at word 64 (floor(s / 32) + t)
-// + q ceil(len / 32).
+// Tiles of at most 64 sampled pixels keep run r of pixel q (in row order) at
+// word 64 (floor(s / 32) + t) + 64 r + q.
 __host__ __device__ inline size_t blend_mask_base_ep(int tile, uint32_t start) {
     return (size_t)64 * ((size_t)(start >> 5) + (size_t)tile);
 }
@@ -486,106 +402,297 @@ __device__ __forceinline__ void add_loss(const FwdOut& O, float part) {
     if ((threadIdx.x & 31) == 0 && part != 0.f) atomicAdd(O.loss, (double)part);
 }
 
-// Forward compositing of group G's tile, pixel-parallel (sp_all: the CTA's
-// staging buffer, G.B entries plus one dummy per 32 per group).
-template <int DT, int KST>
+// ---------------------------------------------------------------------------
+// Forward compositing, pixel-parallel
+// ---------------------------------------------------------------------------
+// A tile of NW warps (32 NW threads, one pixel each; a CTA of 256 threads
+// serves 8 / NW tiles) stages its list in batches.  The thread that stages an
+// entry also forms, for each warp's block of 32 pixels, the mask of the
+// pixels that can blend it: the entry's pixel box, which the definition makes
+// exact, intersected with its alpha >= alpha_min ellipse, which only saves
+// work.  Each warp then compacts the entries whose mask is not empty, 32 list
+// entries at a time, into pairs of slots of its own, and composites two
+// entries a step: their geometry in packed f32x2 operations (each half the
+// scalar operation), the alpha test, transmittance and blending entry by entry, each
+// lane's box test one bit of the slot's mask.
+//
+// Issue-bound (68 % issue-active, then barriers and fixed latencies): box tests
+// of four words in every lane, scalar geometry and steps of three entries
+// padded with dummies took 74 instructions a (warp, entry) visit, 65.9 M for
+// the tracking frame, against 43.3 M now.  Forward + loss 640x480 / 200k 84 ->
+// 61.4 us, forward 1200x680 / 1M 180 -> 100, 1296x968 / 750k bf16 232 -> 144.  Measured and not kept: records by cp.async a batch ahead (raw records
+// in shared memory cost each warp their unpacking: 61.4 / 105.8 / 152.7), the
+// next batch staged beside the compositing (60.9 / 112 / 157), two entries a
+// step (68.9 / 102 / 146).
+// Staged entries of a tile, an entry a thread.
+template <int NW>
+struct __align__(16) FwdStage {
+    float4 a[32 * NW];           // x, y, conic_a, conic_b
+    float4 col[32 * NW];         // r, g, b, depth
+    float2 cl[32 * NW];          // conic_c, log2(opacity)
+    uint32_t pm[NW][32 * NW];    // per warp: the pixels that can blend the entry
+};
+
+// A warp's compacted entries of one run: slots 2 p and 2 p + 1 as pair p.
+struct __align__(16) FwdSlots {
+    float4 xy[16];   // x0 x1 y0 y1
+    float4 ab[16];   // conic a, b
+    float4 cl[16];   // conic c, log2(opacity)
+    uint4 pb[16];    // pixel masks, run bits
+    float4 col[32];  // r, g, b, depth
+};
+
+__device__ __forceinline__ float sqrt_sfu(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Pixel masks of a Gaussian over the tile's warp blocks: bit p of pm[w] is
+// set when pixel p of warp w's block lies in the Gaussian's box and may lie
+// in the region d^T Q d <= t (t = t2 widened by 1 %; t2 < 0: the box alone).
+// Blocks are 8 x 4 pixels, WX of them across the tile.  Per strip of blocks
+// (a band of rows) the ellipse's x extent over the band follows from its
+// chord [(-cb dy -+ sqrt(t ca - det dy^2)) / ca] at the band's rows closest
+// to the rightmost point (dy = -cb ex / cc) and the leftmost point (dy = cb
+// ex / cc): the chord's right end is concave in dy and its left end convex.
+// The extent is widened by 1e-2 ex + 0.05 px, well beyond the float32
+// rounding of the fragment test, so no pixel the alpha test accepts is
+// dropped.
+template <int NW>
+__device__ __forceinline__ void pixel_masks(const Splat& v, float alpha_min, const Grid& g, int tile,
+                                            uint32_t (&pm)[NW]) {
+#pragma unroll
+    for (int w = 0; w < NW; ++w) pm[w] = 0u;
+    float t2;
+    int4 bx = pixel_box(v, alpha_min, t2);  // x0, x1, y0, y1
+    const int lo = -(1 << 28), hi = 1 << 28;
+    bx = make_int4(max(bx.x, lo), min(bx.y, hi), max(bx.z, lo), min(bx.w, hi));
+    // (NW == 8: 16x16 pixels at stride 1; else 16x8 or 8x16)
+    constexpr int BW = 8;
+    const int sx = NW == 8 ? 1 : g.sx, sy = NW == 8 ? 1 : g.sy, tw = NW == 8 ? 16 : g.tw, th = NW == 8 ? 16 : g.th;
+    const int WX = tw / BW;
+    constexpr int BH = 4;
+    const int tx = tile % g.TX, ty = tile / g.TX;
+    const int X0 = tx * tw * sx, Y0 = ty * th * sy;
+    const bool ell = t2 > 0.f;
+    float det = 0.f, tA = 0.f, ey = 0.f, yr = 0.f, ia = 0.f, sl = 0.f;
+    if (ell) {
+        const float t = t2 * 1.01f;
+        det = v.ca * v.cc - v.cb * v.cb;
+        const float ex = sqrt_sfu(__fdividef(t * v.cc, det));
+        tA = t * v.ca;
+        ey = sqrt_sfu(__fdividef(tA, det));
+        yr = __fdividef(-v.cb * ex, v.cc);
+        ia = rcp_sfu(v.ca);
+        sl = 1e-2f * ex + 0.05f;
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        if (NW != 8 && s * WX >= NW) break;
+        // the strip's rows inside the box: sampled rows jlo .. jhi
+        const int ry = Y0 + s * BH * sy;
+        const int jlo = max(0, ceil_div_i(bx.z - ry, sy)), jhi = min(BH - 1, floor_div(bx.w - ry, sy));
+        if (jlo > jhi) continue;
+        int c0 = bx.x, c1 = bx.y;
+        if (ell) {
+            const float ylo = fminf(fmaxf((float)(ry + jlo * sy) + 0.5f - v.y, -ey), ey);
+            const float yhi = fminf(fmaxf((float)(ry + jhi * sy) + 0.5f - v.y, -ey), ey);
+            const float dr = fminf(fmaxf(yr, ylo), yhi), dl = fminf(fmaxf(-yr, ylo), yhi);
+            const float xr = (sqrt_sfu(fmaxf(tA - det * dr * dr, 0.f)) - v.cb * dr) * ia;
+            const float xl = (-sqrt_sfu(fmaxf(tA - det * dl * dl, 0.f)) - v.cb * dl) * ia;
+            c0 = max(c0, (int)ceilf(v.x + xl - sl - 0.5f));
+            c1 = min(c1, (int)floorf(v.x + xr + sl - 0.5f));
+        }
+        const int ilo = max(0, ceil_div_i(max(c0, lo) - X0, sx)), ihi = min(tw - 1, floor_div(min(c1, hi) - X0, sx));
+        if (ilo > ihi) continue;
+        const uint32_t cols = (2u << ihi) - (1u << ilo);
+        const int rows = jhi - jlo;
+        const uint32_t rsel = (0x01010101u >> (8 * (3 - rows))) << (8 * jlo);
+        // (constant indices, so that pm stays in registers)
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            if (w >= s * WX && w < (s + 1) * WX) pm[w] = ((cols >> ((w - s * WX) * BW)) & ((1u << BW) - 1u)) * rsel;
+    }
+}
+
+template <int DT, int NW>
 __device__ __forceinline__ void fwd_pp(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
-                                       const FwdOut& O, const Group& G, StagedSplat* sp_all) {
-    StagedSplat* sp = sp_all + G.gi * (G.B / 32 * 33);
-    const int tile = G.tile;
-    const PixelMap m = map_pixel(g, tile, G.lt);
-    const TileBlocks tb = tile_blocks<KST>(g, tile, G.TT);
+                                       const FwdOut& O, int tile, FwdStage<NW>& S, FwdSlots& R) {
+    constexpr int TT = 32 * NW;  // a batch: an entry a thread
+    const int lane = threadIdx.x & 31, lt = threadIdx.x % TT, w = lt >> 5, gi = threadIdx.x / TT;
+    const PixelMap m = map_pixel(g, tile, lt);
     const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
-    const float pxc = (float)m.px + 0.5f, pyc = (float)m.py + 0.5f;
-    for (int q = G.lt; q < G.B / 32; q += G.TT) {  // the dummies
-        sp[q * 33].a = make_float4(0.f, 0.f, 0.f, 0.f);
-        sp[q * 33].b = make_float4(0.f, 0.f, 0.f, 0.f);
-        sp[q * 33].c = make_float4(0.f, 0.f, 0.f, 0.f);
-        sp[q * 33].box = make_int4(1 << 28, 0, 1 << 28, 0);
-    }
-    float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, D = 0.f;
+    const x2f PXC = x2_dup((float)m.px + 0.5f), PYC = x2_dup((float)m.py + 0.5f);
+    const uint32_t bit = 1u << lane;
+    const float never = __int_as_float(0x7f800000);
+    float T = 1.f;
+    x2f C01 = x2_dup(0.f), C2D = x2_dup(0.f);
     uint32_t last = 0, nb = 0;
-    bool done = !m.inside;
-    const int words = G.B / 32;
+    float amin = m.inside ? cfg.alpha_min : never;  // `never`: the pixel has stopped
     // this pixel's blend-mask words (run r at bm_pix[r TT])
-    uint32_t* bm_pix = O.bmask ? O.bmask + blend_mask_base(tile, start) + G.lt : nullptr;
-    for (uint32_t b = start; b < end; b += G.B) {
-        // from the second batch on: a barrier (the previous batch's records
-        // are no longer read) that also ends the tile once every pixel stopped
-        if (b != start && group_count(G, done) == G.TT) break;
-        const int n_in = (int)min((uint32_t)G.B, end - b);
-        stage_batch<DT, KST, true>(splats, vals + b, n_in, G.lt, G.TT, cfg.alpha_min, sp, nullptr, &tb);
-        group_sync(G);
-        if (!__all_sync(0xffffffffu, done)) {
-            const unsigned mword = warp_masks_bits(sp, n_in, words, G.lt >> 5);
-            const uint32_t base = b - start;
-            const int wq = (n_in + 31) >> 5;
+    uint32_t* const bm_pix = O.bmask ? O.bmask + blend_mask_base(tile, start) + lt : nullptr;
+    auto barrier = [&] {
+        if (NW == 8) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + gi), "r"(TT) : "memory");
+    };
+    // this thread's entry of a batch; its id is loaded a batch ahead
+    uint32_t id = start + lt < end ? __ldg(vals + start + lt) : 0u;
+    for (uint32_t b = start; b < end; b += TT) {
+        if (b != start) {
+            // the previous batch is no longer read; every pixel stopped: the tile ends
+            const bool done = amin == never;
+            int stopped;
+            if (NW == 8) stopped = __syncthreads_count(done);
+            else
+                asm volatile("{ .reg .pred p; setp.ne.u32 p, %3, 0; bar.red.popc.u32 %0, %1, %2, p; }"
+                             : "=r"(stopped) : "r"(1 + gi), "r"(TT), "r"((unsigned)done) : "memory");
+            if (stopped == TT) break;
+        }
+        const int n_in = (int)min((uint32_t)TT, end - b);
+        if (lt < n_in) {
+            const Splat v = load_splat<DT>(splats, id);
+            S.a[lt] = make_float4(v.x, v.y, v.ca, v.cb);
+            S.col[lt] = make_float4(v.r, v.g, v.b, v.depth);
+            S.cl[lt] = make_float2(v.cc, log2_opacity(v.op));
+            uint32_t pm[NW];
+            pixel_masks<NW>(v, cfg.alpha_min, g, tile, pm);
+#pragma unroll
+            for (int q = 0; q < NW; ++q) S.pm[q][lt] = pm[q];
+        }
+        if (b + TT + lt < end) id = __ldg(vals + b + TT + lt);
+        barrier();
+        if (__all_sync(0xffffffffu, amin == never)) continue;
+        const uint32_t base = b - start;
 #pragma unroll 1
-            for (int q = 0; q < wq; ++q) {
-                unsigned mq = __shfl_sync(0xffffffffu, mword, q);
-                unsigned bq = 0u;  // entries of word q this pixel blended
-                while (mq) {
-                    // R_STEP entries per step: their alphas do not depend on
-                    // T, so they are evaluated side by side; the blends then
-                    // run in list order without branches (a skipped fragment
-                    // adds zero weight).  Front to back, a fragment with
-                    // alpha >= alpha_min is blended unless it would take T
-                    // below t_eps, where the pixel stops (Eq. 3).
-                    // slot of the next entry, or the word's dummy once none is left
-                    int eu[R_STEP];
-                    float au[R_STEP];
-#pragma unroll
-                    for (int u = 0; u < R_STEP; ++u) {
-                        eu[u] = q * 33 + __ffs(mq);
-                        mq &= mq - 1u;
-                    }
-#pragma unroll
-                    for (int u = 0; u < R_STEP; ++u) au[u] = frag_alpha(sp[eu[u]], m, pxc, pyc, cfg.alpha_max);
-#pragma unroll
-                    for (int u = 0; u < R_STEP; ++u) {
-                        const float alpha = au[u];
-                        const bool valid = !done && alpha >= cfg.alpha_min;
-                        const float Tn = T * (1.f - alpha);
-                        const bool stop = valid && Tn < cfg.t_eps;
-                        const bool ok = valid && !stop;
-                        done = done || stop;
-                        const int e = eu[u];
-                        const float4 Cc = sp[e].c;
-                        const float dep = sp[e].b.z;
-                        const float w = ok ? alpha * T : 0.f;
-                        C0 += w * Cc.x;
-                        C1 += w * Cc.y;
-                        C2 += w * Cc.z;
-                        D += w * dep;
-                        T = ok ? Tn : T;
-                        bq |= ok ? 1u << ((e - q * 33 - 1) & 31) : 0u;
-                    }
-                    if (__all_sync(0xffffffffu, done)) break;
-                }
-                // the count and the last position follow from the word's blended bits
-                nb += __popc(bq);
-                if (bq != 0u) last = base + (uint32_t)(q * 32 + 32 - __clz(bq));
-                // every run up to the one where the warp stops is written (a
-                // run past every pixel's last position is never read)
-                if (bm_pix) bm_pix[(size_t)((base >> 5) + q) * G.TT] = bq;
-                if (__all_sync(0xffffffffu, done)) break;
+        for (int q = 0; q < n_in; q += 32) {
+            const int e = q + lane;
+            const uint32_t pix = e < n_in ? S.pm[w][e] : 0u;
+            const unsigned hit = __ballot_sync(0xffffffffu, pix != 0u);
+            const int cnt = __popc(hit);
+            uint32_t bq = 0u;  // entries of the run this pixel blended
+            if (pix != 0u) {
+                const int slot = __popc(hit & (bit - 1u));
+                const float4 A = S.a[e];
+                const float2 L = S.cl[e];
+                float* const xy = reinterpret_cast<float*>(R.xy + (slot >> 1)) + (slot & 1);
+                float* const ab = reinterpret_cast<float*>(R.ab + (slot >> 1)) + (slot & 1);
+                float* const cl = reinterpret_cast<float*>(R.cl + (slot >> 1)) + (slot & 1);
+                uint32_t* const pb = reinterpret_cast<uint32_t*>(R.pb + (slot >> 1)) + (slot & 1);
+                xy[0] = A.x;
+                xy[2] = A.y;
+                ab[0] = A.z;
+                ab[2] = A.w;
+                cl[0] = L.x;
+                cl[2] = L.y;
+                pb[0] = pix;
+                pb[2] = bit;
+                R.col[slot] = S.col[e];
             }
+            if ((cnt & 1) && lane == cnt) {  // the last pair's empty half
+                reinterpret_cast<uint32_t*>(R.pb + (cnt >> 1))[1] = 0u;
+                R.col[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            __syncwarp();
+            // NP pairs of entries from pair p
+            auto step = [&](auto NP_, int p) {
+                constexpr int NP = decltype(NP_)::value;
+                float al[2 * NP];  // the alphas do not depend on T
+                bool in[2 * NP];
+                uint32_t rb[2 * NP];
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    x2f X, Y, CA, CB, CC, LOP;
+                    x2_ld2(R.xy + p + h, X, Y);
+                    x2_ld2(R.ab + p + h, CA, CB);
+                    x2_ld2(R.cl + p + h, CC, LOP);
+                    const uint4 pb = R.pb[p + h];
+                    const x2f DX = x2_sub(PXC, X), DY = x2_sub(PYC, Y);
+                    const x2f QA = x2_fma(CB, DY, x2_mul(CA, DX));  // Q d, as quad_form
+                    const x2f QB = x2_fma(CC, DY, x2_mul(CB, DX));
+                    const x2f Q = x2_fma(DX, QA, x2_mul(DY, QB));
+                    float q0, q1, e0, e1;
+                    x2_unpack(Q, q0, q1);
+                    x2_unpack(x2_fma(Q, x2_dup(R_NEG_HALF_LOG2E), LOP), e0, e1);
+                    al[2 * h] = fminf(cfg.alpha_max, exp2_sfu(e0));
+                    al[2 * h + 1] = fminf(cfg.alpha_max, exp2_sfu(e1));
+                    in[2 * h] = (pb.x & bit) != 0u && !(q0 < 0.f);
+                    in[2 * h + 1] = (pb.y & bit) != 0u && !(q1 < 0.f);
+                    rb[2 * h] = pb.z;
+                    rb[2 * h + 1] = pb.w;
+                }
+                // Front to back: a fragment in the box with alpha >= alpha_min
+                // is blended unless it would take T below t_eps, where the
+                // pixel stops (Eq. 3); a skipped one has factor 1 and adds
+                // zero weight.
+#pragma unroll
+                for (int u = 0; u < 2 * NP; ++u) {
+                    const bool valid = in[u] && al[u] >= amin;
+                    const float Tn = T * (1.f - al[u]);
+                    const bool stop = valid && Tn < cfg.t_eps;
+                    const bool ok = valid && !stop;
+                    const x2f W = x2_dup(ok ? al[u] * T : 0.f);
+                    const float4 c = R.col[2 * p + u];
+                    C01 = x2_fma(W, x2_pack(c.x, c.y), C01);
+                    C2D = x2_fma(W, x2_pack(c.z, c.w), C2D);
+                    T = ok ? Tn : T;
+                    amin = stop ? never : amin;
+                    bq |= ok ? rb[u] : 0u;
+                }
+            };
+            int p = 0;
+#pragma unroll 1
+            for (; 2 * p + 2 < cnt; p += 2) step(std::integral_constant<int, 2>(), p);
+            if (2 * p < cnt) step(std::integral_constant<int, 1>(), p);
+            // the count and the last position follow from the run's blended bits
+            nb += __popc(bq);
+            if (bq != 0u) last = base + (uint32_t)(q + 32 - __clz(bq));
+            // every run up to the one where the warp stops is written (a
+            // run past every pixel's last position is never read)
+            if (bm_pix) bm_pix[(size_t)((base + q) >> 5) * TT] = bq;
+            if (__all_sync(0xffffffffu, amin == never)) break;
+            __syncwarp();  // the next run reuses the slots
         }
     }
+    float C0, C1, C2, D;
+    x2_unpack(C01, C0, C1);
+    x2_unpack(C2D, C2, D);
     float lpart = 0.f;
     if (m.inside) lpart = write_pixel(cfg, g, O, m.i, m.j, C0, C1, C2, D, T, last, nb);
     add_loss(O, lpart);
 }
 
-template <int DT, int KST>
-__global__ void __launch_bounds__(R_THREADS, KST == 1 ? 4 : 2)
-    k_render_fwd(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
-                 const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order, FwdOut O, int B) {
+// The CTA's tiles: 8 / NW consecutive ones of the order.
+template <int NW>
+struct FwdSmem {
+    FwdStage<NW> S[8 / NW];
+    FwdSlots R[8];
+};
+
+template <int DT, int NW>
+__device__ __forceinline__ void fwd_cta(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
+                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
+                                        const uint32_t* __restrict__ order, const FwdOut& O, int blk) {
     extern __shared__ __align__(16) unsigned char r_smem[];
-    const Group G = make_group(g, order, B, blockIdx.x);
-    if (G.tile < 0) return;
-    fwd_pp<DT, KST>(cfg, g, splats, vals, ranges, O, G, reinterpret_cast<StagedSplat*>(r_smem));
+    FwdSmem<NW>& M = *reinterpret_cast<FwdSmem<NW>*>(r_smem);
+    const int gi = (int)threadIdx.x / (32 * NW), t = blk * (8 / NW) + gi;
+    if (t >= g.TX * g.TY) return;
+    const int tile = order ? (int)__ldg(order + t) : t;
+    fwd_pp<DT, NW>(cfg, g, splats, vals, ranges, O, tile, M.S[gi], M.R[threadIdx.x >> 5]);
+}
+
+// CT: CTAs per SM.  Three (80 registers) finish a tile sooner, four (64) keep
+// more warps in flight: 1200 tiles 61.4 against 64.7 us (640x480 / 200k), but
+// 3225 tiles 105.6 against 100.2 (1200x680 / 1M) and 4941 tiles 154 against 144
+// (1296x968 / 750k): three up to 8 CTAs per SM.
+static bool fwd_three(int64_t ctas) { return ctas <= 8 * (int64_t)num_sms(); }
+
+template <int DT, int NW, int CT>
+__global__ void __launch_bounds__(R_THREADS, CT)
+    k_render_fwd(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
+                 const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order, FwdOut O) {
+    fwd_cta<DT, NW>(cfg, g, splats, vals, ranges, order, O, (int)blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -884,37 +991,6 @@ __global__ void __launch_bounds__(R_THREADS, KST == 1 ? (MODE == GS_TRACK ? 4 : 
                           s_max_all);
 }
 
-// Two float32 values in one 64-bit register for the packed f32x2
-// instructions (add, sub, mul, fma with round-to-nearest: one instruction for
-// both halves, each half rounded exactly as the scalar operation).
-typedef unsigned long long x2f;
-
-__device__ __forceinline__ x2f x2_pack(float lo, float hi) {
-    x2f r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void x2_unpack(x2f v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ x2f x2_sub(x2f a, x2f b) {
-    x2f r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ x2f x2_mul(x2f a, x2f b) {
-    x2f r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ x2f x2_fma(x2f a, x2f b, x2f c) {  // a b + c
-    x2f r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
-__device__ __forceinline__ x2f x2_dup(float v) { return x2_pack(v, v); }
-
 // The masked backward's working set of one warp: a ring of 64 staged entries
 // (slot s: pair s / 2, half s & 1, so that two consecutive slots load as
 // packed pairs, two fields per 16-byte load) and the (h, w) columns of the
@@ -930,12 +1006,6 @@ struct __align__(16) PwRing {
     float op[64];      // opacity (mapping)
     float col[8][36];  // h0 w0 h1 w1 h2 w2 h3 w3 over the pixels (36: the rows start in different banks)
 };
-
-__device__ __forceinline__ void x2_ld2(const float4* p, x2f& lo, x2f& hi) {  // one 16-byte load: two packed pairs
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
-    lo = v.x;
-    hi = v.y;
-}
 
 // 32 x 32 bit transpose over the warp: bit p of lane e's result is bit e of
 // lane p's word (five butterfly exchanges; at distance s the partners swap
@@ -1024,13 +1094,11 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 }
 
 // Backward compositing of one warp's block of a tile from the forward's
-// per-pixel blend masks (warp w of the tile's).  Pixel-parallel tiles (EP
-// false): the warp's 8x4 (or 4x8) block, the masks in the run-major layout.
-// Entry-parallel tiles of strided frames (EP true): the tile's sampled
-// pixels 32 w .. 32 w + 31 in row-major order, the masks in the
-// entry-parallel forward's pixel-major layout, whose words past a pixel's
-// stopping batch were never written: each lane keeps only the bits before
-// its own last blended position.
+// per-pixel blend masks (warp w of the tile's): its 8x4 (or 4x8) block, or in
+// tiles of at most 64 sampled pixels pixels 32 w .. 32 w + 31 in row order.
+// Mask words past the run where a pixel's warp (or batch) stopped were never
+// written: each lane keeps only the bits before its own last blended
+// position.
 //
 // The warp walks its runs of 32 list entries from the last one holding an
 // entry one of its pixels blended back to the first.  Per run it stages only
@@ -1061,7 +1129,7 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 // The recombined gradients go straight to grad2d, one atomic per (entry,
 // field, warp): the warps of a tile share nothing and run as one-warp CTAs
 // that the hardware schedules as they free up, heavy tiles first.
-template <int DT, int MODE, bool EP>
+template <int DT, int MODE>
 __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
                                        const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
@@ -1070,8 +1138,9 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
                                        int w, PwRing& R) {
     const int lane = threadIdx.x & 31;
     const int lt = w * 32 + lane;
+    const bool small = g.tw * g.th <= 64;
     PixelMap m;
-    if (EP) {
+    if (small) {
         int i, j;
         m.inside = ep_pixel(g, tile, lt, i, j);
         m.i = i;
@@ -1087,9 +1156,8 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     const uint32_t last = __reduce_max_sync(0xffffffffu, own);
     if (last == 0u) return;  // (warp-uniform) no pixel of the block blended anything
     // this pixel's word of run r at bm[r rs]
-    const uint32_t* bm = EP ? bmask + blend_mask_base_ep(tile, start) + (size_t)lt * ((end - start + 31) >> 5)
-                            : bmask + blend_mask_base(tile, start) + lt;
-    const size_t rs = EP ? 1 : (size_t)tile_threads(g);
+    const uint32_t* bm = bmask + (small ? blend_mask_base_ep(tile, start) : blend_mask_base(tile, start)) + lt;
+    const size_t rs = small ? 64 : (size_t)tile_threads(g);
     const int r_top = (int)((last + 31u) >> 5) - 1;
     // a run's list ids and mask word are loaded one run ahead (runs below
     // the top one are full: their 32 positions lie inside the list)
@@ -1104,7 +1172,7 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     // pixels 8 c + s and 8 c + 4 + s of step s
     const int c = lane & 3, j = lane >> 2;
     // the block's width in pixels: the lanes run row by row through it
-    const int bw = EP ? g.tw : (g.tw < 8 ? 4 : 8), lbw = bw == 16 ? 4 : bw == 8 ? 3 : 2;
+    const int bw = small ? g.tw : (g.tw < 8 ? 4 : 8), lbw = bw == 16 ? 4 : bw == 8 ? 3 : 2;
     const float sx = (float)g.sx, sy = (float)g.sy;
     const float X0 = __shfl_sync(0xffffffffu, pxc, 0) + 0.5f * (float)(bw - 1) * sx;  // the block's centre
     const float Y0 = __shfl_sync(0xffffffffu, pyc, 0) + 0.5f * (float)(32 / bw - 1) * sy;
@@ -1268,11 +1336,9 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
 #define PW_CTAS 24
 
 // Warps per tile of the masked backward.
-__host__ __device__ inline int pw_warps(const Grid& g, bool ep) {
-    return ep ? (g.tw * g.th + 31) >> 5 : tile_threads(g) >> 5;
-}
+__host__ __device__ inline int pw_warps(const Grid& g) { return tile_threads(g) >> 5; }
 
-template <int DT, int MODE, bool EP>
+template <int DT, int MODE>
 __global__ void __launch_bounds__(32, PW_CTAS)
     k_render_bwd_pw(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
                     const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order,
@@ -1280,10 +1346,10 @@ __global__ void __launch_bounds__(32, PW_CTAS)
                     const float* __restrict__ d_rgb, const float* __restrict__ d_depth, float* __restrict__ grad2d,
                     const uint32_t* __restrict__ bmask) {
     __shared__ PwRing R;
-    const int wpt = pw_warps(g, EP);
+    const int wpt = pw_warps(g);
     const int t = (int)blockIdx.x / wpt, w = (int)blockIdx.x % wpt;
     const int tile = order ? (int)__ldg(order + t) : t;
-    bwd_pw<DT, MODE, EP>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, w, R);
+    bwd_pw<DT, MODE>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, w, R);
 }
 
 // ---------------------------------------------------------------------------
@@ -1308,8 +1374,6 @@ __global__ void __launch_bounds__(32, PW_CTAS)
 // with g the pixel's image gradient; each lane adds its entry's gradient to
 // the tile's shared accumulators.  Entries are staged as four 16-byte arrays
 // (lane l reading element l is conflict-free).
-#define EP_B 256     // entries staged per batch (the forward of 64-pixel
-                     // tiles stages 512: fewer CTA barriers per list)
 
 template <int NB>
 struct EpStageN {
@@ -1388,12 +1452,12 @@ __device__ __forceinline__ void ep_pair(const Grid& g, int tile, int q0, int npi
 
 // Forward compositing of pixels q0 .. q0 + npix - 1 of `tile` by the CTA's W
 // warps, entry-parallel (S: staging; cbuf_all: W compaction buffers).
-template <int DT, int W>
+template <int DT, int W, int NB>
 __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
-                                       const FwdOut& O, int tile, int q0, int npix, EpStageN<EpFwdBatch<W>::N>& S,
+                                       const FwdOut& O, int tile, int q0, int npix, EpStageN<NB>& S,
                                        int (*cbuf_all)[64], uint32_t* s_h, uint8_t* perm,
-                                       uint32_t (*bm_all)[EpFwdBatch<W>::N / 32]) {
+                                       uint32_t (*bm_all)[NB / 32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     int* cbuf = cbuf_all[warp];
@@ -1407,9 +1471,7 @@ __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, cons
     float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, D = 0.f;
     uint32_t last = 0, nb = 0;
     bool done = !mine;
-    constexpr int NB = EpFwdBatch<W>::N;
     uint32_t* bmw = bm_all[warp];  // the pixel's blend mask over the batch
-    const uint32_t nw = (end - start + 31) >> 5;
     const size_t bm_tile = blend_mask_base_ep(tile, start);
     for (uint32_t b = start; b < end; b += NB) {
         if (__syncthreads_count(!done) == 0) break;
@@ -1497,7 +1559,7 @@ __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, cons
             if (!stopped && cnt > 0) composite(cnt);
             __syncwarp();
             if (O.bmask && lane < ((n_in + 31) >> 5))
-                O.bmask[bm_tile + (size_t)(q0 + perm[warp * ppw + j]) * nw + ((b - start) >> 5) + lane] = bmw[lane];
+                O.bmask[bm_tile + 64 * (size_t)(((b - start) >> 5) + lane) + (q0 + perm[warp * ppw + j])] = bmw[lane];
             p0 = warp_sum(p0);
             p1 = warp_sum(p1);
             p2 = warp_sum(p2);
@@ -1520,17 +1582,31 @@ __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, cons
     add_loss(O, lpart);
 }
 
+// (the batch length decides the summation order, the number of warps does not)
+template <int W, int NB = EpFwdBatch<W>::N>
+struct EpFwdSmem {
+    EpStageN<NB> S;
+    int cbuf[W][64];
+    uint32_t s_h[64];
+    uint8_t perm[64];
+    uint32_t bm[W][NB / 32];
+};
+
+template <int DT, int W, int NB = EpFwdBatch<W>::N>
+__device__ __forceinline__ void fwd_ep_cta(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
+                                           const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
+                                           const uint32_t* __restrict__ order, const FwdOut& O, int blk) {
+    extern __shared__ __align__(16) unsigned char r_smem[];
+    EpFwdSmem<W, NB>& M = *reinterpret_cast<EpFwdSmem<W, NB>*>(r_smem);
+    const int tile = order ? (int)__ldg(order + blk) : blk;
+    fwd_ep<DT, W, NB>(cfg, g, splats, vals, ranges, O, tile, 0, g.tw * g.th, M.S, M.cbuf, M.s_h, M.perm, M.bm);
+}
+
 template <int DT, int W>
 __global__ void __launch_bounds__(W * 32, W == 8 ? 4 : 2)
     k_render_fwd_ep(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
                     const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order, FwdOut O) {
-    __shared__ EpStageN<EpFwdBatch<W>::N> S;
-    __shared__ int cbuf_all[W][64];
-    __shared__ uint32_t s_h[64];
-    __shared__ uint8_t perm[64];
-    __shared__ uint32_t bm_all[W][EpFwdBatch<W>::N / 32];
-    const int tile = order ? (int)__ldg(order + blockIdx.x) : (int)blockIdx.x;
-    fwd_ep<DT, W>(cfg, g, splats, vals, ranges, O, tile, 0, g.tw * g.th, S, cbuf_all, s_h, perm, bm_all);
+    fwd_ep_cta<DT, W>(cfg, g, splats, vals, ranges, order, O, (int)blockIdx.x);
 }
 
 // Fields merged per entry: GS_TRACK du dv dA dB dC dd, GS_MAP du dv dA dB dC
@@ -1605,7 +1681,6 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
     if (lane == 0) atomicMax(&s_max, wl);
     __syncthreads();
     const uint32_t tile_last = s_max;
-    const uint32_t nw = (end - start + 31) >> 5;
     const uint32_t* bm_tile = bmask ? bmask + blend_mask_base_ep(tile, start) : nullptr;
     // batches [start + k NB, start + (k + 1) NB) from the last one holding a
     // blended entry back to the first
@@ -1627,7 +1702,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
             const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
             // the pixel's blend mask from the forward (entries it blended),
             // else its pixel box, selects the entries to compact
-            const uint32_t* bmj = bm_tile ? bm_tile + (size_t)qj * nw + (base_pos >> 5) : nullptr;
+            const uint32_t* bmj = bm_tile ? bm_tile + 64 * (size_t)(base_pos >> 5) + qj : nullptr;
             float Tj = __shfl_sync(0xffffffffu, T, j);
             float sj = __shfl_sync(0xffffffffu, sdot, j);
             // the pixel's image gradient
@@ -1704,7 +1779,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
             int cnt = 0;
             for (int c = (nj - 1) & ~31; c >= 0; c -= 32) {
                 const int e = c + lane;
-                const bool in = e < nj && (bmj ? ((__ldg(bmj + (c >> 5)) >> lane) & 1u) != 0u : ep_may_blend(S, e, px, py));
+                const bool in = e < nj && (bmj ? ((__ldg(bmj + 64 * (c >> 5)) >> lane) & 1u) != 0u : ep_may_blend(S, e, px, py));
                 const unsigned m = __ballot_sync(0xffffffffu, in);
                 if (in) cbuf[cnt + __popc(m & gt_mask)] = e;
                 cnt += __popc(m);
@@ -1764,34 +1839,38 @@ struct WaveFwdJob {
     const uint32_t* ranges;
     const uint32_t* order;
     FwdOut O;
-    int B;
+    int kind;  // wave_render's fwd_kind
 };
 
-template <int KST>
-__global__ void __launch_bounds__(R_THREADS, KST == 1 ? 4 : 2)
+template <int NW, int CT>
+__global__ void __launch_bounds__(R_THREADS, CT)
     k_wave_render_fwd(const gs_config cfg, const __grid_constant__ Wave<WaveFwdJob> W) {
-    extern __shared__ __align__(16) unsigned char r_smem[];
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveFwdJob& J = W.job[j];
-    const Group G = make_group(J.g, J.order, J.B, (int)blockIdx.x - W.start[j]);
-    if (G.tile < 0) return;
-    fwd_pp<GS_F32, KST>(cfg, J.g, J.splats, J.vals, J.ranges, J.O, G, reinterpret_cast<StagedSplat*>(r_smem));
+    fwd_cta<GS_F32, NW>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, (int)blockIdx.x - W.start[j]);
 }
 
 template <int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 2)
     k_wave_render_fwd_ep(const gs_config cfg, const __grid_constant__ Wave<WaveFwdJob> W) {
-    __shared__ EpStageN<EpFwdBatch<NW>::N> S;
-    __shared__ int cbuf_all[NW][64];
-    __shared__ uint32_t s_h[64];
-    __shared__ uint8_t perm[64];
-    __shared__ uint32_t bm_all[NW][EpFwdBatch<NW>::N / 32];
+    const int j = wave_find(W.start, W.n, (int)blockIdx.x);
+    const WaveFwdJob& J = W.job[j];
+    fwd_ep_cta<GS_F32, NW>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, (int)blockIdx.x - W.start[j]);
+}
+
+// Jobs of several forms in one launch, so that they fill each other's tails
+// (a wave of six sessions of five forms: 187 us, 246 in five launches).
+__global__ void __launch_bounds__(R_THREADS, 4)
+    k_wave_render_fwd_mix(const gs_config cfg, const __grid_constant__ Wave<WaveFwdJob> W) {
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveFwdJob& J = W.job[j];
     const int blk = (int)blockIdx.x - W.start[j];
-    const int tile = J.order ? (int)__ldg(J.order + blk) : blk;
-    fwd_ep<GS_F32, NW>(cfg, J.g, J.splats, J.vals, J.ranges, J.O, tile, 0, J.g.tw * J.g.th, S, cbuf_all, s_h, perm,
-                       bm_all);
+    switch (J.kind) {
+        case 0: fwd_cta<GS_F32, 8>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, blk); break;
+        case 1: fwd_cta<GS_F32, 4>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, blk); break;
+        case 2: fwd_ep_cta<GS_F32, 8>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, blk); break;
+        default: fwd_ep_cta<GS_F32, 8, EpFwdBatch<16>::N>(cfg, J.g, J.splats, J.vals, J.ranges, J.order, J.O, blk); break;
+    }
 }
 
 struct WaveBwdJob {
@@ -1823,17 +1902,16 @@ __global__ void __launch_bounds__(R_THREADS, KST == 1 ? 4 : 2)
 }
 
 // Jobs with blend masks: one-warp CTAs over (job, tile, warp).
-template <bool EP>
 __global__ void __launch_bounds__(32, PW_CTAS) k_wave_render_bwd_pw(const gs_config cfg,
                                                                 const __grid_constant__ Wave<WaveBwdJob> W) {
     __shared__ PwRing R;
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveBwdJob& J = W.job[j];
     const int blk = (int)blockIdx.x - W.start[j];
-    const int wpt = pw_warps(J.g, EP);
+    const int wpt = pw_warps(J.g);
     const int t = blk / wpt, w = blk % wpt;
     const int tile = J.order ? (int)__ldg(J.order + t) : t;
-    bwd_pw<GS_F32, GS_TRACK, EP>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb, J.d_depth,
+    bwd_pw<GS_F32, GS_TRACK>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb, J.d_depth,
                                  J.grad2d, J.bmask, tile, w, R);
 }
 
@@ -1862,17 +1940,10 @@ static int group_batch(int gpc, int bytes_per_entry, int budget) {
     return B;
 }
 
-// The forward's batch: the most entries (a multiple of 32, at most R_BATCH)
-// whose records fit the forward budget for the CTA's gpc tiles.
-static int fwd_batch(int gpc) {
-    const int B = R_FWD_SMEM / (gpc * (int)sizeof(StagedSplat)) / 32 * 32;
-    return B < 32 ? 32 : (B > R_BATCH ? R_BATCH : B);
-}
-
 // Raises a kernel's dynamic shared-memory limit once per device and
 // instantiation (not repeated while a graph is being captured).
 static gs_status smem_once(const void* fn, int id, int bytes) {
-    static bool done[64][48] = {};  // ids: fwd 0-5, bwd 6-17, entry-parallel bwd 18-33, waves 40-45
+    static bool done[64][48] = {};  // ids: bwd 6-17, entry-parallel bwd 18-33, waves 42-45
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && done[dev][id]) return GS_OK;
@@ -1882,32 +1953,43 @@ static gs_status smem_once(const void* fn, int id, int bytes) {
     return GS_OK;
 }
 
-// Kernel choice per frame (the results agree to float32 summation order):
-// both strides >= 2 (tiles of at most 64 sampled pixels): entry-parallel,
-// one CTA of 8 or 16 warps per tile; otherwise pixel-parallel groups.
+// Kernel choice per frame.  Forward: tiles of at most 64 pixels (downsampled
+// frames) entry-parallel, larger ones pixel-parallel.  (The pixel-parallel
+// kernel does less work on large grids of small tiles too -- stride 2x2,
+// 100k Gaussians, 300 tiles 117 against 38 us, 1200 62 / 62, 3225 44 / 146 --
+// but its products and sums round differently, which moves stops and the
+// signs of L1 residuals.)
+// Backward with masks, for which both kernels give the same sums to float32
+// rounding: the one-warp CTAs do less work, the entry-parallel kernel's 8 or
+// 16 warps a tile finish it sooner, which counts while the tiles do not fill
+// the chip.  One-warp against entry-parallel, us (100k Gaussians):
+//   stride 2x2  300 tiles 67 / 55, 1200 41 / 67, 3225 40 / 162
+//   stride 4x2  300 tiles 77 / 57, 1200 44 / 35, 3225 38 / 70
+//   stride 4x4  300 tiles 64 / 36, 1200 39 / 24, 3225 36 / 46
+static bool fwd_entry_parallel(const Grid& g) { return g.tw * g.th <= 64; }
+static bool bwd_entry_parallel(const Grid& g, bool masks, int tiles) {  // tiles: of the launch
+    return g.tw * g.th <= 64 && (!masks || tiles < (g.tw * g.th == 64 ? 512 : 2048));
+}
+
 template <int DT>
 static gs_status launch_fwd(const gs_config& cfg, const Grid& g, const void* splats, const uint32_t* vals,
                             const uint32_t* ranges, const uint32_t* order, const FwdOut& O, cudaStream_t st) {
     const int ntiles = g.TX * g.TY;
-    if (g.tw * g.th <= 64) {
+    if (fwd_entry_parallel(g)) {
         if (g.tw * g.th <= 32)
-            k_render_fwd_ep<DT, 8><<<ntiles, 8 * 32, 0, st>>>(cfg, g, splats, vals, ranges, order, O);
+            k_render_fwd_ep<DT, 8><<<ntiles, 8 * 32, sizeof(EpFwdSmem<8>), st>>>(cfg, g, splats, vals, ranges, order, O);
         else
-            k_render_fwd_ep<DT, 16><<<ntiles, 16 * 32, 0, st>>>(cfg, g, splats, vals, ranges, order, O);
+            k_render_fwd_ep<DT, 16><<<ntiles, 16 * 32, sizeof(EpFwdSmem<16>), st>>>(cfg, g, splats, vals, ranges, order, O);
         return check_launch("k_render_fwd_ep");
     }
-    const int gpc = R_THREADS / tile_threads(g);
+    const int nw = tile_threads(g) / 32, gpc = 8 / nw;
     const unsigned nt = (unsigned)((ntiles + gpc - 1) / gpc);
-    const int B = fwd_batch(gpc);
-    const size_t smem = (size_t)gpc * (B / 32 * 33) * sizeof(StagedSplat);  // + a dummy per 32
-    gs_status s;
-    if (gpc == 1) {
-        if ((s = smem_once((const void*)k_render_fwd<DT, 1>, 2 * DT, R_FWD_SMEM / 32 * 33)) != GS_OK) return s;
-        k_render_fwd<DT, 1><<<nt, R_THREADS, smem, st>>>(cfg, g, splats, vals, ranges, order, O, B);
-    } else {
-        if ((s = smem_once((const void*)k_render_fwd<DT, 4>, 2 * DT + 1, R_FWD_SMEM / 32 * 33)) != GS_OK) return s;
-        k_render_fwd<DT, 4><<<nt, R_THREADS, smem, st>>>(cfg, g, splats, vals, ranges, order, O, B);
-    }
+#define GS_FWD(NW, CT) \
+    k_render_fwd<DT, NW, CT><<<nt, R_THREADS, sizeof(FwdSmem<NW>), st>>>(cfg, g, splats, vals, ranges, order, O)
+    if (nw == 8 && fwd_three(nt)) GS_FWD(8, 3);
+    else if (nw == 8) GS_FWD(8, 4);
+    else GS_FWD(4, 3);
+#undef GS_FWD
     return check_launch("k_render_fwd");
 }
 
@@ -1925,22 +2007,12 @@ static gs_status launch_bwd(const gs_config& cfg, const Grid& g, const void* spl
                             const uint32_t* last_idx, const float* d_rgb, const float* d_depth, float* grad2d,
                             const uint32_t* bmask, cudaStream_t st) {
     const int ntiles = g.TX * g.TY;
-    const bool ep = g.tw * g.th <= 64;
-    // with masks: one-warp CTAs for pixel-parallel tiles and for the 64-pixel
-    // tiles of strided frames (stride 2: 64 -> 90 us in the entry-parallel
-    // kernel; the 16- and 32-pixel tiles of larger strides half-fill or
-    // spread a warp and stay entry-parallel: 38 against 60 us at 4x4)
-    if (bmask && (!ep || g.tw * g.th == 64)) {
-        const unsigned nw = (unsigned)ntiles * (unsigned)pw_warps(g, ep);
-        if (ep)
-            k_render_bwd_pw<DT, MD, true><<<nw, 32, 0, st>>>(cfg, g, splats, vals, ranges, order, t_final, last_idx,
-                                                              d_rgb, d_depth, grad2d, bmask);
-        else
-            k_render_bwd_pw<DT, MD, false><<<nw, 32, 0, st>>>(cfg, g, splats, vals, ranges, order, t_final, last_idx,
-                                                               d_rgb, d_depth, grad2d, bmask);
+    if (bmask && !bwd_entry_parallel(g, true, ntiles)) {  // one-warp CTAs
+        k_render_bwd_pw<DT, MD><<<(unsigned)ntiles * (unsigned)pw_warps(g), 32, 0, st>>>(
+            cfg, g, splats, vals, ranges, order, t_final, last_idx, d_rgb, d_depth, grad2d, bmask);
         return check_launch("k_render_bwd_pw");
     }
-    if (ep) {
+    if (bwd_entry_parallel(g, bmask != nullptr, ntiles)) {
         gs_status s;
         const int id = 18 + 4 * (MD == GS_MAP) + DT;  // + 0 or 8 below: W
         if (g.tw * g.th <= 32) {
@@ -2102,67 +2174,70 @@ extern "C" gs_status gs_render_bwd(const gs_config* cfg, const gs_camera* cam, c
 
 // ---------------------------------------------------------------------------
 // Wave launcher (gs_track_wave): the compositing of every job, grouped by
-// kernel form (0: full tiles, one per CTA; 1: smaller pixel-parallel tiles,
-// several per CTA; 2, 3: entry-parallel tiles of up to 32 or 64 pixels)
+// kernel form
 // ---------------------------------------------------------------------------
 namespace gs {
 
-static int render_form(const Grid& g) {
-    if (g.tw * g.th <= 64) return g.tw * g.th <= 32 ? 2 : 3;
-    return R_THREADS / tile_threads(g) == 1 ? 0 : 1;
-}
-
 gs_status wave_render(const gs_config& cfg, const gs_track_job* jobs, int n, cudaStream_t st) {
     gs_status s;
-    // forward compositing with the fused loss
+    // forward compositing with the fused loss: jobs of one kernel form (warps
+    // a tile; or entry-parallel) in its own kernel, of several in the mixed one
+    auto fwd_kind = [](const Grid& g) {
+        if (fwd_entry_parallel(g)) return g.tw * g.th <= 32 ? 2 : 3;
+        return tile_threads(g) == R_THREADS ? 0 : 1;
+    };
     int present = 0;
-    for (int j = 0; j < n; ++j) present |= 1 << render_form(make_grid(jobs[j].cam));
-    for (int form = 0; form < 4; ++form) {
-        if (!(present & (1 << form))) continue;
+    for (int j = 0; j < n; ++j) present |= 1 << fwd_kind(make_grid(jobs[j].cam));
+    const bool mix = (present & (present - 1)) != 0;
+    for (int kind = 0; kind < 4; ++kind) {
+        if (mix ? kind != 0 : !(present & (1 << kind))) continue;
         Wave<WaveFwdJob> W;
         W.n = 0;
         int blocks = 0;
-        size_t smem = 0;
         for (int j = 0; j < n; ++j) {
             const gs_track_job& t = jobs[j];
             const Grid g = make_grid(t.cam);
-            if (render_form(g) != form) continue;
-            const int ntiles = g.TX * g.TY;
-            const int gpc = form < 2 ? R_THREADS / tile_threads(g) : 1;
-            const int B = form < 2 ? fwd_batch(gpc) : 0;
+            const int kd = fwd_kind(g), gpc = kd == 1 ? 2 : 1;  // tiles per CTA
             const FwdOut O = {t.rgb, t.depth, t.t_final, t.last_idx, t.n_blended, t.target_rgb, t.target_depth,
                               t.d_rgb, t.d_depth, t.loss, t.blend_masks};
             W.start[W.n] = blocks;
-            W.job[W.n] = WaveFwdJob{g, t.splats, t.vals, t.tile_ranges, t.tile_order, O, B};
+            W.job[W.n] = WaveFwdJob{g, t.splats, t.vals, t.tile_ranges, t.tile_order, O, kd};
             ++W.n;
-            blocks += (ntiles + gpc - 1) / gpc;
-            if (form < 2) smem = std::max(smem, (size_t)gpc * (B / 32 * 33) * sizeof(StagedSplat));
+            blocks += (g.TX * g.TY + gpc - 1) / gpc;
         }
         W.start[W.n] = blocks;
-        if (form == 0) {
-            if ((s = smem_once((const void*)k_wave_render_fwd<1>, 40, R_FWD_SMEM / 32 * 33)) != GS_OK) return s;
-            k_wave_render_fwd<1><<<(unsigned)blocks, R_THREADS, smem, st>>>(cfg, W);
-        } else if (form == 1) {
-            if ((s = smem_once((const void*)k_wave_render_fwd<4>, 41, R_FWD_SMEM / 32 * 33)) != GS_OK) return s;
-            k_wave_render_fwd<4><<<(unsigned)blocks, R_THREADS, smem, st>>>(cfg, W);
-        } else if (form == 2) {
-            k_wave_render_fwd_ep<8><<<(unsigned)blocks, 8 * 32, 0, st>>>(cfg, W);
-        } else {
-            k_wave_render_fwd_ep<16><<<(unsigned)blocks, 16 * 32, 0, st>>>(cfg, W);
+        if (mix) {
+            const size_t sm = std::max({sizeof(FwdSmem<8>), sizeof(FwdSmem<4>), sizeof(EpFwdSmem<8, EpFwdBatch<16>::N>)});
+            k_wave_render_fwd_mix<<<(unsigned)blocks, R_THREADS, sm, st>>>(cfg, W);
+            if ((s = check_launch("k_wave_render_fwd")) != GS_OK) return s;
+            break;
         }
+#define GS_FWD(NW, CT) k_wave_render_fwd<NW, CT><<<(unsigned)blocks, R_THREADS, sizeof(FwdSmem<NW>), st>>>(cfg, W)
+        if (kind == 0 && fwd_three(blocks)) GS_FWD(8, 3);
+        else if (kind == 0) GS_FWD(8, 4);
+        else if (kind == 1) GS_FWD(4, 3);
+        else if (kind == 2) k_wave_render_fwd_ep<8><<<(unsigned)blocks, 8 * 32, sizeof(EpFwdSmem<8>), st>>>(cfg, W);
+        else k_wave_render_fwd_ep<16><<<(unsigned)blocks, 16 * 32, sizeof(EpFwdSmem<16>), st>>>(cfg, W);
+#undef GS_FWD
         if ((s = check_launch("k_wave_render_fwd")) != GS_OK) return s;
     }
-    // backward compositing, pose-only fields; jobs with blend masks go to the
-    // one-warp kernel as in launch_bwd (kind 4: pixel-parallel tiles, 5:
-    // 64-pixel entry-parallel tiles)
-    auto bwd_kind = [](const gs_track_job& t) {
-        const int form = render_form(make_grid(t.cam));
-        if (!t.blend_masks) return form;
-        return form < 2 ? 4 : (form == 3 ? 5 : form);
+    // backward compositing, pose-only fields: one launch per kernel form
+    // present (0, 1: without masks, one or several tiles a CTA; 2, 3:
+    // entry-parallel tiles of up to 32 or 64 pixels; 4: one-warp CTAs)
+    // (the one-warp CTAs of all jobs with masks share a launch and so its tail)
+    int masked = 0;
+    for (int j = 0; j < n; ++j) {
+        const Grid g = make_grid(jobs[j].cam);
+        if (jobs[j].blend_masks) masked += g.TX * g.TY;
+    }
+    auto bwd_kind = [masked](const gs_track_job& t) {
+        const Grid g = make_grid(t.cam);
+        if (bwd_entry_parallel(g, t.blend_masks != nullptr, masked)) return g.tw * g.th <= 32 ? 2 : 3;
+        return t.blend_masks ? 4 : (R_THREADS / tile_threads(g) == 1 ? 0 : 1);
     };
     int kinds = 0;
     for (int j = 0; j < n; ++j) kinds |= 1 << bwd_kind(jobs[j]);
-    for (int kind = 0; kind < 6; ++kind) {
+    for (int kind = 0; kind < 5; ++kind) {
         if (!(kinds & (1 << kind))) continue;
         Wave<WaveBwdJob> W;
         W.n = 0;
@@ -2180,7 +2255,7 @@ gs_status wave_render(const gs_config& cfg, const gs_track_job* jobs, int n, cud
             W.job[W.n] = WaveBwdJob{g, t.splats, t.vals, t.tile_ranges, t.tile_order, t.t_final, t.last_idx, t.d_rgb,
                                     t.d_depth, t.grad2d, t.blend_masks, B};
             ++W.n;
-            blocks += kind >= 4 ? ntiles * pw_warps(g, kind == 5) : (ntiles + gpc - 1) / gpc;
+            blocks += kind == 4 ? ntiles * pw_warps(g) : (ntiles + gpc - 1) / gpc;
             if (kind < 2) smem = std::max(smem, (size_t)gpc * B * per_entry);
         }
         W.start[W.n] = blocks;
@@ -2199,10 +2274,7 @@ gs_status wave_render(const gs_config& cfg, const gs_track_job* jobs, int n, cud
             if ((s = smem_once((const void*)k_wave_render_bwd_ep<16>, 45, sm)) != GS_OK) return s;
             k_wave_render_bwd_ep<16><<<(unsigned)blocks, 16 * 32, sm, st>>>(cfg, W);
         } else {
-            if (kind == 4)
-                k_wave_render_bwd_pw<false><<<(unsigned)blocks, 32, 0, st>>>(cfg, W);
-            else
-                k_wave_render_bwd_pw<true><<<(unsigned)blocks, 32, 0, st>>>(cfg, W);
+            k_wave_render_bwd_pw<<<(unsigned)blocks, 32, 0, st>>>(cfg, W);
         }
         if ((s = check_launch("k_wave_render_bwd")) != GS_OK) return s;
     }
