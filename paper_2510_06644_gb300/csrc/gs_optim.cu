@@ -20,13 +20,13 @@ struct AdamArgs {
 __global__ void __launch_bounds__(256) k_adam(AdamArgs a, int64_t total, float lr, float b1, float b2, float eps,
                                               float* __restrict__ state) {
     const float step = state[0] + 1.f;
-    const float c1 = 1.f - powf(b1, step), c2 = 1.f - powf(b2, step);
+    const AdamStep as = adam_step(lr, b1, b2, step);
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
         int t = 0;
         while (t < a.nt - 1 && q >= a.end[t]) ++t;
         const int64_t i = q - (t > 0 ? a.end[t - 1] : 0);
         float p = a.p[t][i], m = a.m[t][i], v = a.v[t][i];
-        adam_elem(p, m, v, a.g[t][i], lr, b1, b2, c1, c2, eps);
+        adam_elem(p, m, v, a.g[t][i], b1, b2, as, eps);
         a.p[t][i] = p;
         a.m[t][i] = m;
         a.v[t][i] = v;

@@ -384,7 +384,8 @@ struct AdamMap {
     float* p[5];
     float* m[5];
     float* v[5];
-    float lr, b1, b2, eps, c1, c2;
+    float lr, b1, b2, eps;
+    AdamStep s;  // formed in the kernel
 };
 
 // PER Gaussians per thread: two when the pose is reduced (391 blocks of 256
@@ -547,7 +548,7 @@ __device__ __forceinline__ void project_bwd_body(gs_camera cam, const gs_config&
                     for (int i = 0; i < width[t]; ++i) {
                         const size_t e = (size_t)width[t] * k + i;
                         float pp = A.p[t][e], mm = A.m[t][e], vv = A.v[t][e];
-                        adam_elem(pp, mm, vv, gv[t][i], A.lr, A.b1, A.b2, A.c1, A.c2, A.eps);
+                        adam_elem(pp, mm, vv, gv[t][i], A.b1, A.b2, A.s, A.eps);
                         A.p[t][e] = pp;
                         A.m[t][e] = mm;
                         A.v[t][e] = vv;
@@ -868,8 +869,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_project_bwd_adam(gs_camera cam, 
                                                                  float* __restrict__ state) {
     // the step count: read by every block, advanced by the last (as gs_adam)
     const float step = __ldcg(state) + 1.f;
-    A.c1 = 1.f - powf(A.b1, step);
-    A.c2 = 1.f - powf(A.b2, step);
+    A.s = adam_step(A.lr, A.b1, A.b2, step);
     const gs_pose_step none = {nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 0.f};
     project_bwd_body<true, false, WANT_SCORE, true>(cam, cfg, g, grad2d, grads, score, nullptr, nullptr, nullptr,
                                                     none, (int)blockIdx.x, (int)gridDim.x, &A);
@@ -914,7 +914,7 @@ extern "C" gs_status gs_project_bwd_adam(const gs_config* cfg, const gs_camera* 
     A.b1 = adam->beta1;
     A.b2 = adam->beta2;
     A.eps = adam->eps;
-    A.c1 = A.c2 = 1.f;
+    A.s = AdamStep{0.f, 0.f};
     const gs_grads gg = grads ? *grads : gs_grads{nullptr, nullptr, nullptr, nullptr, nullptr};
     const unsigned nblk = (unsigned)pb_blocks(g->n, 1);
     cudaStream_t st = (cudaStream_t)stream;
