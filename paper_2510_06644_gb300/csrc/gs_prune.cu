@@ -3,10 +3,11 @@
 // downsampling (Sec. 4.2) on sm_103a.
 //
 // Selection is a radix select on the unique 64-bit key (score bits << 32 |
-// id): eight 8-bit digit passes, each CTA re-deriving the prefix chosen so
-// far from the previous passes' histograms (a few hundred integer ops), so
-// no pass needs a separate pick launch or a host round trip.  Scores are
-// non-negative, so their float bits order like their values.
+// id): digits of 11, 11 and 10 bits settle the score, and 11-bit digits of the
+// bits that ids below n have settle ties.  A pass needs only the histogram of
+// the pass before it, which every CTA scans for itself, so no pass needs a
+// pick launch or a host round trip.  Scores are non-negative, so their float
+// bits order like their values.
 #include "gs_internal.cuh"
 
 namespace gs {
@@ -14,190 +15,313 @@ namespace gs {
 typedef unsigned long long u64;
 
 #define PR_THREADS 256
-#define PR_CHUNK 2048
+#define SEL_THREADS 512
+#define SEL_BINS 2048        // 11-bit digits
+#define SEL_MAX_PASSES 6     // 3 of the score, at most 3 of the id
+#define KEEP_PER_THREAD 8
+#define KEEP_STEP (PR_THREADS * KEEP_PER_THREAD)
+#define KEEP_MAX_CHUNKS 2048
 
-struct PruneState {
-    u64 n_active;  // unmasked Gaussians
-};
-
-__device__ __forceinline__ u64 score_key(const float* __restrict__ st, int64_t k, float lam) {
+__device__ __forceinline__ u64 score_key(float mu, float sig, int64_t k, float lam) {
     // Eq. 7 in float32: product rounded, then sum rounded (no fused multiply-add)
-    const float s = __fadd_rn(st[2 * k], __fmul_rn(lam, st[2 * k + 1]));
+    const float s = __fadd_rn(mu, __fmul_rn(lam, sig));
     return ((u64)__float_as_uint(s) << 32) | (u64)(uint32_t)k;
 }
 
-__global__ void __launch_bounds__(PR_THREADS) k_prune_count(const uint8_t* __restrict__ mask, int64_t n,
-                                                            PruneState* __restrict__ state) {
-    __shared__ unsigned int s_cnt;
-    if (threadIdx.x == 0) s_cnt = 0;
-    __syncthreads();
-    unsigned int c = 0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        c += mask[k] == 0 ? 1u : 0u;
-    atomicAdd(&s_cnt, c);
-    __syncthreads();
-    if (threadIdx.x == 0 && s_cnt) atomicAdd(&state->n_active, (u64)s_cnt);
+// ---------------------------------------------------------------------------
+// Selection
+// ---------------------------------------------------------------------------
+// One digit: `bits` wide, its lowest bit at `shift`.
+struct Digit {
+    int shift, bits;
+};
+
+struct SelPasses {
+    Digit d[SEL_MAX_PASSES];
+    int count;
+};
+
+// The digits for ids below n: bits that no id has are not passed over (1M ids:
+// five passes, at most 2048 ids: four).
+static SelPasses sel_passes(int64_t n) {
+    SelPasses P;
+    P.d[0] = {53, 11};
+    P.d[1] = {42, 11};
+    P.d[2] = {32, 10};
+    P.count = 3;
+    int top = 0;
+    while (top < 32 && ((n - 1) >> top) > 0) ++top;
+    while (top > 0) {
+        const int w = top < 11 ? top : 11;
+        top -= w;
+        P.d[P.count++] = {top, w};
+    }
+    return P;
 }
+
+// What the passes so far have fixed: the key prefix, the rank that is left
+// inside it, and whether the threshold is known.
+enum { SEL_OPEN = 0, SEL_DONE = 1, SEL_NONE = 2 };
+struct SelState {
+    u64 prefix, remaining, status;
+};
+
+struct SelArgs {
+    const float* terms;
+    uint8_t* mask;
+    int64_t n;
+    float lam, frac;
+    int64_t max_select;
+    SelState* state;     // [pass]: before that pass
+    unsigned int* hist;  // [pass][SEL_BINS]
+    int pass;            // digits of this pass and of the one before it
+    Digit d, prev;
+    int vec;             // terms 16-byte and mask 4-byte aligned
+};
 
 // m = min(floor(frac * n_active), max_select): rank (1-based) of the largest
 // selected key.
-__device__ __forceinline__ u64 select_count(const PruneState* st, float frac, int64_t max_select) {
-    const double m = floor((double)frac * (double)st->n_active);
+__device__ __forceinline__ u64 select_count(u64 n_active, float frac, int64_t max_select) {
+    const double m = floor((double)frac * (double)n_active);
     u64 mm = (u64)m;
     if ((int64_t)mm > max_select) mm = (u64)(max_select < 0 ? 0 : max_select);
     return mm;
 }
 
-// Re-derives the key prefix fixed by passes [0, p) from their histograms.
-__device__ __forceinline__ void derive_prefix(const unsigned int* __restrict__ hist, int p, u64 m, u64& prefix,
-                                              u64& remaining) {
-    prefix = 0;
-    remaining = m;
-    for (int q = 0; q < p; ++q) {
-        const unsigned int* h = hist + q * 256;
-        u64 cum = 0;
-        int b = 0;
-        for (; b < 256; ++b) {
-            const u64 c = h[b];
-            if (cum + c >= remaining) break;
-            cum += c;
-        }
-        if (b == 256) b = 255;  // only reachable if m exceeds the candidates
-        remaining -= cum;
-        prefix |= (u64)b << (56 - 8 * q);
-    }
-}
-
-__global__ void __launch_bounds__(PR_THREADS) k_select_pass(const float* __restrict__ st, const uint8_t* __restrict__ mask,
-                                                            int64_t n, float lam, float frac, int64_t max_select,
-                                                            const PruneState* __restrict__ state,
-                                                            unsigned int* __restrict__ hist, int p) {
-    __shared__ unsigned int sh[256];
-    __shared__ u64 s_prefix;
-    __shared__ int s_skip;
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) sh[i] = 0;
-    if (threadIdx.x == 0) {
-        const u64 m = select_count(state, frac, max_select);
-        u64 prefix, rem;
-        derive_prefix(hist, p, m, prefix, rem);
-        s_prefix = prefix;
-        s_skip = (m == 0);
-    }
-    __syncthreads();
-    if (s_skip) return;
-    const u64 prefix = s_prefix;
-    const int shift = 56 - 8 * p;
-    const u64 hi_mask = p == 0 ? 0ull : (~0ull << (64 - 8 * p));
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        if (mask[k]) continue;
-        const u64 key = score_key(st, k, lam);
-        if ((key & hi_mask) != prefix) continue;
-        atomicAdd(&sh[(key >> shift) & 0xff], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (sh[i]) atomicAdd(hist + p * 256 + i, sh[i]);
-}
-
-__global__ void __launch_bounds__(PR_THREADS) k_select_mask(const float* __restrict__ st, uint8_t* __restrict__ mask,
-                                                            int64_t n, float lam, float frac, int64_t max_select,
-                                                            const PruneState* __restrict__ state,
-                                                            const unsigned int* __restrict__ hist) {
-    __shared__ u64 s_kth;
-    __shared__ int s_skip;
-    if (threadIdx.x == 0) {
-        const u64 m = select_count(state, frac, max_select);
-        u64 prefix, rem;
-        derive_prefix(hist, 8, m, prefix, rem);
-        s_kth = prefix;
-        s_skip = (m == 0);
-    }
-    __syncthreads();
-    if (s_skip) return;
-    const u64 kth = s_kth;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        if (mask[k]) continue;
-        if (score_key(st, k, lam) <= kth) mask[k] = 1;
-    }
-}
-
-// Compaction map: exclusive scan of (mask == 0) in id order.
-__global__ void __launch_bounds__(PR_THREADS) k_keep_count(const uint8_t* __restrict__ mask, int64_t n,
-                                                           u64* __restrict__ partial) {
-    __shared__ unsigned int s;
-    if (threadIdx.x == 0) s = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * PR_CHUNK;
-    unsigned int c = 0;
-    for (int j = threadIdx.x; j < PR_CHUNK; j += PR_THREADS) {
-        const int64_t k = base + j;
-        if (k < n && mask[k] == 0) ++c;
-    }
-    atomicAdd(&s, c);
-    __syncthreads();
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(1024) k_keep_scan(u64* __restrict__ partial, int nchunk, int64_t* __restrict__ n_kept) {
-    __shared__ u64 s_warp[32];
+// The state before pass p, from the state before pass p - 1 and that pass's
+// histogram: every CTA scans the 2048 counts (four a thread) and block 0 stores
+// the result for the next launch.  The first histogram also counts the active
+// Gaussians.  If all keys of the chosen bin are selected, the digits below
+// cannot matter and the threshold is the bin's last key.
+__device__ __forceinline__ SelState sel_advance(const SelArgs& A) {
+    const int p = A.pass;
+    __shared__ SelState s_new;
+    __shared__ u64 s_warp[SEL_THREADS / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    u64 carry = 0;
-    for (int base = 0; base < nchunk; base += 1024) {
-        const int i = base + threadIdx.x;
-        const u64 v = i < nchunk ? partial[i] : 0ull;
-        u64 x = v;
+    SelState S = {0, 0, SEL_OPEN};
+    if (p == 0) return S;
+    if (p > 1) S = A.state[p - 1];
+    if (S.status == SEL_OPEN) {
+        const uint4 h = reinterpret_cast<const uint4*>(A.hist + (size_t)(p - 1) * SEL_BINS)[threadIdx.x];
+        const u64 mine = (u64)h.x + h.y + h.z + h.w;
+        u64 x = mine;
         for (int o = 1; o < 32; o <<= 1) {
             const u64 y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) s_warp[wid] = x;
         __syncthreads();
-        if (wid == 0) {
-            u64 w = s_warp[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const u64 y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            s_warp[lane] = w;
-        }
-        __syncthreads();
-        const u64 before = wid > 0 ? s_warp[wid - 1] : 0ull;
-        const u64 total = s_warp[31];
-        if (i < nchunk) partial[i] = carry + before + x - v;
-        carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *n_kept = (int64_t)carry;
-}
-
-__global__ void __launch_bounds__(PR_THREADS) k_keep_write(const uint8_t* __restrict__ mask, int64_t n,
-                                                           const u64* __restrict__ partial, uint32_t* __restrict__ map) {
-    // each warp takes 64 consecutive ids (2 per lane) of the chunk, in order
-    __shared__ unsigned int s_warp[PR_THREADS / 32];
-    const int64_t base = (int64_t)blockIdx.x * PR_CHUNK;
-    u64 off = partial[blockIdx.x];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int seg = 0; seg < PR_CHUNK; seg += PR_THREADS) {
-        const int64_t k = base + seg + threadIdx.x;
-        const bool keep = k < n && mask[k] == 0;
-        const unsigned int bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_warp[wid] = __popc(bal);
-        __syncthreads();
-        unsigned int before = 0, total = 0;
-        for (int w = 0; w < PR_THREADS / 32; ++w) {
+        u64 before = 0, total = 0;
+        for (int w = 0; w < SEL_THREADS / 32; ++w) {
             if (w < wid) before += s_warp[w];
             total += s_warp[w];
         }
-        if (k < n) map[k] = keep ? (uint32_t)(off + before + __popc(bal & ((1u << lane) - 1u))) : 0xFFFFFFFFu;
-        off += total;
-        __syncthreads();
+        if (p == 1) {
+            S.remaining = select_count(total, A.frac, A.max_select);
+            if (S.remaining == 0) S.status = SEL_NONE;
+            else if (S.remaining >= total) S = {~0ull, S.remaining, SEL_DONE};
+        }
+        if (S.status == SEL_OPEN) {
+            u64 cum = before + x - mine;  // counts below this thread's bins
+            if (cum < S.remaining && S.remaining <= cum + mine) {
+                unsigned int c = h.x, j = 0;
+                if (cum + c < S.remaining) { cum += c; c = h.y; j = 1; }
+                if (j == 1 && cum + c < S.remaining) { cum += c; c = h.z; j = 2; }
+                if (j == 2 && cum + c < S.remaining) { cum += c; c = h.w; j = 3; }
+                SelState N = {S.prefix | ((u64)(threadIdx.x * 4 + j) << A.prev.shift), S.remaining - cum, SEL_OPEN};
+                if (N.remaining == c) {
+                    N.prefix |= (1ull << A.prev.shift) - 1ull;
+                    N.status = SEL_DONE;
+                }
+                s_new = N;
+            }
+            __syncthreads();
+            S = s_new;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.state[p] = S;
+    return S;
+}
+
+// The keys of ids [4 q, 4 q + 4) and which of them are unmasked (bit j).
+__device__ __forceinline__ unsigned int load_keys(const SelArgs& A, int64_t q, u64* key) {
+    const int64_t k = 4 * q;
+    unsigned int live = 0;
+    if (A.vec && k + 4 <= A.n) {
+        const uchar4 m = reinterpret_cast<const uchar4*>(A.mask)[q];
+        const float4 a = __ldg(reinterpret_cast<const float4*>(A.terms) + 2 * q);
+        const float4 b = __ldg(reinterpret_cast<const float4*>(A.terms) + 2 * q + 1);
+        key[0] = score_key(a.x, a.y, k, A.lam);
+        key[1] = score_key(a.z, a.w, k + 1, A.lam);
+        key[2] = score_key(b.x, b.y, k + 2, A.lam);
+        key[3] = score_key(b.z, b.w, k + 3, A.lam);
+        live = (m.x ? 0u : 1u) | (m.y ? 0u : 2u) | (m.z ? 0u : 4u) | (m.w ? 0u : 8u);
+    } else {
+        for (int j = 0; j < 4; ++j) {
+            key[j] = 0;
+            if (k + j < A.n && A.mask[k + j] == 0) {
+                key[j] = score_key(A.terms[2 * (k + j)], A.terms[2 * (k + j) + 1], k + j, A.lam);
+                live |= 1u << j;
+            }
+        }
+    }
+    return live;
+}
+
+// Histogram of one digit over the unmasked keys under the prefix.  The scores
+// come from L2 in every pass (8 bytes a Gaussian), so a pass is short and the
+// launches count: eight 8-bit passes, each re-deriving the whole prefix by one
+// thread, took 69 us with their count and mask launches at 1M Gaussians;
+// these take 36.  Many scores are equal (zero where nothing was blended), so a warp
+// adds its first key's bin once for all lanes that share it.
+__global__ void __launch_bounds__(SEL_THREADS) k_select_pass(const __grid_constant__ SelArgs A) {
+    __shared__ unsigned int sh[SEL_BINS];
+    for (int i = threadIdx.x; i < SEL_BINS; i += SEL_THREADS) sh[i] = 0;
+    const int p = A.pass;
+    const SelState S = sel_advance(A);
+    if (S.status != SEL_OPEN) return;  // the same in every thread of the grid
+    __syncthreads();
+    const Digit d = A.d;
+    const unsigned int bin_mask = (1u << d.bits) - 1u;
+    const int top = A.prev.shift;
+    const int lane = threadIdx.x & 31;
+    const int64_t nq = (A.n + 3) >> 2;
+    const int64_t stride = (int64_t)gridDim.x * SEL_THREADS;
+    for (int64_t q0 = (int64_t)blockIdx.x * SEL_THREADS + (threadIdx.x & ~31); q0 < nq; q0 += stride) {
+        u64 key[4] = {0, 0, 0, 0};
+        const unsigned int live = q0 + lane < nq ? load_keys(A, q0 + lane, key) : 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool take = (live >> j & 1u) && (p == 0 || ((key[j] ^ S.prefix) >> top) == 0);
+            const unsigned int any = __ballot_sync(0xffffffffu, take);
+            if (any == 0) continue;
+            const int first = __ffs(any) - 1;
+            const unsigned int bin = (unsigned int)(key[j] >> d.shift) & bin_mask;
+            const unsigned int b0 = __shfl_sync(0xffffffffu, bin, first);
+            const unsigned int same = __ballot_sync(0xffffffffu, take && bin == b0);
+            if (lane == first) atomicAdd(&sh[b0], (unsigned int)__popc(same));
+            else if (take && bin != b0) atomicAdd(&sh[bin], 1u);
+        }
+    }
+    __syncthreads();
+    unsigned int* h = A.hist + (size_t)p * SEL_BINS;
+    for (int i = threadIdx.x; i < SEL_BINS; i += SEL_THREADS)
+        if (sh[i]) atomicAdd(h + i, sh[i]);
+}
+
+__global__ void __launch_bounds__(SEL_THREADS) k_select_mask(const __grid_constant__ SelArgs A) {
+    const SelState S = sel_advance(A);
+    if (S.status == SEL_NONE) return;
+    const int64_t nq = (A.n + 3) >> 2;
+    for (int64_t q = (int64_t)blockIdx.x * SEL_THREADS + threadIdx.x; q < nq; q += (int64_t)gridDim.x * SEL_THREADS) {
+        u64 key[4];
+        const unsigned int live = load_keys(A, q, key);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((live >> j & 1u) && key[j] <= S.prefix) A.mask[4 * q + j] = 1;
     }
 }
 
+// ---------------------------------------------------------------------------
+// Compaction map: exclusive scan of (mask == 0) in id order
+// ---------------------------------------------------------------------------
+// Bit j: id k + j exists and is kept.
+__device__ __forceinline__ unsigned int keep_bits(const uint8_t* __restrict__ mask, int64_t k, int64_t n, bool vec) {
+    unsigned int keep = 0;
+    if (vec && k + KEEP_PER_THREAD <= n) {
+        const uint2 m = __ldg(reinterpret_cast<const uint2*>(mask + k));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            keep |= ((m.x >> (8 * j)) & 0xffu) ? 0u : 1u << j;
+            keep |= ((m.y >> (8 * j)) & 0xffu) ? 0u : 16u << j;
+        }
+    } else {
+        for (int j = 0; j < KEEP_PER_THREAD; ++j)
+            if (k + j < n && mask[k + j] == 0) keep |= 1u << j;
+    }
+    return keep;
+}
+
+// Kept ids of each chunk.  A chunk is a multiple of 2048 ids such that there
+// are at most 2048 chunks: few enough that k_keep_write sums those before its
+// own itself, without a scan launch between the two.
+__global__ void __launch_bounds__(PR_THREADS) k_keep_count(const uint8_t* __restrict__ mask, int64_t n, int64_t chunk,
+                                                           bool vec, u64* __restrict__ partial) {
+    __shared__ unsigned int s;
+    if (threadIdx.x == 0) s = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * chunk;
+    unsigned int c = 0;
+    for (int64_t o = (int64_t)threadIdx.x * KEEP_PER_THREAD; o < chunk; o += KEEP_STEP)
+        c += __popc(keep_bits(mask, base + o, n, vec));
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s, c);
+    __syncthreads();
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+__global__ void __launch_bounds__(PR_THREADS) k_keep_write(const uint8_t* __restrict__ mask, int64_t n, int64_t chunk,
+                                                           bool vec, bool vec_out, const u64* __restrict__ partial,
+                                                           uint32_t* __restrict__ map, int64_t* __restrict__ n_kept) {
+    __shared__ u64 s_before;
+    __shared__ unsigned int s_warp[2][PR_THREADS / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_before = 0;
+    __syncthreads();
+    u64 part = 0;
+    for (unsigned int b = threadIdx.x; b < blockIdx.x; b += PR_THREADS) part += partial[b];
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (lane == 0 && part) atomicAdd(&s_before, part);
+    __syncthreads();
+    u64 off = s_before;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_kept = (int64_t)(off + partial[blockIdx.x]);
+    const int64_t base = (int64_t)blockIdx.x * chunk;
+    int buf = 0;
+    for (int64_t o = 0; o < chunk && base + o < n; o += KEEP_STEP, buf ^= 1) {
+        const int64_t k = base + o + (int64_t)threadIdx.x * KEEP_PER_THREAD;
+        const unsigned int keep = keep_bits(mask, k, n, vec);
+        const unsigned int mine = __popc(keep);
+        unsigned int x = mine;
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned int y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) s_warp[buf][wid] = x;
+        __syncthreads();  // the other buffer is read before the next barrier at the latest
+        unsigned int before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < PR_THREADS / 32; ++w) {
+            const unsigned int t = s_warp[buf][w];
+            before += w < wid ? t : 0u;
+            total += t;
+        }
+        uint32_t to[KEEP_PER_THREAD], at = (uint32_t)off + before + x - mine;
+#pragma unroll
+        for (int j = 0; j < KEEP_PER_THREAD; ++j) to[j] = (keep >> j & 1u) ? at++ : 0xFFFFFFFFu;
+        if (vec_out && k + KEEP_PER_THREAD <= n) {
+            uint4* dst = reinterpret_cast<uint4*>(map + k);
+            dst[0] = make_uint4(to[0], to[1], to[2], to[3]);
+            dst[1] = make_uint4(to[4], to[5], to[6], to[7]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < KEEP_PER_THREAD; ++j)
+                if (k + j < n) map[k + j] = to[j];
+        }
+        off += total;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Change ratio
+// ---------------------------------------------------------------------------
 // |rect_a| + |rect_b| - 2 |rect_a & rect_b| and |rect_a| summed over Gaussians.
 template <int DT>
 __global__ void __launch_bounds__(PR_THREADS) k_change(gs_camera cam, float alpha_min, const void* __restrict__ sa,
-                                                       const void* __restrict__ sb, int64_t n, u64* __restrict__ acc) {
+                                                       const void* __restrict__ sb, int64_t n, u64* __restrict__ acc,
+                                                       float* __restrict__ out) {
+    __shared__ u64 s_acc[2];
+    if (threadIdx.x < 2) s_acc[threadIdx.x] = 0;
+    __syncthreads();
     const Grid grid = make_grid(cam);
     u64 sym = 0, na = 0;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -216,24 +340,56 @@ __global__ void __launch_bounds__(PR_THREADS) k_change(gs_camera cam, float alph
         sym += __shfl_xor_sync(0xffffffffu, sym, o);
         na += __shfl_xor_sync(0xffffffffu, na, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(acc, sym);
-        atomicAdd(acc + 1, na);
+    if ((threadIdx.x & 31) == 0 && (sym | na)) {
+        atomicAdd(&s_acc[0], sym);
+        atomicAdd(&s_acc[1], na);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_acc[0]) atomicAdd(acc, s_acc[0]);
+        if (s_acc[1]) atomicAdd(acc + 1, s_acc[1]);
+        __threadfence();
+        if (atomicAdd(acc + 2, 1ull) == gridDim.x - 1) {  // every block has added its share
+            const u64 tot = atomicAdd(acc, 0ull);
+            const double in_a = (double)atomicAdd(acc + 1, 0ull);
+            *out = (float)((double)tot / (in_a > 1.0 ? in_a : 1.0));
+        }
     }
 }
 
-__global__ void k_change_final(const u64* __restrict__ acc, float* __restrict__ out) {
-    const double na = (double)acc[1];
-    *out = (float)((double)acc[0] / (na > 1.0 ? na : 1.0));
-}
-
+// Rows of a parameter array to their places in the compacted one; W floats a
+// row (1 to 4 as constants: 0 takes any width).  A block moves 256 rows, so the
+// row of an element is a 32-bit division by a constant and every load of the
+// block is in flight at once.  One 64-bit division an element made it
+// instruction-bound: 1M rows of 3 floats 11.3 us, now 6.3 (29 MB moved).
+template <int W>
 __global__ void __launch_bounds__(256) k_compact(const float* __restrict__ src, int64_t n, int width,
                                                  const uint32_t* __restrict__ map, float* __restrict__ dst) {
-    const int64_t total = n * (int64_t)width;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = q / width;
-        const uint32_t to = map[k];
-        if (to != 0xFFFFFFFFu) dst[(int64_t)to * width + (q - k * width)] = src[q];
+    if (W == 0) {
+        const int64_t total = n * (int64_t)width;
+        for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
+             q += (int64_t)gridDim.x * blockDim.x) {
+            const int64_t k = q / width;
+            const uint32_t to = map[k];
+            if (to != 0xFFFFFFFFu) dst[(int64_t)to * width + (q - k * width)] = src[q];
+        }
+        return;
+    }
+    constexpr int WC = W > 0 ? W : 1;
+    for (int64_t r0 = (int64_t)blockIdx.x * 256; r0 < n; r0 += (int64_t)gridDim.x * 256) {
+        const unsigned int rows = (unsigned int)(n - r0 < 256 ? n - r0 : 256);
+        uint32_t to[WC];
+        float v[WC];
+#pragma unroll
+        for (int j = 0; j < WC; ++j) {
+            const unsigned int e = threadIdx.x + 256u * j;
+            const bool in = e < rows * WC;
+            to[j] = in ? __ldg(map + r0 + e / WC) : 0xFFFFFFFFu;
+            v[j] = in ? __ldg(src + r0 * WC + e) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < WC; ++j)
+            if (to[j] != 0xFFFFFFFFu) dst[(int64_t)to[j] * WC + (threadIdx.x + 256u * j) % WC] = v[j];
     }
 }
 
@@ -271,33 +427,45 @@ extern "C" gs_status gs_prune(const gs_config* cfg, const float* score_terms, in
     if (!cfg || !workspace_bytes || !k_inout) return set_error(GS_ERR_INVALID_ARG, "config, k_inout or workspace_bytes NULL");
     if (n < 0 || n > (int64_t)0xFFFFFFF0LL) return set_error(GS_ERR_INVALID_ARG, "bad Gaussian count");
     if (*k_inout < 1) return set_error(GS_ERR_INVALID_ARG, "interval K must be >= 1");
-    const int64_t nchunk = (n + PR_CHUNK - 1) / PR_CHUNK;
-    const size_t off_hist = 0, off_state = a256(8 * 256 * sizeof(unsigned int));
-    const size_t off_part = a256(off_state + sizeof(PruneState));
-    const size_t need = a256(off_part + sizeof(u64) * (size_t)(nchunk > 0 ? nchunk : 1));
+    const int64_t steps = (n + KEEP_STEP - 1) / KEEP_STEP;
+    const int64_t chunk = KEEP_STEP * ((steps + KEEP_MAX_CHUNKS - 1) / KEEP_MAX_CHUNKS);
+    const size_t hist_bytes = SEL_MAX_PASSES * SEL_BINS * sizeof(unsigned int);
+    const size_t off_state = a256(hist_bytes);
+    const size_t off_part = a256(off_state + (SEL_MAX_PASSES + 1) * sizeof(SelState));
+    const size_t need = a256(off_part + sizeof(u64) * KEEP_MAX_CHUNKS);
     if (!workspace) { *workspace_bytes = need; return GS_OK; }
     if (*workspace_bytes < need) return set_error(GS_ERR_WORKSPACE, "workspace %zu < %zu", *workspace_bytes, need);
     cudaStream_t st = (cudaStream_t)stream;
     char* ws = (char*)workspace;
-    const int sms = num_sms();
-    const int64_t want = (n + PR_THREADS - 1) / PR_THREADS;
-    const unsigned nb = (unsigned)(want < 4 * sms ? (want > 0 ? want : 1) : 4 * sms);
     gs_status s;
     if (iter_in_interval == 0) {
         if (n == 0) return GS_OK;
         if (!score_terms || !mask_inout) return set_error(GS_ERR_INVALID_ARG, "score_terms or mask NULL");
-        if (cudaMemsetAsync(ws, 0, off_part, st) != cudaSuccess) return set_error(GS_ERR_CUDA, "memset prune state");
-        unsigned int* hist = (unsigned int*)(ws + off_hist);
-        PruneState* state = (PruneState*)(ws + off_state);
-        k_prune_count<<<nb, PR_THREADS, 0, st>>>(mask_inout, n, state);
-        if ((s = check_launch("k_prune_count")) != GS_OK) return s;
-        for (int p = 0; p < 8; ++p) {
-            k_select_pass<<<nb, PR_THREADS, 0, st>>>(score_terms, mask_inout, n, cfg->lambda_score, cfg->prune_frac,
-                                                     max_select, state, hist, p);
+        SelArgs A;
+        A.terms = score_terms;
+        A.mask = mask_inout;
+        A.n = n;
+        A.lam = cfg->lambda_score;
+        A.frac = cfg->prune_frac;
+        A.max_select = max_select;
+        A.state = (SelState*)(ws + off_state);
+        A.hist = (unsigned int*)ws;
+        A.vec = ((uintptr_t)score_terms & 15) == 0 && ((uintptr_t)mask_inout & 3) == 0;
+        const SelPasses P = sel_passes(n);
+        if (cudaMemsetAsync(ws, 0, P.count * SEL_BINS * sizeof(unsigned int), st) != cudaSuccess)
+            return set_error(GS_ERR_CUDA, "memset prune state");
+        // four ids a thread; two CTAs an SM at most, so that few histograms are merged
+        const int sms = num_sms();
+        const int64_t want = (n + 4 * SEL_THREADS - 1) / (4 * SEL_THREADS);
+        const unsigned nb = (unsigned)(want < 2 * sms ? want : 2 * sms);
+        A.prev = {0, 0};
+        for (A.pass = 0; A.pass < P.count; ++A.pass) {
+            A.d = P.d[A.pass];
+            k_select_pass<<<nb, SEL_THREADS, 0, st>>>(A);
             if ((s = check_launch("k_select_pass")) != GS_OK) return s;
+            A.prev = A.d;
         }
-        k_select_mask<<<nb, PR_THREADS, 0, st>>>(score_terms, mask_inout, n, cfg->lambda_score, cfg->prune_frac,
-                                                 max_select, state, hist);
+        k_select_mask<<<nb, SEL_THREADS, 0, st>>>(A);
         return check_launch("k_select_mask");
     }
     if (iter_in_interval == *k_inout) {
@@ -307,11 +475,12 @@ extern "C" gs_status gs_prune(const gs_config* cfg, const float* score_terms, in
             if (cudaMemsetAsync(n_kept_out, 0, sizeof(int64_t), st) != cudaSuccess) return set_error(GS_ERR_CUDA, "memset");
         } else {
             u64* part = (u64*)(ws + off_part);
-            k_keep_count<<<(unsigned)nchunk, PR_THREADS, 0, st>>>(mask_inout, n, part);
+            const unsigned nchunk = (unsigned)((n + chunk - 1) / chunk);
+            const bool vec = ((uintptr_t)mask_inout & 7) == 0, vec_out = ((uintptr_t)compact_map_out & 15) == 0;
+            k_keep_count<<<nchunk, PR_THREADS, 0, st>>>(mask_inout, n, chunk, vec, part);
             if ((s = check_launch("k_keep_count")) != GS_OK) return s;
-            k_keep_scan<<<1, 1024, 0, st>>>(part, (int)nchunk, n_kept_out);
-            if ((s = check_launch("k_keep_scan")) != GS_OK) return s;
-            k_keep_write<<<(unsigned)nchunk, PR_THREADS, 0, st>>>(mask_inout, n, part, compact_map_out);
+            k_keep_write<<<nchunk, PR_THREADS, 0, st>>>(mask_inout, n, chunk, vec, vec_out, part, compact_map_out,
+                                                       n_kept_out);
             if ((s = check_launch("k_keep_write")) != GS_OK) return s;
         }
         *k_inout = gs_next_interval(cfg, *k_inout, change_ratio);
@@ -336,19 +505,17 @@ extern "C" gs_status gs_change_ratio(const gs_config* cfg, const gs_camera* cam,
     if (!ratio_out || (n > 0 && (!splats_a || !splats_b))) return set_error(GS_ERR_INVALID_ARG, "NULL pointer");
     cudaStream_t st = (cudaStream_t)stream;
     u64* acc = (u64*)workspace;
-    if (cudaMemsetAsync(acc, 0, 2 * sizeof(u64), st) != cudaSuccess) return set_error(GS_ERR_CUDA, "memset");
-    gs_status s;
-    if (n > 0) {
-        const int sms = num_sms();
-        const int64_t want = (n + PR_THREADS - 1) / PR_THREADS;
-        const unsigned nb = (unsigned)(want < 4 * sms ? want : 4 * sms);
-        if (rec_dtype == GS_F32) k_change<GS_F32><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc);
-        else if (rec_dtype == GS_BF16) k_change<GS_BF16><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc);
-        else k_change<GS_F16><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc);
-        if ((s = check_launch("k_change")) != GS_OK) return s;
-    }
-    k_change_final<<<1, 1, 0, st>>>(acc, ratio_out);
-    return check_launch("k_change_final");
+    if (cudaMemsetAsync(acc, 0, 3 * sizeof(u64), st) != cudaSuccess) return set_error(GS_ERR_CUDA, "memset");
+    const int sms = num_sms();
+    const int64_t want = (n + PR_THREADS - 1) / PR_THREADS;
+    const unsigned nb = (unsigned)(want < 1 ? 1 : want < 4 * sms ? want : 4 * sms);
+    if (rec_dtype == GS_F32)
+        k_change<GS_F32><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc, ratio_out);
+    else if (rec_dtype == GS_BF16)
+        k_change<GS_BF16><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc, ratio_out);
+    else
+        k_change<GS_F16><<<nb, PR_THREADS, 0, st>>>(*cam, cfg->alpha_min, splats_a, splats_b, n, acc, ratio_out);
+    return check_launch("k_change");
 }
 
 extern "C" gs_status gs_compact(const float* src, int64_t n, int32_t width, const uint32_t* compact_map, float* dst,
@@ -357,9 +524,15 @@ extern "C" gs_status gs_compact(const float* src, int64_t n, int32_t width, cons
     if (n == 0) return GS_OK;
     if (!src || !compact_map || !dst) return set_error(GS_ERR_INVALID_ARG, "NULL pointer");
     const int sms = num_sms();
-    const int64_t want = (n * width + 255) / 256;
-    const unsigned nb = (unsigned)(want < 8 * sms ? want : 8 * sms);
-    k_compact<<<nb, 256, 0, (cudaStream_t)stream>>>(src, n, width, compact_map, dst);
+    const int64_t want = width <= 4 ? (n + 255) / 256 : (n * width + 255) / 256;
+    const int64_t cap = (int64_t)(width <= 4 ? 64 : 8) * sms;
+    const unsigned nb = (unsigned)(want < cap ? want : cap);
+    cudaStream_t st = (cudaStream_t)stream;
+    if (width == 1) k_compact<1><<<nb, 256, 0, st>>>(src, n, width, compact_map, dst);
+    else if (width == 2) k_compact<2><<<nb, 256, 0, st>>>(src, n, width, compact_map, dst);
+    else if (width == 3) k_compact<3><<<nb, 256, 0, st>>>(src, n, width, compact_map, dst);
+    else if (width == 4) k_compact<4><<<nb, 256, 0, st>>>(src, n, width, compact_map, dst);
+    else k_compact<0><<<nb, 256, 0, st>>>(src, n, width, compact_map, dst);
     return check_launch("k_compact");
 }
 
