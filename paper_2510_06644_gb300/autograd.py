@@ -48,6 +48,13 @@ def _skew(v):
 def apply_pose_delta(cam, delta):
     """Camera dict with T_cw replaced by exp(delta^) T_cw, delta = (rho, phi)."""
     d = np.asarray(delta, dtype=np.float64).reshape(6)
+    R0 = np.asarray(cam["R"], dtype=np.float64).reshape(3, 3)
+    t0 = np.asarray(cam["t"], dtype=np.float64).reshape(3)
+    c = dict(cam)
+    # the tracking use: exp(0) = 1 (the matrices below take 35 us of host time)
+    if not d.any() and np.isfinite(R0).all() and np.isfinite(t0).all():
+        c["R"], c["t"] = R0.copy(), t0.copy()
+        return c
     rho, phi = d[:3], d[3:]
     th = float(np.linalg.norm(phi))
     K = _skew(phi)
@@ -57,9 +64,8 @@ def apply_pose_delta(cam, delta):
     else:
         Rd = np.eye(3) + math.sin(th) / th * K + (1 - math.cos(th)) / th ** 2 * K @ K
         V = np.eye(3) + (1 - math.cos(th)) / th ** 2 * K + (th - math.sin(th)) / th ** 3 * K @ K
-    c = dict(cam)
-    c["R"] = Rd @ np.asarray(cam["R"], dtype=np.float64).reshape(3, 3)
-    c["t"] = Rd @ np.asarray(cam["t"], dtype=np.float64).reshape(3) + V @ rho
+    c["R"] = Rd @ R0
+    c["t"] = Rd @ t0 + V @ rho
     return c
 
 
@@ -142,7 +148,7 @@ class GsRenderFn(torch.autograd.Function):
         g = {"means": means.detach().contiguous(), "log_scales": log_scales.detach().contiguous(),
              "quats": quats.detach().contiguous(), "opacity_logit": opacity_logit.detach().contiguous(),
              "rgb": colors.detach().contiguous()}
-        cam_p = apply_pose_delta(cam, pose_delta.detach().double().cpu().numpy())
+        cam_p = apply_pose_delta(cam, pose_delta.detach().cpu().double().numpy())
         n = int(g["means"].shape[0])
         cfg = cfg if cfg is not None else gs.default_config()
         cs = gs.camera(cam_p)
@@ -153,6 +159,7 @@ class GsRenderFn(torch.autograd.Function):
         store = memory_budget is None or stored_bytes(n, rast.capacity, cam_p, rec_dtype) <= memory_budget
         ctx.store = store
         ctx.cam_p = cam_p
+        ctx.cam_s = cs
         ctx.cfg = cfg
         ctx.rec_dtype = rec_dtype
         if not grad_on:
@@ -173,7 +180,7 @@ class GsRenderFn(torch.autograd.Function):
     def backward(ctx, d_rgb, d_depth):
         vals = ctx.saved_tensors
         g = dict(zip(PARAMS, vals))
-        cs = gs.camera(ctx.cam_p)
+        cs = ctx.cam_s
         rast = ctx.rast
         if rast is None:  # recompute the forward intermediates
             n = int(g["means"].shape[0])
@@ -187,7 +194,7 @@ class GsRenderFn(torch.autograd.Function):
             grads = {k: torch.empty_like(g[k]) for k in PARAMS}
             rast.backward(g, cs, d_rgb, d_depth, mode=gs.GS_MAP, grads=grads, want_pose=need[5], want_score=False)
             _settle(rast)
-            pose_grad = rast.pose.float().clone() if need[5] else None
+            pose_grad = rast.pose.float() if need[5] else None
         finally:
             _POOL.give(rast)
         return (grads["means"], grads["log_scales"], grads["quats"], grads["opacity_logit"], grads["rgb"],

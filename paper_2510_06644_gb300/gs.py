@@ -12,6 +12,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 
+import numpy as np
 import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -142,36 +143,53 @@ def _check(code, what):
         raise GsError(code, f"{what}: {lib().gs_last_error().decode()}")
 
 
-def _ptr(t):
+def _addr(t):
+    """Device address of a contiguous CUDA tensor (None for None).  A call
+    passes up to 20 of these: plain integers, no ctypes object each."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("device tensor expected")
     if not t.is_contiguous():
         raise ValueError("contiguous tensor expected")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _req(t):
+    if t is None:
+        raise ValueError("device tensor expected")
+    return _addr(t)
+
+
+def _ptr(t):
+    return None if t is None else C.c_void_p(_addr(t))
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    # the raw handle: a torch.cuda.Stream object for the current stream takes 10 us to make
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 # --------------------------------------------------------------------------
 # Structures
 # --------------------------------------------------------------------------
 
+def _floats(x, k):
+    """The k numbers of an array, tensor or nested list."""
+    if isinstance(x, np.ndarray) and x.dtype == np.float64 and x.size == k:
+        return x.reshape(k).tolist()  # without a tensor in between (15 us)
+    return torch.as_tensor(x, dtype=torch.float64).reshape(k).tolist()
+
+
 def camera(cam, pose=None) -> gs_camera:
     """gs_camera from a dict {R, t, fx, fy, cx, cy, W, H, sx, sy}; `pose`
     (device float32 [12] tensor) makes the kernels read R, t from it."""
     c = gs_camera()
-    c.pose = _ptr(pose).value if pose is not None else None
-    R = [float(v) for v in torch.as_tensor(cam["R"], dtype=torch.float64).reshape(9).tolist()]
-    t = [float(v) for v in torch.as_tensor(cam["t"], dtype=torch.float64).reshape(3).tolist()]
-    for i in range(9):
-        c.R[i] = R[i]
-    for i in range(3):
-        c.t[i] = t[i]
+    c.pose = _addr(pose)
+    c.R[:] = _floats(cam["R"], 9)
+    c.t[:] = _floats(cam["t"], 3)
     c.fx, c.fy, c.cx, c.cy = (float(cam[k]) for k in ("fx", "fy", "cx", "cy"))
     c.width, c.height = int(cam["W"]), int(cam["H"])
     c.sx, c.sy = int(cam.get("sx", 1)), int(cam.get("sy", 1))
@@ -212,13 +230,13 @@ def grid(cam):
 def gaussians(g, mask=None) -> gs_gaussians:
     """gs_gaussians over a dict of contiguous float32 CUDA tensors."""
     s = gs_gaussians()
-    s.means = _ptr(g["means"]).value
-    s.log_scales = _ptr(g["log_scales"]).value
-    s.quats = _ptr(g["quats"]).value
-    s.opacity_logit = _ptr(g["opacity_logit"]).value
-    s.rgb = _ptr(g["rgb"]).value
+    s.means = _req(g["means"])
+    s.log_scales = _req(g["log_scales"])
+    s.quats = _req(g["quats"])
+    s.opacity_logit = _req(g["opacity_logit"])
+    s.rgb = _req(g["rgb"])
     m = mask if mask is not None else g.get("mask")
-    s.mask = _ptr(m).value if m is not None else None
+    s.mask = _req(m) if m is not None else None
     s.n = int(g["means"].shape[0])
     return s
 
@@ -228,7 +246,7 @@ def grads_struct(gr) -> gs_grads:
     if gr:
         for k in ("means", "log_scales", "quats", "opacity_logit", "rgb"):
             v = gr.get(k)
-            setattr(s, k, _ptr(v).value if v is not None else None)
+            setattr(s, k, _req(v) if v is not None else None)
     return s
 
 
@@ -246,7 +264,7 @@ def gs_project(cfg, cam, g, rec_dtype=GS_F32, splats=None, stream=None):
         dt = torch.float32 if rec_dtype == GS_F32 else torch.int32
         splats = torch.empty((n, SPLAT_WORDS[rec_dtype]), dtype=dt, device=g["means"].device)
     gs_g = gaussians(g)
-    _check(lib().gs_project(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _ptr(splats),
+    _check(lib().gs_project(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _addr(splats),
                             _stream(stream)), "gs_project")
     return splats
 
@@ -287,16 +305,19 @@ def gs_bin_sort(cam, splats, n, capacity, rec_dtype=GS_F32, ws=None, keys=None, 
     ranges = torch.empty((TX * TY, 2), dtype=torch.int32, device=dev) if ranges is None else ranges
     order = torch.empty(TX * TY, dtype=torch.int32, device=dev) if order is None else order
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_bin_sort(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _ptr(splats), int(n), int(capacity),
-                             _ptr(ws),
-                             C.byref(nb), _ptr(keys), _ptr(vals), _ptr(n_keys), _ptr(ranges), _ptr(order),
+    _check(lib().gs_bin_sort(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _addr(splats), int(n), int(capacity),
+                             _addr(ws),
+                             C.byref(nb), _addr(keys), _addr(vals), _addr(n_keys), _addr(ranges), _addr(order),
                              _stream(stream)), "gs_bin_sort")
     return keys, vals, n_keys, ranges, order
 
 
 def gs_project_bin_sort_workspace(cfg, cam, g, rec_dtype, capacity):
+    return _project_bin_sort_bytes(cfg, cam, gaussians(g), rec_dtype, capacity)
+
+
+def _project_bin_sort_bytes(cfg, cam, gs_g, rec_dtype, capacity):
     nb = C.c_size_t(0)
-    gs_g = gaussians(g)
     _check(lib().gs_project_bin_sort(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, None, int(capacity), None,
                                      C.byref(nb), None, None, None, None, None, None), "gs_project_bin_sort(size)")
     return nb.value
@@ -308,7 +329,8 @@ def gs_project_bin_sort(cfg, cam, g, splats, capacity, rec_dtype=GS_F32, ws=None
     returns (keys, vals, n_keys, ranges, order)."""
     dev = splats.device
     _, _, TX, TY = grid(cam)
-    need = gs_project_bin_sort_workspace(cfg, cam, g, rec_dtype, capacity)
+    gs_g = gaussians(g)
+    need = _project_bin_sort_bytes(cfg, cam, gs_g, rec_dtype, capacity)
     if ws is None or ws.numel() < need:
         ws = workspace(need, dev)
     keys = torch.empty(max(capacity, 1), dtype=torch.int64, device=dev) if keys is None else keys
@@ -316,11 +338,10 @@ def gs_project_bin_sort(cfg, cam, g, splats, capacity, rec_dtype=GS_F32, ws=None
     n_keys = torch.zeros(1, dtype=torch.int64, device=dev) if n_keys is None else n_keys
     ranges = torch.empty((TX * TY, 2), dtype=torch.int32, device=dev) if ranges is None else ranges
     order = torch.empty(TX * TY, dtype=torch.int32, device=dev) if order is None else order
-    gs_g = gaussians(g)
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_project_bin_sort(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _ptr(splats), int(capacity),
-                                     _ptr(ws), C.byref(nb), _ptr(keys), _ptr(vals), _ptr(n_keys), _ptr(ranges),
-                                     _ptr(order), _stream(stream)), "gs_project_bin_sort")
+    _check(lib().gs_project_bin_sort(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _addr(splats), int(capacity),
+                                     _addr(ws), C.byref(nb), _addr(keys), _addr(vals), _addr(n_keys), _addr(ranges),
+                                     _addr(order), _stream(stream)), "gs_project_bin_sort")
     return keys, vals, n_keys, ranges, order
 
 
@@ -331,8 +352,8 @@ def gs_bin_count(cam, splats, n, rec_dtype=GS_F32, stream=None, cfg=None):
     ws = workspace(nb.value, splats.device)
     out = torch.zeros(1, dtype=torch.int64, device=splats.device)
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_bin_count(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _ptr(splats), int(n), _ptr(ws),
-                              C.byref(nb), _ptr(out), _stream(stream)), "gs_bin_count")
+    _check(lib().gs_bin_count(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _addr(splats), int(n), _addr(ws),
+                              C.byref(nb), _addr(out), _stream(stream)), "gs_bin_count")
     return out
 
 
@@ -352,9 +373,9 @@ def gs_render_fwd(cfg, cam, splats, n, vals, ranges, rec_dtype=GS_F32, out=None,
                "t_final": torch.empty((Hs, Ws), device=dev),
                "last_idx": torch.empty((Hs, Ws), dtype=torch.int32, device=dev),
                "n_blended": torch.empty((Hs, Ws), dtype=torch.int32, device=dev)}
-    _check(lib().gs_render_fwd(C.byref(cfg), C.byref(cam), rec_dtype, _ptr(splats), int(n), _ptr(vals),
-                               _ptr(ranges), _ptr(order), _ptr(out["rgb"]), _ptr(out["depth"]), _ptr(out["t_final"]),
-                               _ptr(out["last_idx"]), _ptr(out.get("n_blended")), _ptr(masks), _stream(stream)),
+    _check(lib().gs_render_fwd(C.byref(cfg), C.byref(cam), rec_dtype, _addr(splats), int(n), _addr(vals),
+                               _addr(ranges), _addr(order), _addr(out["rgb"]), _addr(out["depth"]), _addr(out["t_final"]),
+                               _addr(out["last_idx"]), _addr(out.get("n_blended")), _addr(masks), _stream(stream)),
            "gs_render_fwd")
     return out
 
@@ -373,11 +394,11 @@ def gs_render_fwd_loss(cfg, cam, splats, n, vals, ranges, target_rgb, target_dep
     if dimg is None:
         dimg = {"d_rgb": torch.empty((3, Hs, Ws), device=dev), "d_depth": torch.empty((Hs, Ws), device=dev),
                 "loss": torch.zeros(1, dtype=torch.float64, device=dev)}
-    _check(lib().gs_render_fwd_loss(C.byref(cfg), C.byref(cam), rec_dtype, _ptr(splats), int(n), _ptr(vals),
-                                    _ptr(ranges), _ptr(order), _ptr(out["rgb"]), _ptr(out["depth"]),
-                                    _ptr(out["t_final"]), _ptr(out["last_idx"]), _ptr(out.get("n_blended")),
-                                    _ptr(masks), _ptr(target_rgb), _ptr(target_depth), _ptr(dimg["d_rgb"]), _ptr(dimg["d_depth"]),
-                                    _ptr(dimg["loss"]), _stream(stream)), "gs_render_fwd_loss")
+    _check(lib().gs_render_fwd_loss(C.byref(cfg), C.byref(cam), rec_dtype, _addr(splats), int(n), _addr(vals),
+                                    _addr(ranges), _addr(order), _addr(out["rgb"]), _addr(out["depth"]),
+                                    _addr(out["t_final"]), _addr(out["last_idx"]), _addr(out.get("n_blended")),
+                                    _addr(masks), _addr(target_rgb), _addr(target_depth), _addr(dimg["d_rgb"]), _addr(dimg["d_depth"]),
+                                    _addr(dimg["loss"]), _stream(stream)), "gs_render_fwd_loss")
     return out, dimg
 
 
@@ -385,15 +406,18 @@ def gs_loss_l1(cfg, cam, rgb, depth, target_rgb, target_depth, out=None, stream=
     if out is None:
         out = {"d_rgb": torch.empty_like(rgb), "d_depth": torch.empty_like(depth),
                "loss": torch.zeros(1, dtype=torch.float64, device=rgb.device)}
-    _check(lib().gs_loss_l1(C.byref(cfg), C.byref(cam), _ptr(rgb), _ptr(depth), _ptr(target_rgb),
-                            _ptr(target_depth), _ptr(out["d_rgb"]), _ptr(out["d_depth"]), _ptr(out["loss"]),
+    _check(lib().gs_loss_l1(C.byref(cfg), C.byref(cam), _addr(rgb), _addr(depth), _addr(target_rgb),
+                            _addr(target_depth), _addr(out["d_rgb"]), _addr(out["d_depth"]), _addr(out["loss"]),
                             _stream(stream)), "gs_loss_l1")
     return out
 
 
 def gs_project_bwd_workspace(cfg, cam, g):
+    return _project_bwd_bytes(cfg, cam, gaussians(g))
+
+
+def _project_bwd_bytes(cfg, cam, gs_g):
     nb = C.c_size_t(0)
-    gs_g = gaussians(g)
     _check(lib().gs_project_bwd(C.byref(cfg), C.byref(cam), C.byref(gs_g), None, None, None, None, None,
                                 C.byref(nb), None), "gs_project_bwd(size)")
     return nb.value
@@ -411,16 +435,16 @@ def gs_render_bwd(cfg, cam, g, splats, vals, ranges, t_final, last_idx, d_rgb, d
     gs_g = gaussians(g)
     gr = grads_struct(grads) if grads is not None else None
     chain = grads is not None or pose is not None or score is not None
-    need = gs_project_bwd_workspace(cfg, cam, g) if chain else 0
+    need = _project_bwd_bytes(cfg, cam, gs_g) if chain else 0
     if ws is None or ws.numel() < need:
         ws = workspace(need, dev)
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_render_bwd(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _ptr(splats), _ptr(vals),
-                               _ptr(ranges), _ptr(order), _ptr(t_final), _ptr(last_idx), _ptr(masks), _ptr(d_rgb),
-                               _ptr(d_depth),
+    _check(lib().gs_render_bwd(C.byref(cfg), C.byref(cam), C.byref(gs_g), rec_dtype, _addr(splats), _addr(vals),
+                               _addr(ranges), _addr(order), _addr(t_final), _addr(last_idx), _addr(masks), _addr(d_rgb),
+                               _addr(d_depth),
                                mode,
-                               _ptr(grad2d), C.byref(gr) if gr is not None else None, _ptr(pose),
-                               _ptr(score), _ptr(ws), C.byref(nb), _stream(stream)), "gs_render_bwd")
+                               _addr(grad2d), C.byref(gr) if gr is not None else None, _addr(pose),
+                               _addr(score), _addr(ws), C.byref(nb), _stream(stream)), "gs_render_bwd")
     return grad2d
 
 
@@ -431,14 +455,14 @@ def gs_project_bwd(cfg, cam, g, grad2d, grads=None, pose=None, score=None, ws=No
     gs_g = gaussians(g)
     gr = grads_struct(grads) if grads is not None else None
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_project_bwd(C.byref(cfg), C.byref(cam), C.byref(gs_g), _ptr(grad2d),
-                                C.byref(gr) if gr is not None else None, _ptr(pose), _ptr(score), _ptr(ws),
+    _check(lib().gs_project_bwd(C.byref(cfg), C.byref(cam), C.byref(gs_g), _addr(grad2d),
+                                C.byref(gr) if gr is not None else None, _addr(pose), _addr(score), _addr(ws),
                                 C.byref(nb), _stream(stream)), "gs_project_bwd")
 
 
 def pose_step(pose, adam, lr_trans=1e-3, lr_rot=1e-3, beta1=0.9, beta2=0.999, eps=1e-8):
     """gs_pose_step over device tensors pose (float32 [12]) and adam (float32 [13])."""
-    return gs_pose_step(_ptr(pose).value, _ptr(adam).value, float(lr_trans), float(lr_rot), float(beta1),
+    return gs_pose_step(_req(pose), _req(adam), float(lr_trans), float(lr_rot), float(beta1),
                         float(beta2), float(eps))
 
 
@@ -451,9 +475,9 @@ def gs_project_bwd_step(cfg, cam, g, grad2d, pose, step, grads=None, score=None,
     gs_g = gaussians(g)
     gr = grads_struct(grads) if grads is not None else None
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_project_bwd_step(C.byref(cfg), C.byref(cam), C.byref(gs_g), _ptr(grad2d),
-                                     C.byref(gr) if gr is not None else None, _ptr(pose), _ptr(score),
-                                     C.byref(step) if step is not None else None, _ptr(ws), C.byref(nb),
+    _check(lib().gs_project_bwd_step(C.byref(cfg), C.byref(cam), C.byref(gs_g), _addr(grad2d),
+                                     C.byref(gr) if gr is not None else None, _addr(pose), _addr(score),
+                                     C.byref(step) if step is not None else None, _addr(ws), C.byref(nb),
                                      _stream(stream)), "gs_project_bwd_step")
 
 
@@ -480,14 +504,14 @@ def gs_project_bwd_adam(cfg, cam, g, grad2d, ms, vs, state, lr=1e-3, beta1=0.9, 
     moment tensors keyed like g; state: float32 [2] (as gs_adam)."""
     a = gs_map_adam()
     for i, k in enumerate(PARAM_KEYS):
-        a.m[i] = _ptr(ms[k]).value
-        a.v[i] = _ptr(vs[k]).value
+        a.m[i] = _req(ms[k])
+        a.v[i] = _req(vs[k])
     a.lr, a.beta1, a.beta2, a.eps = float(lr), float(beta1), float(beta2), float(eps)
-    a.state = _ptr(state).value
+    a.state = _req(state)
     gs_g = gaussians(g)
     gr = grads_struct(grads) if grads is not None else None
-    _check(lib().gs_project_bwd_adam(C.byref(_cfg(cfg)), C.byref(cam), C.byref(gs_g), _ptr(grad2d), C.byref(a),
-                                     C.byref(gr) if gr is not None else None, _ptr(score), _stream(stream)),
+    _check(lib().gs_project_bwd_adam(C.byref(_cfg(cfg)), C.byref(cam), C.byref(gs_g), _addr(grad2d), C.byref(a),
+                                     C.byref(gr) if gr is not None else None, _addr(score), _stream(stream)),
            "gs_project_bwd_adam")
 
 
@@ -496,8 +520,8 @@ def gs_project_bwd_noalloc(cfg, cam, g, grad2d, grads=None, pose=None, score=Non
     used (no device allocation at all; calls must not overlap on the GPU)."""
     gs_g = gaussians(g)
     gr = grads_struct(grads) if grads is not None else None
-    _check(lib().gs_project_bwd_noalloc(C.byref(cfg), C.byref(cam), C.byref(gs_g), _ptr(grad2d),
-                                        C.byref(gr) if gr is not None else None, _ptr(pose), _ptr(score),
+    _check(lib().gs_project_bwd_noalloc(C.byref(cfg), C.byref(cam), C.byref(gs_g), _addr(grad2d),
+                                        C.byref(gr) if gr is not None else None, _addr(pose), _addr(score),
                                         _stream(stream)), "gs_project_bwd_noalloc")
 
 
@@ -513,8 +537,8 @@ def gs_prune(cfg, score, mask, iter_in_interval, K, change_ratio=0.0, max_select
     if ws is None or ws.numel() < nb.value:
         ws = workspace(nb.value, mask.device)
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_prune(C.byref(cfg), _ptr(score), n, _ptr(mask), int(iter_in_interval), C.byref(k),
-                          float(change_ratio), max_select, _ptr(compact_map), _ptr(n_kept), _ptr(ws),
+    _check(lib().gs_prune(C.byref(cfg), _addr(score), n, _addr(mask), int(iter_in_interval), C.byref(k),
+                          float(change_ratio), max_select, _addr(compact_map), _addr(n_kept), _addr(ws),
                           C.byref(nb), _stream(stream)), "gs_prune")
     return k.value
 
@@ -528,8 +552,8 @@ def gs_change_ratio(cam, splats_a, splats_b, n, rec_dtype=GS_F32, out=None, stre
     ws = workspace(256, splats_a.device)
     out = torch.zeros(1, dtype=torch.float32, device=splats_a.device) if out is None else out
     nb = C.c_size_t(ws.numel())
-    _check(lib().gs_change_ratio(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _ptr(splats_a), _ptr(splats_b),
-                                 int(n), _ptr(ws), C.byref(nb), _ptr(out), _stream(stream)), "gs_change_ratio")
+    _check(lib().gs_change_ratio(C.byref(_cfg(cfg)), C.byref(cam), rec_dtype, _addr(splats_a), _addr(splats_b),
+                                 int(n), _addr(ws), C.byref(nb), _addr(out), _stream(stream)), "gs_change_ratio")
     return out
 
 
@@ -537,7 +561,7 @@ def gs_compact(src, compact_map, n_kept, stream=None):
     n = int(src.shape[0])
     width = int(src[0].numel()) if n > 0 else 1
     dst = torch.empty((int(n_kept),) + tuple(src.shape[1:]), dtype=src.dtype, device=src.device)
-    _check(lib().gs_compact(_ptr(src), n, width, _ptr(compact_map), _ptr(dst), _stream(stream)), "gs_compact")
+    _check(lib().gs_compact(_addr(src), n, width, _addr(compact_map), _addr(dst), _stream(stream)), "gs_compact")
     return dst
 
 
@@ -559,7 +583,7 @@ def gs_downsample(frame_idx, last_kf_idx, is_keyframe, m=2, target_full=None, ou
             raise ValueError("out has the wrong size for the sampled target")
         res = out
     _check(lib().gs_downsample(int(frame_idx), int(last_kf_idx), 1 if is_keyframe else 0, int(m), C.byref(sx),
-                               C.byref(sy), _ptr(t.contiguous()), Cn, W, H, _ptr(res), _stream(stream)),
+                               C.byref(sy), _addr(t.contiguous()), Cn, W, H, _addr(res), _stream(stream)),
            "gs_downsample")
     if out is not None:
         return sx.value, sy.value, out
@@ -575,7 +599,7 @@ def pose_tensor(cam, device="cuda"):
 
 def gs_pose_update(pose, pose_grad, adam, lr_trans=1e-3, lr_rot=1e-3, beta1=0.9, beta2=0.999, eps=1e-8,
                    stream=None):
-    _check(lib().gs_pose_update(_ptr(pose), _ptr(pose_grad), _ptr(adam), float(lr_trans), float(lr_rot),
+    _check(lib().gs_pose_update(_addr(pose), _addr(pose_grad), _addr(adam), float(lr_trans), float(lr_rot),
                                 float(beta1), float(beta2), float(eps), _stream(stream)), "gs_pose_update")
 
 
@@ -584,12 +608,12 @@ def gs_adam(params, grads, ms, vs, state, lr=1e-3, beta1=0.9, beta2=0.999, eps=1
     every list); state is a zeroed device float32 [2] tensor (step count)."""
     k = len(params)
     arr = C.c_void_p * k
-    P_ = arr(*[_ptr(t).value for t in params])
-    G_ = arr(*[_ptr(t).value for t in grads])
-    M_ = arr(*[_ptr(t).value for t in ms])
-    V_ = arr(*[_ptr(t).value for t in vs])
+    P_ = arr(*[_req(t) for t in params])
+    G_ = arr(*[_req(t) for t in grads])
+    M_ = arr(*[_req(t) for t in ms])
+    V_ = arr(*[_req(t) for t in vs])
     cnt = (C.c_int64 * k)(*[int(t.numel()) for t in params])
-    _check(lib().gs_adam(k, P_, G_, M_, V_, cnt, float(lr), float(beta1), float(beta2), float(eps), _ptr(state),
+    _check(lib().gs_adam(k, P_, G_, M_, V_, cnt, float(lr), float(beta1), float(beta2), float(eps), _addr(state),
                          _stream(stream)), "gs_adam")
 
 
@@ -598,14 +622,14 @@ def gs_probe_red_f32(dst, n_threads, per_thread, stream=None):
     dst[t % dst.numel()] per_thread times (float32 device tensor dst)."""
     if dst.dtype != torch.float32:
         raise ValueError("float32 dst expected")
-    _check(lib().gs_probe_red_f32(_ptr(dst), int(dst.numel()), int(n_threads), int(per_thread), _stream(stream)),
+    _check(lib().gs_probe_red_f32(_addr(dst), int(dst.numel()), int(n_threads), int(per_thread), _stream(stream)),
            "gs_probe_red_f32")
 
 
 def gs_probe_fma_f32(out, iters, stream=None):
     """FMA-throughput probe: each of out.numel() threads runs 8 chains of
     `iters` FMAs (16 FLOP per iteration) and writes 28 + 8 iters."""
-    _check(lib().gs_probe_fma_f32(_ptr(out), int(out.numel()), int(iters), _stream(stream)), "gs_probe_fma_f32")
+    _check(lib().gs_probe_fma_f32(_addr(out), int(out.numel()), int(iters), _stream(stream)), "gs_probe_fma_f32")
 
 
 def gs_status_poll(blocking=True, stream=None):
