@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_count(gs_camera cam, float
 //   k_tile_scatter_rows  CTA c starts tile t's slots at start[t] +
 //                    hist[c][t] and deals them out with shared-memory atomics.
 #define AGG_MAX_TILES 8192
+#define AGG_ROWS 912         // one wave of six counting CTAs on 152 SMs
 
 template <int DT>
 __global__ void __launch_bounds__(BIN_THREADS) k_tile_hist(gs_camera cam, float alpha_min, const void* __restrict__ splats, int64_t n,
@@ -951,7 +952,9 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // would pass 2^24 entries (64 MB).
 static int64_t agg_per_cta(int64_t n, int ntiles) {
     const int64_t lim = (int64_t)1 << 24;
-    const int64_t want = (n * (int64_t)ntiles + lim - 1) / lim;
+    int64_t want = (n * (int64_t)ntiles + lim - 1) / lim;
+    const int64_t wave = (n + AGG_ROWS - 1) / AGG_ROWS;
+    if (want < wave) want = wave;
     return want > 2 * BIN_THREADS ? want : 2 * BIN_THREADS;
 }
 

@@ -192,7 +192,11 @@ __device__ __forceinline__ void project_hist_body(gs_camera cam, const gs_config
 }
 
 template <int DT>
-__global__ void __launch_bounds__(256) k_project_hist(gs_camera cam, gs_config cfg, gs_gaussians g, void* out,
+// Issue-bound (its 32 instructions a byte are the projection and the rect), and
+// the shared row's zeroing and writing wait on barriers: six CTAs an SM in 40
+// registers hide them best (1M Gaussians 40 -> 36.5 us, 3M 122 -> 112, both
+// with the rows of one wave).
+__global__ void __launch_bounds__(256, 6) k_project_hist(gs_camera cam, gs_config cfg, gs_gaussians g, void* out,
                                                       int64_t per, int ntiles, uint32_t* __restrict__ hist,
                                                       uint2* __restrict__ rects) {
     project_hist_body<DT>(cam, cfg, g, out, per, ntiles, hist, rects, (int)blockIdx.x);
@@ -203,10 +207,25 @@ __global__ void __launch_bounds__(256) k_project_hist(gs_camera cam, gs_config c
 // ---------------------------------------------------------------------------
 
 #define PB_THREADS 256
-#define PB_PER 2          // Gaussians per thread of the backward projection with the pose
+#define PB_PER 2          // least Gaussians per thread of the backward projection with the pose
+#define PB_CTAS 3         // its CTAs per SM
 
 // Blocks of the backward projection for n Gaussians, per Gaussians a thread.
-static inline int64_t pb_blocks(int64_t n, int per) { return (n + per * PB_THREADS - 1) / (per * PB_THREADS); }
+static inline int64_t pb_blocks(int64_t n, int per) {
+    return (n + (int64_t)per * PB_THREADS - 1) / ((int64_t)per * PB_THREADS);
+}
+
+// Gaussians a thread takes when the pose is reduced: as many as make the launch
+// one wave of PB_CTAS CTAs an SM.  Every CTA pays a block reduction of the six
+// components and its partial is read again by the last block, alone on the chip
+// at the end: with two a thread at any size, 3M Gaussians with gradients took
+// 188 us at 2 CTAs an SM (128 registers), 151 at 4, and in one wave 130 at 4
+// and 119 at 3; 1M 72, 63, 55 and 51; 458k without gradients 24.4 and 20.5.
+static int pb_per(int64_t n) {
+    const int64_t wave = (int64_t)PB_THREADS * PB_CTAS * num_sms();
+    const int64_t per = (n + wave - 1) / wave;
+    return per > PB_PER ? (int)per : PB_PER;
+}
 
 // The pose gradient is a sum over every Gaussian of terms of both signs
 // (the Merging Tree of Sec. 5.1 reduces it in hardware).  Inside a block the
@@ -388,16 +407,27 @@ struct AdamMap {
     AdamStep s;  // formed in the kernel
 };
 
-// PER Gaussians per thread: two when the pose is reduced (391 blocks of 256
-// fit one wave on the tracking frame: 21.5 -> 19.5 us), one otherwise (the
-// mapping step's per-Gaussian gradients and Adam update are memory-bound and
-// want every thread: 0.936 against 0.979 ms per mapping iteration).
-template <bool WANT_GRADS, bool WANT_POSE, bool WANT_SCORE, bool ADAM = false, int PER = WANT_POSE ? PB_PER : 1>
+// A Gaussian's 14 values of the five arrays (3, 3, 4, 1 and 3 wide), in order.
+__device__ __forceinline__ void adam_load(float* const* a, int64_t k, float* x) {
+    for (int i = 0; i < 3; ++i) { x[i] = a[0][3 * k + i]; x[3 + i] = a[1][3 * k + i]; x[11 + i] = a[4][3 * k + i]; }
+    for (int i = 0; i < 4; ++i) x[6 + i] = a[2][4 * k + i];
+    x[10] = a[3][k];
+}
+__device__ __forceinline__ void adam_store(float* const* a, int64_t k, const float* x) {
+    for (int i = 0; i < 3; ++i) { a[0][3 * k + i] = x[i]; a[1][3 * k + i] = x[3 + i]; a[4][3 * k + i] = x[11 + i]; }
+    for (int i = 0; i < 4; ++i) a[2][4 * k + i] = x[6 + i];
+    a[3][k] = x[10];
+}
+
+// per: Gaussians per thread when the pose is reduced (pb_per), one otherwise
+// (the mapping step's per-Gaussian gradients and Adam update want every thread:
+// 0.936 against 0.979 ms per mapping iteration).
+template <bool WANT_GRADS, bool WANT_POSE, bool WANT_SCORE, bool ADAM = false>
 __device__ __forceinline__ void project_bwd_body(gs_camera cam, const gs_config& cfg, const gs_gaussians& g,
                                                  const float* __restrict__ grad2d, const gs_grads& grads,
                                                  float* __restrict__ score, float2* __restrict__ pose_part,
                                                  double* __restrict__ pose_out, unsigned int* __restrict__ ticket,
-                                                 const gs_pose_step& step, int blk, int nblk,
+                                                 const gs_pose_step& step, int blk, int nblk, int per,
                                                  const AdamMap* adam = nullptr) {
     // the thread's pose terms, summed as float32 pairs over its Gaussians
     DF pacc[6];
@@ -405,8 +435,8 @@ __device__ __forceinline__ void project_bwd_body(gs_camera cam, const gs_config&
     for (int i = 0; i < 6; ++i) pacc[i] = DF{0.f, 0.f};
     resolve_pose(cam);
 #pragma unroll 1
-    for (int rep = 0; rep < PER; ++rep) {
-        const int64_t k = ((int64_t)blk * PER + rep) * blockDim.x + threadIdx.x;
+    for (int rep = 0; rep < (WANT_POSE ? per : 1); ++rep) {
+        const int64_t k = ((int64_t)blk * (WANT_POSE ? per : 1) + rep) * blockDim.x + threadIdx.x;
         float pose[6] = {0, 0, 0, 0, 0, 0};
         if (k < g.n) {
             float mu[3], ls[3], q[4];
@@ -539,20 +569,26 @@ __device__ __forceinline__ void project_bwd_body(gs_camera cam, const gs_config&
                 // which is zero for culled Gaussians; keep zeros.
             }
             if (ADAM) {
+                // All 31 loads before the first store: element by element they
+                // would wait behind the stores to arrays that might overlap, a
+                // trip to memory each (1.5M Gaussians 170 us; now 142 at 3 CTAs
+                // an SM in 80 registers, 184 at 2.  4 CTAs would take 137, but
+                // in 64 registers the compiler rounds the gradients' products
+                // otherwise than in the kernel without Adam).
                 const AdamMap& A = *adam;
-                float* const gv[5] = {gmu, gls, gq, &gol, grgb};
-                const int width[5] = {3, 3, 4, 1, 3};
-    #pragma unroll
-                for (int t = 0; t < 5; ++t)
-    #pragma unroll
-                    for (int i = 0; i < width[t]; ++i) {
-                        const size_t e = (size_t)width[t] * k + i;
-                        float pp = A.p[t][e], mm = A.m[t][e], vv = A.v[t][e];
-                        adam_elem(pp, mm, vv, gv[t][i], A.b1, A.b2, A.s, A.eps);
-                        A.p[t][e] = pp;
-                        A.m[t][e] = mm;
-                        A.v[t][e] = vv;
-                    }
+                float am[14], av[14], ac[3];
+                adam_load(adam->m, k, am);
+                adam_load(adam->v, k, av);
+                for (int i = 0; i < 3; ++i) ac[i] = adam->p[4][3 * k + i];
+                float pp[14] = {mu[0], mu[1], mu[2], ls[0], ls[1], ls[2], q[0],
+                                q[1], q[2], q[3], ol, ac[0], ac[1], ac[2]};
+                const float gg[14] = {gmu[0], gmu[1], gmu[2], gls[0], gls[1], gls[2], gq[0],
+                                      gq[1], gq[2], gq[3], gol, grgb[0], grgb[1], grgb[2]};
+#pragma unroll
+                for (int i = 0; i < 14; ++i) adam_elem(pp[i], am[i], av[i], gg[i], A.b1, A.b2, A.s, A.eps);
+                adam_store(A.p, k, pp);
+                adam_store(A.m, k, am);
+                adam_store(A.v, k, av);
             }
             if (WANT_GRADS) {
                 if (grads.means) for (int i = 0; i < 3; ++i) grads.means[3 * k + i] = gmu[i];
@@ -596,14 +632,15 @@ __device__ __forceinline__ void project_bwd_body(gs_camera cam, const gs_config&
 }
 
 template <bool WANT_GRADS, bool WANT_POSE, bool WANT_SCORE>
-__global__ void __launch_bounds__(PB_THREADS) k_project_bwd(gs_camera cam, gs_config cfg,
+__global__ void __launch_bounds__(PB_THREADS, PB_CTAS) k_project_bwd(gs_camera cam, gs_config cfg,
                                                             gs_gaussians g, const float* __restrict__ grad2d,
                                                             gs_grads grads, float* __restrict__ score,
                                                             float2* __restrict__ pose_part,
                                                             double* __restrict__ pose_out,
-                                                            unsigned int* __restrict__ ticket, gs_pose_step step) {
+                                                            unsigned int* __restrict__ ticket, gs_pose_step step,
+                                                            int per) {
     project_bwd_body<WANT_GRADS, WANT_POSE, WANT_SCORE>(cam, cfg, g, grad2d, grads, score, pose_part, pose_out,
-                                                        ticket, step, (int)blockIdx.x, (int)gridDim.x);
+                                                        ticket, step, (int)blockIdx.x, (int)gridDim.x, per);
 }
 
 // ---------------------------------------------------------------------------
@@ -626,7 +663,7 @@ struct WaveProjJob {
     float* grad2d;
 };
 
-__global__ void __launch_bounds__(256) k_wave_project_hist(const gs_config cfg,
+__global__ void __launch_bounds__(256, 6) k_wave_project_hist(const gs_config cfg,
                                                            const __grid_constant__ Wave<WaveProjJob> W) {
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WaveProjJob& J = W.job[j];
@@ -652,17 +689,18 @@ struct WavePbJob {
     double* pose_out;
     unsigned int* ticket;
     gs_pose_step step;
+    int per;  // Gaussians a thread
 };
 
 template <bool WANT_SCORE>
-__global__ void __launch_bounds__(PB_THREADS) k_wave_project_bwd(const gs_config cfg,
-                                                                 const __grid_constant__ Wave<WavePbJob> W) {
+__global__ void __launch_bounds__(PB_THREADS, PB_CTAS) k_wave_project_bwd(const gs_config cfg,
+                                                                          const __grid_constant__ Wave<WavePbJob> W) {
     const int j = wave_find(W.start, W.n, (int)blockIdx.x);
     const WavePbJob& J = W.job[j];
     const gs_grads none = {nullptr, nullptr, nullptr, nullptr, nullptr};
     project_bwd_body<false, true, WANT_SCORE>(J.cam, cfg, J.g, J.grad2d, none, J.score, J.part, J.pose_out,
                                               J.ticket, J.step, (int)blockIdx.x - W.start[j],
-                                              W.start[j + 1] - W.start[j]);
+                                              W.start[j + 1] - W.start[j], J.per);
 }
 
 // Launches k_project_hist (nb CTAs of `per` Gaussians; ntiles words of
@@ -733,7 +771,7 @@ extern "C" gs_status gs_project(const gs_config* cfg, const gs_camera* cam, cons
 }
 
 size_t gs_project_bwd_ws(int64_t n) {
-    const size_t nblk = (size_t)pb_blocks(n, PB_PER);
+    const size_t nblk = (size_t)pb_blocks(n, PB_PER);  // at least the launch's blocks
     return ((nblk * 6 * sizeof(double)) + 255 + 256) & ~(size_t)255;  // partials + ticket
 }
 
@@ -779,14 +817,15 @@ extern "C" gs_status gs_project_bwd_step(const gs_config* cfg, const gs_camera* 
     }
     if (!grad2d) return set_error(GS_ERR_INVALID_ARG, "grad2d is NULL");
     gs_grads gg = grads ? *grads : gs_grads{nullptr, nullptr, nullptr, nullptr, nullptr};
-    const unsigned nblk = (unsigned)pb_blocks(g->n, want_pose ? PB_PER : 1);
+    const int per = want_pose ? pb_per(g->n) : 1;
+    const unsigned nblk = (unsigned)pb_blocks(g->n, per);
     float2* part = (float2*)workspace;
     unsigned int* ticket = (unsigned int*)((char*)workspace + need - 256);
     if (want_pose && cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st) != cudaSuccess)
         return set_error(GS_ERR_CUDA, "memset ticket");
 #define GS_PB_LAUNCH(A, B, C_) \
     k_project_bwd<A, B, C_><<<nblk, PB_THREADS, 0, st>>>(*cam, *cfg, *g, grad2d, gg, score_terms, part, pose_grad6, \
-                                                         ticket, ps)
+                                                         ticket, ps, per)
     if (want_grads) {
         if (want_pose) { if (want_score) GS_PB_LAUNCH(true, true, true); else GS_PB_LAUNCH(true, true, false); }
         else { if (want_score) GS_PB_LAUNCH(true, false, true); else GS_PB_LAUNCH(true, false, false); }
@@ -863,7 +902,7 @@ extern "C" gs_status gs_project_bwd_noalloc(const gs_config* cfg, const gs_camer
 // ---------------------------------------------------------------------------
 namespace gs {
 template <bool WANT_SCORE>
-__global__ void __launch_bounds__(PB_THREADS) k_project_bwd_adam(gs_camera cam, gs_config cfg, gs_gaussians g,
+__global__ void __launch_bounds__(PB_THREADS, PB_CTAS) k_project_bwd_adam(gs_camera cam, gs_config cfg, gs_gaussians g,
                                                                  const float* __restrict__ grad2d, gs_grads grads,
                                                                  float* __restrict__ score, AdamMap A,
                                                                  float* __restrict__ state) {
@@ -872,7 +911,7 @@ __global__ void __launch_bounds__(PB_THREADS) k_project_bwd_adam(gs_camera cam, 
     A.s = adam_step(A.lr, A.b1, A.b2, step);
     const gs_pose_step none = {nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 0.f};
     project_bwd_body<true, false, WANT_SCORE, true>(cam, cfg, g, grad2d, grads, score, nullptr, nullptr, nullptr,
-                                                    none, (int)blockIdx.x, (int)gridDim.x, &A);
+                                                    none, (int)blockIdx.x, (int)gridDim.x, 1, &A);
     __shared__ bool last;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -963,9 +1002,10 @@ gs_status wave_project_bwd(const gs_config& cfg, const gs_track_job* jobs, int n
     for (int j = 0; j < n; ++j) {
         const gs_track_job& t = jobs[j];
         W.start[j] = blocks;
-        blocks += (int)pb_blocks(t.g.n, PB_PER);
+        const int per = pb_per(t.g.n);
+        blocks += (int)pb_blocks(t.g.n, per);
         W.job[j] = WavePbJob{t.cam, t.g, t.grad2d, t.score_terms, (float2*)t.bwd_workspace, t.pose_grad6,
-                             wave_bwd_ticket(t), t.step};
+                             wave_bwd_ticket(t), t.step, per};
     }
     W.start[n] = blocks;
     if (score) {  // (gs_track_wave checked that every job has one)
