@@ -102,7 +102,8 @@ __device__ __forceinline__ SelState sel_advance(const SelArgs& A) {
     if (p == 0) return S;
     if (p > 1) S = A.state[p - 1];
     if (S.status == SEL_OPEN) {
-        const uint4 h = reinterpret_cast<const uint4*>(A.hist + (size_t)(p - 1) * SEL_BINS)[threadIdx.x];
+        const unsigned int* hp = A.hist + (size_t)(p - 1) * SEL_BINS + 4 * threadIdx.x;
+        const uint4 h = make_uint4(hp[0], hp[1], hp[2], hp[3]);  // (a workspace may be 8-byte aligned)
         const u64 mine = (u64)h.x + h.y + h.z + h.w;
         u64 x = mine;
         for (int o = 1; o < 32; o <<= 1) {
