@@ -204,7 +204,8 @@ gs_status gs_project(const gs_config* cfg, const gs_camera* cam, const gs_gaussi
  * blend is in its tile's list; lists hold about 20 % fewer keys than with
  * the integer box alone.
  * Implementation: a counting scatter on the tile id (per-CTA tile rows and a
- * column scan) and a merge sort of each tile's (depth, id) bucket.
+ * column scan) and a distribution sort by depth of each tile's (depth, id)
+ * bucket (a merge sort where depths crowd).
  * keys_out [keys_capacity] u64, vals_out [keys_capacity] u32,
  * n_keys_out: one device int64 receiving the true key count, tile_ranges
  * [2*TX*TY] u32.  If the count exceeds keys_capacity, only keys_capacity keys

@@ -420,7 +420,8 @@ __device__ __forceinline__ void add_loss(const FwdOut& O, float part) {
 // of four words in every lane, scalar geometry and steps of three entries
 // padded with dummies took 74 instructions a (warp, entry) visit, 65.9 M for
 // the tracking frame, against 43.3 M now.  Forward + loss 640x480 / 200k 84 ->
-// 61.4 us, forward 1200x680 / 1M 180 -> 100, 1296x968 / 750k bf16 232 -> 144.  Measured and not kept: records by cp.async a batch ahead (raw records
+// 61.4 us, forward 1200x680 / 1M 180 -> 100, 1296x968 / 750k bf16 232 -> 144.
+// Measured and not kept: records by cp.async a batch ahead (raw records
 // in shared memory cost each warp their unpacking: 61.4 / 105.8 / 152.7), the
 // next batch staged beside the compositing (60.9 / 112 / 157), two entries a
 // step (68.9 / 102 / 146).
