@@ -103,16 +103,6 @@ __device__ __forceinline__ void group_sync(const Group& G) {
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + G.gi), "r"(G.TT) : "memory");
 }
 
-// Number of threads of the group with `pred` set (also a group barrier).
-__device__ __forceinline__ int group_count(const Group& G, bool pred) {
-    if (G.TT == R_THREADS) return __syncthreads_count(pred);
-    if (G.TT == 32) return __popc(__ballot_sync(0xffffffffu, pred));
-    int r;
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %3, 0; bar.red.popc.u32 %0, %1, %2, p; }"
-                 : "=r"(r) : "r"(1 + G.gi), "r"(G.TT), "r"((unsigned)pred) : "memory");
-    return r;
-}
-
 __device__ __forceinline__ PixelMap map_pixel(const Grid& g, int tile, int lt) {
     PixelMap m;
     const int tx = tile % g.TX, ty = tile / g.TX;
@@ -221,7 +211,6 @@ __device__ __forceinline__ x2f x2_fma(x2f a, x2f b, x2f c) {  // a b + c
 
 __device__ __forceinline__ x2f x2_dup(float v) { return x2_pack(v, v); }
 
-__device__ __forceinline__ x2f x2_ld(const float* p) { return *reinterpret_cast<const x2f*>(p); }
 __device__ __forceinline__ void x2_ld2(const float4* p, x2f& lo, x2f& hi) {  // one 16-byte load: two packed pairs
     const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
     lo = v.x;
