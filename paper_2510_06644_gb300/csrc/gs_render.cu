@@ -25,15 +25,13 @@
 // one-warp CTA: it visits the entries one of its pixels blended, takes each
 // lane's decision from the lane's own mask bit, walks the fragments in
 // reverse recovering T_k by division (Eq. 5), and sums the per-pixel terms
-// of each Gaussian over the warp on the tensor cores, four entries at a
+// of each Gaussian over the warp through shared memory, four entries at a
 // time, before one global atomic per (Gaussian, warp, field).  Without masks
 // a CTA per tile stages the list, visits the entries whose pixel box meets
 // each warp's block, merges the per-pixel gradients with a reduce-scatter
 // butterfly (each level halves the fields a lane carries) and sums the warps
 // in shared memory first.  This replaces the paper's Gradient
 // Merging Unit (Sec. 5.3).
-#include <stddef.h>
-
 #include <algorithm>
 #include <type_traits>
 
@@ -192,6 +190,11 @@ __device__ __forceinline__ x2f x2_pack(float lo, float hi) {
 }
 __device__ __forceinline__ void x2_unpack(x2f v, float& lo, float& hi) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ x2f x2_add(x2f a, x2f b) {
+    x2f r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 __device__ __forceinline__ x2f x2_sub(x2f a, x2f b) {
     x2f r;
@@ -983,8 +986,9 @@ __global__ void __launch_bounds__(R_THREADS, KST == 1 ? (MODE == GS_TRACK ? 4 : 
 
 // The masked backward's working set of one warp: a ring of 64 staged entries
 // (slot s: pair s / 2, half s & 1, so that two consecutive slots load as
-// packed pairs, two fields per 16-byte load) and the (h, w) columns of the
-// step being merged, one row of 32 pixels each.
+// packed pairs, two fields per 16-byte load) and what the lanes hand over to
+// be summed in a step of two pairs.
+#define PW_TERMS 6  // per pair: a h, b h, u dx, u dy, v dy, and w gD (pose only) or the opacity's (mapping)
 struct __align__(16) PwRing {
     float4 xy[32];     // x0 x1 y0 y1
     float4 ab[32];     // conic a, b
@@ -993,9 +997,16 @@ struct __align__(16) PwRing {
     float4 gb[32];     // green, blue
     uint32_t id[64];
     uint32_t pm[64];   // pixels that blended the entry
-    float op[64];      // opacity (mapping)
-    float col[8][36];  // h0 w0 h1 w1 h2 w2 h3 w3 over the pixels (36: the rows start in different banks)
+    // [half of the block's pixels][pair, term][pixel]: the terms of the pair's
+    // two entries (18: eight rows' 16-byte words lie in different banks)
+    x2f term[2][2 * PW_TERMS][18];
 };
+struct __align__(16) PwRingMap : PwRing {
+    float op[64];      // opacity
+    float w[4][36];    // w = T alpha of the step's entries over the pixels (36: as above)
+};
+template <int MODE>
+using PwShared = typename std::conditional<MODE == GS_MAP, PwRingMap, PwRing>::type;
 
 // 32 x 32 bit transpose over the warp: bit p of lane e's result is bit e of
 // lane p's word (five butterfly exchanges; at distance s the partners swap
@@ -1015,42 +1026,16 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x) {
     return x;
 }
 
-// d += a b on the tensor cores: a 16 x 8 (row i, column k), b 8 x 8 in tf32,
-// accumulated in float32.  Lane 4 r + c holds a(r, c), a(r + 8, c),
-// a(r, c + 4), a(r + 8, c + 4); b(c, r), b(c + 4, r); d(r, 2 c), d(r, 2 c + 1),
-// d(r + 8, 2 c), d(r + 8, 2 c + 1).
-// FIRST: d = a b.
-template <bool FIRST>
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    if (FIRST)
-        asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-            "{%10, %10, %10, %10};"
-            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
-    else
-        asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-            "{%0, %1, %2, %3};"
-            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-            : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// v = hi + lo with hi the nearest float of 11 significand bits (a tf32 value;
-// ties away from zero) and lo the exact rest, of which the tensor cores use
-// the first 11 bits: 23 of v's 24 bits in the worst case.
-__device__ __forceinline__ void tf32_split(float v, uint32_t& hi, uint32_t& lo) {
-    hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
-    lo = __float_as_uint(v - __uint_as_float(hi));
-}
-
 // Two consecutive fragments of a warp's ring, back to front (slot s first):
-// the geometry of both in packed pairs with the forward's arithmetic in every
-// half (the same alpha), the transmittance and suffix recursions (Eq. 5)
-// fragment by fragment.  c0, c1: whether the forward blended them into this
-// pixel; a fragment that was not keeps the state (alpha 0: T / 1, s + 0).
-// Returns per fragment w = T alpha and h = alpha dL/dalpha = w (c . g - s),
-// the gradient of the exponent (0 where alpha was clamped).
-__device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pair, bool c0, bool c1, x2f PXC, x2f PYC,
-                                          float alpha_max, float& h0, float& w0, float& h1, float& w1) {
+// the geometry and the gradient products of both in packed pairs with the
+// forward's arithmetic in every half (the same alpha), the transmittance and
+// suffix recursions (Eq. 5) fragment by fragment as in back_frag.  c0, c1:
+// whether the forward blended them into this pixel; a fragment that was not
+// keeps the state (alpha 0: T / 1, s + 0) and adds zeros.  Writes the pair's
+// terms, term k to term[18 k], and when mapping w to wcol[0] and wcol[36].
+template <int MODE>
+__device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pair, bool c0, bool c1, x2f PXC,
+                                          x2f PYC, float alpha_max, x2f* term, float* wcol) {
     x2f X, Y, CA, CB, CC, LOP, DEP, CR, CG, CL;
     x2_ld2(R.xy + pair, X, Y);
     x2_ld2(R.ab + pair, CA, CB);
@@ -1071,16 +1056,29 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
     // T / (1 - alpha) by the reciprocal instruction (at most 1 ulp) and a
     // product, as the fast division of back_frag
     S.T *= rcp_sfu(1.f - al0);
-    w0 = al0 * S.T;
+    const float w0 = al0 * S.T;
     const float dif0 = c0 ? cg0 - S.sg : 0.f;
     S.sg = __fmaf_rn(al0, dif0, S.sg);
     S.T *= rcp_sfu(1.f - al1);
-    w1 = al1 * S.T;
+    const float w1 = al1 * S.T;
     const float dif1 = c1 ? cg1 - S.sg : 0.f;
     S.sg = __fmaf_rn(al1, dif1, S.sg);
     // the clamp passes no gradient to opacity or shape
-    h0 = raw0 > alpha_max ? 0.f : w0 * dif0;
-    h1 = raw1 > alpha_max ? 0.f : w1 * dif1;
+    const bool cl0 = raw0 > alpha_max, cl1 = raw1 > alpha_max;
+    const x2f H = x2_mul(x2_pack(cl0 ? 0.f : -0.5f * w0, cl1 ? 0.f : -0.5f * w1), x2_pack(dif0, dif1));
+    const x2f U = x2_mul(H, DX), V = x2_mul(H, DY);
+    term[0] = x2_mul(A, H);
+    term[18] = x2_mul(B, H);
+    term[36] = x2_mul(U, DX);
+    term[54] = x2_mul(U, DY);
+    term[72] = x2_mul(V, DY);
+    if (MODE == GS_MAP) {
+        term[90] = x2_mul(x2_dup(-2.f), H);  // alpha dL/dalpha
+        wcol[0] = w0;
+        wcol[36] = w1;
+    } else {
+        term[90] = x2_mul(x2_pack(w0, w1), x2_dup(S.gD));
+    }
 }
 
 // Backward compositing of one warp's block of a tile from the forward's
@@ -1101,23 +1099,23 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 // construction, and the alpha it recomputes is the forward's (same staged
 // values, same arithmetic).
 //
-// The sums over the pixels are a contraction on the tensor cores.  With h and
-// w as in back_pair and pixel p at lattice offset (u, v) from the block's
-// centre (u, v half-integers up to 7.5, so 1, u, v, u u, u v, v v are exact in
-// tf32), every gradient of an entry is a combination of the moments
-// sum_p h {1, u, v, u u, u v, v v} and of sum_p w g, g the pixel's image
-// gradient (depth and colour): rows 0-5 of the left matrix hold the moments'
-// factors, rows 8-11 g's leading tf32 part and rows 12-15 its remainder, and
-// the right matrix holds four entries' (h, w) columns, split into tf32 pairs
-// (tf32_split; the products of two such parts are exact in the float32
-// accumulator).  Against 64-bit sums the split is as close as the float32
-// butterfly it replaced.  That butterfly took 94 instructions for four
-// entries' 24 pose-only fields (82 for two entries' 20 mapping fields) and
-// 13 per entry to form them; the columns, splits, 8 tensor instructions and
-// the moments' recombination take about 85 for four entries in either mode.
+// The sums over the pixels go through shared memory: a lane writes each of
+// its terms of a pair of entries as one 8-byte word, and a lane a (term, half
+// of the block) adds that half's 16 words in packed float32 pairs, as a tree;
+// the two halves then exchange an entry's partial sum each.  When mapping,
+// the depth and colour sums are products of the entries' weights w with the
+// pixels' image gradients: a lane a (channel, entry, half of the block) keeps
+// its channel's 16 gradients in registers and reads w.
 //
-// The recombined gradients go straight to grad2d, one atomic per (entry,
-// field, warp): the warps of a tile share nothing and run as one-warp CTAs
+// Every term is formed about the Gaussian's own mean and added in float32, as
+// in the kernels without masks.  Moments of h over the block, moved to the
+// mean after the sum, need fewer values but lose digits: second moments about
+// the block's centre (block / Gaussian)^2 of them (a Gaussian of 0.55 px: 1.6e-6
+// relative at stride 1, 2e-5 at 4x4, against 1e-7), and Q sum h d in place
+// of sum (Q d) h is three times as far from 64 bits on a needle.
+//
+// They go straight to grad2d, one atomic per (entry, field, warp): the warps
+// of a tile share nothing and run as one-warp CTAs
 // that the hardware schedules as they free up, heavy tiles first.
 template <int DT, int MODE>
 __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
@@ -1125,7 +1123,8 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
                                        const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
                                        const float* __restrict__ d_rgb, const float* __restrict__ d_depth,
                                        float* __restrict__ grad2d, const uint32_t* __restrict__ bmask, int tile,
-                                       int w, PwRing& R) {
+                                       int w, PwShared<MODE>& R) {
+    constexpr int ROWS = 2 * PW_TERMS;
     const int lane = threadIdx.x & 31;
     const int lt = w * 32 + lane;
     const bool small = g.tw * g.th <= 64;
@@ -1157,111 +1156,84 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     uint32_t bm_nx = __ldg(bm + (size_t)r_top * rs);
     const float pxc = (float)m.px + 0.5f, pyc = (float)m.py + 0.5f;
     const x2f PXC = x2_dup(pxc), PYC = x2_dup(pyc);
-    // the left matrix: lane 4 j + c holds row j (moment j) and row j + 8
-    // (image gradient channel j & 3: leading part, j >= 4: remainder) at
-    // pixels 8 c + s and 8 c + 4 + s of step s
-    const int c = lane & 3, j = lane >> 2;
-    // the block's width in pixels: the lanes run row by row through it
-    const int bw = small ? g.tw : (g.tw < 8 ? 4 : 8), lbw = bw == 16 ? 4 : bw == 8 ? 3 : 2;
-    const float sx = (float)g.sx, sy = (float)g.sy;
-    const float X0 = __shfl_sync(0xffffffffu, pxc, 0) + 0.5f * (float)(bw - 1) * sx;  // the block's centre
-    const float Y0 = __shfl_sync(0xffffffffu, pyc, 0) + 0.5f * (float)(32 / bw - 1) * sy;
-    uint32_t am[4][4];
-    R.col[0][lane] = S.gD;
-    R.col[1][lane] = MODE == GS_MAP ? S.gC0 : 0.f;
-    R.col[2][lane] = MODE == GS_MAP ? S.gC1 : 0.f;
-    R.col[3][lane] = MODE == GS_MAP ? S.gC2 : 0.f;
-    __syncwarp();
+    // where the lane writes its terms, and the half row it sums: half, pair
+    // and term; after the halves' exchange entry `ent` of the step
+    x2f* const mine_t = &R.term[lane >> 4][0][lane & 15];
+    const bool sums = lane < 2 * ROWS;
+    const int half = lane >= ROWS ? 1 : 0, row = lane - half * ROWS, term = row % PW_TERMS;
+    const int ent = 2 * (row / PW_TERMS) + half, partner = half ? row : row + ROWS;
+    const int col = MODE == GS_MAP ? term : field_col<MODE>(term);
+    const float scale = field_scale(term);
+    // mapping: the lane's entry, half and channel (depth, red, green, blue) of
+    // the weighted sums, and that channel's image gradients
+    const int we = lane & 3, wh = (lane >> 2) & 1, wc = lane >> 3;
+    float gw[16];
+    if constexpr (MODE == GS_MAP) {
+        R.w[0][lane] = S.gD;
+        R.w[1][lane] = S.gC0;
+        R.w[2][lane] = S.gC1;
+        R.w[3][lane] = S.gC2;
+        __syncwarp();
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int q = 8 * c + 4 * b + s;
-            const float u = (float)(q & (bw - 1)) - 0.5f * (float)(bw - 1);
-            const float v = (float)(q >> lbw) - 0.5f * (float)(32 / bw - 1);
-            const float f1 = j == 0 ? 1.f : (j == 1 || j == 3 || j == 4) ? u : j < 6 ? v : 0.f;
-            const float f2 = j == 3 ? u : (j == 4 || j == 5) ? v : 1.f;
-            uint32_t hi, lo;
-            tf32_split(R.col[j & 3][q], hi, lo);
-            am[s][2 * b] = __float_as_uint(f1 * f2);
-            am[s][2 * b + 1] = j < 4 ? hi : lo;
-        }
-    __syncwarp();
-    // recombination (see the step): the factor of the lane's own moment
-    const float own_f = j == 3 ? -0.5f * sx * sx : j == 4 ? -sx * sy : j == 5 ? -0.5f * sy * sy : 0.f;
-    // its two coefficients: k1 = ca, cb, -ox / 2, -oy, -oy / 2 and k2 = cb, cc,
-    // 0, -ox, 0 for j = 1..5, (ox, oy) = (X0, Y0) - (x, y)
-    constexpr int AB = offsetof(PwRing, ab) / 4, CL = offsetof(PwRing, cl) / 4;
-    const int slot_off = (c >> 1) * 4 + (c & 1);
-    const int k1o = j == 1 ? AB : j == 2 ? AB + 2 : j == 3 ? 0 : 2;
-    const int k2o = j == 1 ? AB + 2 : j == 2 ? CL : 0;
-    const float k1s = j == 3 || j == 5 ? 0.5f : 1.f, k2s = j == 1 || j == 2 || j == 4 ? 1.f : 0.f;
-    const float k1c = j == 3 ? -0.5f * X0 : j == 4 ? -Y0 : j == 5 ? -0.5f * Y0 : 0.f;
-    const float k2c = j == 4 ? -X0 : 0.f;
-    const float v1f = j == 3 || j == 5 ? 1.f : 0.f;
+        for (int k = 0; k < 16; ++k) gw[k] = R.w[wc][16 * wh + k];
+        __syncwarp();
+    }
 
     // One step: slots g0 .. g0 + 3 of the ring (g0 a multiple of 4), the
     // first nv of them entries.
     auto step = [&](int g0, int nv) {
         const uint4 pm = *reinterpret_cast<const uint4*>(R.pm + g0);
         const uint32_t bit = 1u << lane;
-        float h[4], wt[4];
-        back_pair(S, R, g0 >> 1, (pm.x & bit) != 0u, (pm.y & bit) != 0u, PXC, PYC, cfg.alpha_max, h[0], wt[0], h[1],
-                  wt[1]);
-        back_pair(S, R, (g0 >> 1) + 1, (pm.z & bit) != 0u, (pm.w & bit) != 0u, PXC, PYC, cfg.alpha_max, h[2], wt[2],
-                  h[3], wt[3]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {  // (after all of the step's loads)
-            R.col[2 * e][lane] = h[e];
-            R.col[2 * e + 1][lane] = wt[e];
-        }
+        float* wcol = nullptr;
+        if constexpr (MODE == GS_MAP) wcol = &R.w[0][lane];
+        back_pair<MODE>(S, R, g0 >> 1, (pm.x & bit) != 0u, (pm.y & bit) != 0u, PXC, PYC, cfg.alpha_max, mine_t, wcol);
+        back_pair<MODE>(S, R, (g0 >> 1) + 1, (pm.z & bit) != 0u, (pm.w & bit) != 0u, PXC, PYC, cfg.alpha_max,
+                        mine_t + 18 * PW_TERMS, wcol + (MODE == GS_MAP ? 72 : 0));
         __syncwarp();
-        const float4 va = *reinterpret_cast<const float4*>(&R.col[j][8 * c]);
-        const float4 vb = *reinterpret_cast<const float4*>(&R.col[j][8 * c + 4]);
-        __syncwarp();  // the next step reuses the columns
-        float d[4], dl[4];  // two chains of 4 instead of one of 8
-        const float fa[4] = {va.x, va.y, va.z, va.w}, fb[4] = {vb.x, vb.y, vb.z, vb.w};
+        float own = 0.f, other = 0.f;  // this half's sums of the entry kept and of the partner's
+        if (sums) {
+            const ulonglong2* t = reinterpret_cast<const ulonglong2*>(&R.term[0][0][0] + 18 * lane);
+            x2f a[8];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            uint32_t ah, al, bh, bl;
-            tf32_split(fa[s], ah, al);
-            tf32_split(fb[s], bh, bl);
-            if (s == 0) {
-                mma_tf32<true>(d, am[s], ah, bh);
-                mma_tf32<true>(dl, am[s], al, bl);
-            } else {
-                mma_tf32<false>(d, am[s], ah, bh);
-                mma_tf32<false>(dl, am[s], al, bl);
+            for (int i = 0; i < 8; ++i) {
+                const ulonglong2 v = t[i];
+                a[i] = x2_add(v.x, v.y);
             }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < o; ++i) a[i] = x2_add(a[i], a[i + o]);
+            float lo, hi;
+            x2_unpack(a[0], lo, hi);
+            own = half ? hi : lo;
+            other = half ? lo : hi;
         }
-        // lane 4 j + e (e = c): moment j of entry e's h, and sum w g of
-        // channel j & 3 (its two parts on lanes 16 apart)
-        const float mo = d[0] + dl[0];
-        float wg = d[3] + dl[3];
-        wg += __shfl_xor_sync(0xffffffffu, wg, 16);
-        const float M1 = __shfl_sync(0xffffffffu, mo, c);
-        const float MX = sx * __shfl_sync(0xffffffffu, mo, 4 + c);
-        const float MY = sy * __shfl_sync(0xffffffffu, mo, 8 + c);
-        // sums of h dx and h dy about the Gaussian's mean, (dx, dy) = (ox +
-        // sx u, oy + sy v), and the lane's field k1 v1 + k2 v2 + own_f mo:
-        // j = 1, 2 dL/dmean = Q sum h d; j = 3..5 dL/dconic = -(1/2, 1, 1/2)
-        // sum h (dx dx, dx dy, dy dy), with sum h dx dx = sx^2 m_uu + ox (MX +
-        // SX) and likewise; j = 0 dL/ddepth (pose only) or dL/dopacity
-        // (mapping).  k1 and k2 are one staged field each, scaled and shifted.
-        const int slot = g0 + c;
-        const float* fld = reinterpret_cast<const float*>(R.xy + (g0 >> 1)) + slot_off;
-        const float SX = __fmaf_rn(X0 - fld[0], M1, MX), SY = __fmaf_rn(Y0 - fld[2], M1, MY);
-        const float k1 = __fmaf_rn(k1s, fld[k1o], k1c), k2 = __fmaf_rn(k2s, fld[k2o], k2c);
-        const float v1 = __fmaf_rn(v1f, j == 5 ? MY : MX, j == 5 ? SY : SX);
-        const float v2 = j == 4 ? MY : SY;
-        float f = __fmaf_rn(k1, v1, __fmaf_rn(k2, v2, own_f * mo));
-        if (MODE == GS_TRACK && j == 0) f = wg;
-        if (MODE == GS_MAP && j == 0) f = __fdividef(mo, R.op[slot]);  // alpha = opacity e^(-q/2)
-        if (c < nv) {
-            float* dst = grad2d + (size_t)R.id[slot] * GS_GRAD2D_STRIDE;
-            // columns: du dv dA dB dC dop dd . dr dg db
-            if (j < 6 && f != 0.f) atomicAdd(dst + (j == 0 ? (MODE == GS_MAP ? 5 : 6) : j - 1), f);
-            if (MODE == GS_MAP && j < 4 && wg != 0.f) atomicAdd(dst + (j == 0 ? 6 : j + 7), wg);
+        float wg = 0.f;
+        if constexpr (MODE == GS_MAP) {
+            const float4* t = reinterpret_cast<const float4*>(&R.w[we][16 * wh]);
+            float a[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 v = t[i];
+                a[0] = i ? __fmaf_rn(v.x, gw[4 * i], a[0]) : v.x * gw[0];
+                a[1] = i ? __fmaf_rn(v.y, gw[4 * i + 1], a[1]) : v.y * gw[1];
+                a[2] = i ? __fmaf_rn(v.z, gw[4 * i + 2], a[2]) : v.z * gw[2];
+                a[3] = i ? __fmaf_rn(v.w, gw[4 * i + 3], a[3]) : v.w * gw[3];
+            }
+            wg = (a[0] + a[1]) + (a[2] + a[3]);
+        }
+        __syncwarp();  // the next step reuses the words
+        float f = own + __shfl_sync(0xffffffffu, other, partner & 31);
+        if (sums && ent < nv) {
+            const int slot = g0 + ent;
+            if constexpr (MODE == GS_MAP)
+                if (term == 5) f = __fdividef(f, R.op[slot]);  // alpha = opacity e^(-q/2)
+            if (f != 0.f) atomicAdd(grad2d + (size_t)R.id[slot] * GS_GRAD2D_STRIDE + col, f * scale);
+        }
+        if constexpr (MODE == GS_MAP) {
+            wg += __shfl_xor_sync(0xffffffffu, wg, 4);
+            if (wh == 0 && we < nv && wg != 0.f)
+                atomicAdd(grad2d + (size_t)R.id[g0 + we] * GS_GRAD2D_STRIDE + (wc == 0 ? 6 : wc + 7), wg);
         }
     };
 
@@ -1303,12 +1275,12 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
             gb[2] = v.b;
             R.id[slot] = id;
             R.pm[slot] = pix;
-            if (MODE == GS_MAP) R.op[slot] = v.op;
+            if constexpr (MODE == GS_MAP) R.op[slot] = v.op;
         }
         tail += __popc(mw);
         __syncwarp();
-        // at most 3 entries stay behind, so the next run's 32 find room; the
-        // slots it overwrites were read before the last step's barriers
+        // at most 3 entries stay behind, so the next run's 32 find room beside
+        // them and the four stepped over last, whose fields lanes may still read
 #pragma unroll 1
         for (; tail - head >= 4; head += 4) step(head & 63, 4);
     }
@@ -1319,10 +1291,11 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     }
 }
 
-// One-warp CTAs of the masked backward per SM: 24 at 80 registers (tracking
-// 640x480 / 200k: 71.7 us, mapping 1200x680 / 1M: 153 us; 32 at 64 registers
-// spill: 88 and 164 us; 28: 75 and 159; 20: 71.9 and 161).  The float32
-// butterfly kernel it replaced took 87 and 210 us.
+// One-warp CTAs of the masked backward per SM: 24 (78 registers).  us of the
+// kernel, tracking 640x480 / 200k, 1200x680 / 458k at 2x2, mapping 1200x680 /
+// 1M and 1920x1080 / 1M f16: 20 a SM 69, 63, 239 and 491; 24 69, 65, 229 and
+// 464; 28 72, 67, 228 and 460.  (One float32 butterfly per two to four entries
+// instead of the sums through shared memory: 85, 79, 260 and 535.)
 #define PW_CTAS 24
 
 // Warps per tile of the masked backward.
@@ -1335,7 +1308,7 @@ __global__ void __launch_bounds__(32, PW_CTAS)
                     const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
                     const float* __restrict__ d_rgb, const float* __restrict__ d_depth, float* __restrict__ grad2d,
                     const uint32_t* __restrict__ bmask) {
-    __shared__ PwRing R;
+    __shared__ PwShared<MODE> R;
     const int wpt = pw_warps(g);
     const int t = (int)blockIdx.x / wpt, w = (int)blockIdx.x % wpt;
     const int tile = order ? (int)__ldg(order + t) : t;
