@@ -1002,7 +1002,6 @@ struct __align__(16) PwRing {
     x2f term[2][2 * PW_TERMS][18];
 };
 struct __align__(16) PwRingMap : PwRing {
-    float op[64];      // opacity
     float w[4][36];    // w = T alpha of the step's entries over the pixels (36: as above)
 };
 template <int MODE>
@@ -1055,12 +1054,12 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
     const float al0 = c0 ? fminf(alpha_max, raw0) : 0.f, al1 = c1 ? fminf(alpha_max, raw1) : 0.f;
     // T / (1 - alpha) by the reciprocal instruction (at most 1 ulp) and a
     // product, as the fast division of back_frag
-    S.T *= rcp_sfu(1.f - al0);
-    const float w0 = al0 * S.T;
+    const float T0 = S.T *= rcp_sfu(1.f - al0);
+    const float w0 = al0 * T0;
     const float dif0 = c0 ? cg0 - S.sg : 0.f;
     S.sg = __fmaf_rn(al0, dif0, S.sg);
-    S.T *= rcp_sfu(1.f - al1);
-    const float w1 = al1 * S.T;
+    const float T1 = S.T *= rcp_sfu(1.f - al1);
+    const float w1 = al1 * T1;
     const float dif1 = c1 ? cg1 - S.sg : 0.f;
     S.sg = __fmaf_rn(al1, dif1, S.sg);
     // the clamp passes no gradient to opacity or shape
@@ -1073,7 +1072,10 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
     term[54] = x2_mul(U, DY);
     term[72] = x2_mul(V, DY);
     if (MODE == GS_MAP) {
-        term[90] = x2_mul(x2_dup(-2.f), H);  // alpha dL/dalpha
+        // dalpha/dopacity = e^(-q/2): not alpha / opacity, which an opacity
+        // that rounds to 0 (blended where alpha_min is 0) does not have
+        x2_unpack(x2_mul(Q, x2_dup(R_NEG_HALF_LOG2E)), e0, e1);
+        term[90] = x2_pack(c0 && !cl0 ? exp2_sfu(e0) * (T0 * dif0) : 0.f, c1 && !cl1 ? exp2_sfu(e1) * (T1 * dif1) : 0.f);
         wcol[0] = w0;
         wcol[36] = w1;
     } else {
@@ -1224,12 +1226,8 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
         }
         __syncwarp();  // the next step reuses the words
         float f = own + __shfl_sync(0xffffffffu, other, partner & 31);
-        if (sums && ent < nv) {
-            const int slot = g0 + ent;
-            if constexpr (MODE == GS_MAP)
-                if (term == 5) f = __fdividef(f, R.op[slot]);  // alpha = opacity e^(-q/2)
-            if (f != 0.f) atomicAdd(grad2d + (size_t)R.id[slot] * GS_GRAD2D_STRIDE + col, f * scale);
-        }
+        if (sums && ent < nv && f != 0.f)
+            atomicAdd(grad2d + (size_t)R.id[g0 + ent] * GS_GRAD2D_STRIDE + col, f * scale);
         if constexpr (MODE == GS_MAP) {
             wg += __shfl_xor_sync(0xffffffffu, wg, 4);
             if (wh == 0 && we < nv && wg != 0.f)
@@ -1275,7 +1273,6 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
             gb[2] = v.b;
             R.id[slot] = id;
             R.pm[slot] = pix;
-            if constexpr (MODE == GS_MAP) R.op[slot] = v.op;
         }
         tail += __popc(mw);
         __syncwarp();
