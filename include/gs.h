@@ -510,7 +510,10 @@ typedef struct {
 #define GS_WAVE_MAX 32
 
 /* One tracking iteration of every job (Sec. 2.1 Steps 1-3, Sec. 2.2 Steps
- * 4-5, Sec. 4.1 Eq. 6), each with the results of its own fused iteration,
+ * 4-5, Sec. 4.1 Eq. 6), each with the results of its own fused iteration --
+ * the lists and the forward bit for bit, the backward to float32 rounding
+ * (it adds with float atomics, and in strided frames the tiles of the whole
+ * wave decide between two kernels that form the same terms) --
  * in launches whose grids span all jobs: projection with the binning's tile
  * counts, the column scan with the tile scan and order, the key scatter, the
  * bucket sort, the forward compositing with the loss, the backward

@@ -2190,8 +2190,11 @@ gs_status wave_render(const gs_config& cfg, const gs_track_job* jobs, int n, cud
     }
     // backward compositing, pose-only fields: one launch per kernel form
     // present (0, 1: without masks, one or several tiles a CTA; 2, 3:
-    // entry-parallel tiles of up to 32 or 64 pixels; 4: one-warp CTAs)
-    // (the one-warp CTAs of all jobs with masks share a launch and so its tail)
+    // entry-parallel tiles of up to 32 or 64 pixels; 4: one-warp CTAs).  The
+    // masked sessions' tiles together decide between the last three (they
+    // share a launch and so its tail: six sessions 682 us, 740 in three
+    // launches by each session's own tiles); both kernels form the same float32
+    // terms, so a session's gradients move by their rounding alone.
     int masked = 0;
     for (int j = 0; j < n; ++j) {
         const Grid g = make_grid(jobs[j].cam);
