@@ -390,26 +390,46 @@ __global__ void __launch_bounds__(1024) k_col_scan_tail(uint32_t* __restrict__ h
 
 // k_tile_scatter_rows with the rects the fused projection kept (no
 // geometry re-read, no tile-rect arithmetic): only the depth is loaded.
-// Block 0 computes the heavy-first order beside the scatter.  The others
-// cover `nrow` groups of per_cta Gaussians for each of the bands of `band`
-// tile rows, one band after the other: the keys' 8-byte writes land all over
-// their band's buckets, so a band is what L2 holds at once (written as one
-// region of 188 MB, the 23.4 M keys of 1920x1080 / 3M took 582 us, 340 MB of
-// it reads of partly written lines).
+// Block 0 computes the heavy-first order beside the scatter.  The others take
+// groups of per_cta Gaussians through the bands of tile rows, one band after
+// the other: the keys' 8-byte writes land all over their band's buckets, so a
+// band is what L2 holds at once (written as one region of 188 MB, the 23.4 M
+// keys of 1920x1080 / 3M took 582 us, 340 MB of it reads of partly written
+// lines).
 struct ScatterArgs {
     int TX;
     const void* splats;
     int64_t n, per_cta;
-    int nrow, ntiles, band;  // groups of Gaussians; tiles; tile rows per band
+    int nrow, ntiles;      // groups of Gaussians; tiles
+    int max_rows, stride;  // most tile rows of a band (the shared memory); a block's next band is `stride` on
     const uint32_t* start;
     const uint32_t* hist;
     const uint2* rects;
     int64_t cap;
     u64* keys;
+    const int64_t* n_keys;
     const uint32_t* ranges;
     uint32_t* order;
     uint32_t* n_big;
 };
+
+// Tile rows per band: one band for every SCATTER_BAND bytes of keys there
+// are, at most 6 (every band reads the rects again), and no more rows than
+// the shared memory holds.  Scatter times by number of bands: 1200x680 / 1M
+// (34 MB of keys) 1 band 55 us, 2 43.7, 4 47, 7 60; 1296x968 / 750k (32 MB) 49,
+// 2 40, 3 37, 6 44; 1200x680 / 458k at stride 2 (15 MB) 21.7, 2 19.6; 1920x1080 /
+// 3M (188 MB) 3 bands 307, 6 263, 12 277, 24 392.
+// From the count on the device, not from the capacity: with room for 16 M
+// keys, 1M Gaussians took 32 us at 320x240 (1.5 M keys; 6 bands) and 39 at
+// 640x480 (2.5 M); with the count's bands 16 and 24.
+#define SCATTER_BAND (13 << 20)
+#define SCATTER_SMEM_TILES 6144  // 24 KB
+
+__host__ __device__ inline int scatter_bands(int64_t keys, int TY) {
+    const int64_t want = (keys * (int64_t)sizeof(u64) + SCATTER_BAND - 1) / SCATTER_BAND;
+    const int most = TY < 6 ? TY : 6;
+    return want < 1 ? 1 : want < most ? (int)want : most;
+}
 
 template <int DT>
 __device__ __forceinline__ void scatter_rects_body(const ScatterArgs& A, int blk) {
@@ -418,31 +438,36 @@ __device__ __forceinline__ void scatter_rects_body(const ScatterArgs& A, int blk
         return;
     }
     extern __shared__ uint32_t h[];  // next free place of each of the band's tiles
-    const int grp = (blk - 1) % A.nrow, yb = (blk - 1) / A.nrow * A.band;
-    const int t0 = yb * A.TX, nt = min(A.ntiles - t0, A.band * A.TX);
-    const uint32_t* row = A.hist + (size_t)grp * A.ntiles + t0;
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) h[t] = A.start[t0 + t] + row[t];
-    __syncthreads();
+    const int TY = A.ntiles / A.TX, grp = (blk - 1) % A.nrow, band0 = (blk - 1) / A.nrow;
+    const int bands = scatter_bands(min(__ldcg(A.n_keys), A.cap), TY), rows = min((TY + bands - 1) / bands, A.max_rows);
     const int64_t k0 = (int64_t)grp * A.per_cta, k1 = min(A.n, k0 + A.per_cta);
-    for (int64_t kb = k0; kb < k1; kb += blockDim.x) {
-        const int64_t k = kb + threadIdx.x;
-        int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
-        float depth = 0.f;
-        if (k < k1) {
-            const uint2 r = __ldg(A.rects + k);
-            x0 = (int)(r.x & 0xffffu);
-            x1 = (int)(r.x >> 16);
-            y0 = max((int)(r.y & 0xffffu), yb);
-            y1 = max(min((int)(r.y >> 16), yb + A.band), y0);
-            if (x1 > x0 && y1 > y0)
-                depth = DT == GS_F32 ? __ldg(reinterpret_cast<const float*>(A.splats) + 12 * (size_t)k + 6)
-                                     : __ldg(reinterpret_cast<const float*>(A.splats) + 8 * (size_t)k + 2);
+    for (int yb = band0 * rows; yb < TY; yb += A.stride * rows) {
+        const int t0 = yb * A.TX, nt = min(A.ntiles - t0, rows * A.TX);
+        const uint32_t* row = A.hist + (size_t)grp * A.ntiles + t0;
+        if (yb != band0 * rows) __syncthreads();  // the last band's places are dealt out
+        for (int t = threadIdx.x; t < nt; t += blockDim.x) h[t] = A.start[t0 + t] + row[t];
+        __syncthreads();
+        for (int64_t kb = k0; kb < k1; kb += blockDim.x) {
+            const int64_t k = kb + threadIdx.x;
+            int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
+            float depth = 0.f;
+            if (k < k1) {
+                const uint2 r = __ldg(A.rects + k);
+                x0 = (int)(r.x & 0xffffu);
+                x1 = (int)(r.x >> 16);
+                y0 = max((int)(r.y & 0xffffu), yb);
+                y1 = max(min((int)(r.y >> 16), yb + rows), y0);
+                if (x1 > x0 && y1 > y0)
+                    depth = DT == GS_F32 ? __ldg(reinterpret_cast<const float*>(A.splats) + 12 * (size_t)k + 6)
+                                         : __ldg(reinterpret_cast<const float*>(A.splats) + 8 * (size_t)k + 2);
+            }
+            const uint32_t kw = (uint32_t)(kb + (threadIdx.x & ~31u));  // the id: lane o's Gaussian is kw + o
+            warp_rect_tiles(x0, y0 - yb, x1 - x0, y1 - y0, __float_as_uint(depth),
+                            [&](int tx, int ty, uint32_t d, uint32_t o) {
+                const u64 pos = (u64)atomicAdd(h + ty * A.TX + tx, 1u);
+                if ((int64_t)pos < A.cap) A.keys[pos] = ((u64)d << 32) | (u64)(kw + o);
+            });
         }
-        const uint32_t kw = (uint32_t)(kb + (threadIdx.x & ~31u));  // the id: lane o's Gaussian is kw + o
-        warp_rect_tiles(x0, y0 - yb, x1 - x0, y1 - y0, __float_as_uint(depth), [&](int tx, int ty, uint32_t d, uint32_t o) {
-            const u64 pos = (u64)atomicAdd(h + ty * A.TX + tx, 1u);
-            if ((int64_t)pos < A.cap) A.keys[pos] = ((u64)d << 32) | (u64)(kw + o);
-        });
     }
 }
 
@@ -451,18 +476,14 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter_rects(const Scatte
     scatter_rects_body<DT>(A, (int)blockIdx.x);
 }
 
-// Tile rows per band of the scatter (see ScatterArgs): one band for every 20
-// MB of keys the capacity allows, at most 6 (every band reads the rects
-// again).  Scatter times by number of bands: 1200x680 / 1M (capacity 51 MB) 1
-// band 55 us, 2 43.7, 4 47, 7 60; 1296x968 / 750k (48 MB) 49, 2 40, 3 37, 6 44;
-// 1200x680 / 458k at stride 2 (22 MB) 21.7, 2 19.6; 1920x1080 / 3M (384 MB) 3
-// bands 307, 6 263, 12 277, 24 392.
-static int scatter_band(const Grid& g, int64_t cap) {
-    const int64_t per = 20 << 20;
-    const int64_t want = (cap * (int64_t)sizeof(u64) + per - 1) / per;
-    const int64_t bands = std::min<int64_t>(std::max<int64_t>(std::min<int64_t>(want, 6), 1), g.TY);
-    return (int)((g.TY + bands - 1) / bands);
-}
+static int scatter_max_rows(const Grid& g) { return std::min(std::max(SCATTER_SMEM_TILES / g.TX, 1), g.TY); }
+
+// Blocks for this many bands side by side: those of four keys a Gaussian (a
+// surface map at up to 1200x680), which the blocks go through in their order
+// (3M Gaussians 280 us, one block a group for all six bands 297); a block
+// returns at once where there are fewer bands and goes on to another where
+// there are more.
+static int scatter_stride(const Grid& g, int64_t n, int64_t cap) { return scatter_bands(std::min(cap, 4 * n), g.TY); }
 
 template <int DT>
 __global__ void __launch_bounds__(BIN_THREADS) k_tile_scatter(gs_camera cam, float alpha_min, const void* __restrict__ splats,
@@ -1224,11 +1245,11 @@ extern "C" gs_status gs_project_bin_sort(const gs_config* cfg, const gs_camera* 
     if ((s = check_launch("k_col_scan_tail")) != GS_OK) return s;
     if (keys_capacity == 0) return GS_OK;
     if ((s = set_agg_smem_attrs()) != GS_OK) return s;
-    const int band = scatter_band(grid, keys_capacity);
-    const ScatterArgs A = {grid.TX, splats, n, per, (int)nb, ntiles, band, start, hist, (const uint2*)rects, keys_capacity,
-                           (u64*)keys_out, tile_ranges, order, n_big};
-    const unsigned blocks = 1u + nb * (unsigned)((grid.TY + band - 1) / band);
-    const size_t sm = sizeof(uint32_t) * (size_t)grid.TX * (size_t)band;
+    const int rows = scatter_max_rows(grid), stride = scatter_stride(grid, n, keys_capacity);
+    const ScatterArgs A = {grid.TX, splats, n, per, (int)nb, ntiles, rows, stride, start, hist, (const uint2*)rects, keys_capacity,
+                           (u64*)keys_out, n_keys_out, tile_ranges, order, n_big};
+    const unsigned blocks = 1u + nb * (unsigned)stride;
+    const size_t sm = sizeof(uint32_t) * (size_t)grid.TX * (size_t)rows;
     if (rec_dtype == GS_F32) k_tile_scatter_rects<GS_F32><<<blocks, BIN_THREADS, sm, st>>>(A);
     else if (rec_dtype == GS_BF16) k_tile_scatter_rects<GS_BF16><<<blocks, BIN_THREADS, sm, st>>>(A);
     else k_tile_scatter_rects<GS_F16><<<blocks, BIN_THREADS, sm, st>>>(A);
@@ -1296,13 +1317,13 @@ gs_status wave_bin_sort(const gs_track_job* jobs, const WaveBin* bins, int n, cu
             const gs_track_job& t = jobs[j];
             const WaveBin& b = bins[j];
             const Grid g = make_grid(t.cam);
-            const int band = scatter_band(g, t.keys_capacity);
+            const int rows = scatter_max_rows(g), stride = scatter_stride(g, t.g.n, t.keys_capacity);
             W.start[j] = blocks;
-            blocks += 1 + (int)b.nb * ((g.TY + band - 1) / band);
-            smax = std::max(smax, g.TX * band);
-            W.job[j] = ScatterArgs{g.TX, t.splats, t.g.n, b.per, (int)b.nb, b.ntiles, band, b.start, b.hist,
-                                   (const uint2*)b.rects, t.keys_capacity, (u64*)t.keys, t.tile_ranges, t.tile_order,
-                                   b.n_big};
+            blocks += 1 + (int)b.nb * stride;
+            smax = std::max(smax, g.TX * rows);
+            W.job[j] = ScatterArgs{g.TX, t.splats, t.g.n, b.per, (int)b.nb, b.ntiles, rows, stride, b.start, b.hist,
+                                   (const uint2*)b.rects, t.keys_capacity, (u64*)t.keys, t.n_keys, t.tile_ranges,
+                                   t.tile_order, b.n_big};
         }
         W.start[n] = blocks;
         k_wave_scatter_rects<<<(unsigned)blocks, BIN_THREADS, sizeof(uint32_t) * (size_t)smax, st>>>(W);
