@@ -645,8 +645,10 @@ __device__ __noinline__ void merge_sort_group(const u64* src, u64* key, uint32_t
 // number of smaller keys there (neighbouring threads hold neighbouring
 // places, so they read the same few keys).  Surfaces cluster the depths:
 // about 8 keys share a bin on the tracking frame, 15 at 3M / 1920x1080.
-// A bin of more than DS_MAX_BIN keys (equal depths, a far outlier) sends the
-// bucket to the merge sort.  About 10 instructions a key and pass instead of
+// Keys of one depth (a wall parallel to the image) go by the range of their
+// ids instead: 3196 and 7223 equal depths a tile 99 -> 28 and 101 -> 33 us.  A
+// bin of more than DS_MAX_BIN keys (a far outlier) sends the bucket to the
+// merge sort.  About 10 instructions a key and pass instead of
 // 25 dependent shared-memory loads a key and merge round (8 to 12 rounds):
 // 640x480 / 200k (496 k keys) 34.5 -> 13.2 us, 1200x680 / 1M (4.2 M keys)
 // 145 -> 54 us, 1920x1080 / 3M (23.4 M keys) 896 -> 332 us (two CTAs per SM;
@@ -665,35 +667,47 @@ __device__ __forceinline__ void dist_sort_group(const u64* src, u64* key, uint32
     static_assert(1 << LOGM == M, "bins per group");
     const int lane = t & 31, w = t >> 5;
     u64 v[KPT];
-    uint32_t lo = ~0u, up = 0u;
 #pragma unroll
     for (int r = 0; r < KPT; ++r)
         if (t + r * TPG < n) v[r] = __ldcg(src + t + r * TPG);
 #pragma unroll
     for (int r = 0; r < KPT / 4; ++r) reinterpret_cast<uint4*>(bin)[t + r * TPG] = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t lo, up;
+    bool ids = false;  // one depth for all keys: the bins cut the range of their ids
+    auto word = [&](u64 k) { return ids ? (uint32_t)k : (uint32_t)(k >> 32); };
+    auto range = [&] {
+        lo = ~0u;
+        up = 0u;
 #pragma unroll
-    for (int r = 0; r < KPT; ++r)
-        if (t + r * TPG < n) {
-            lo = min(lo, (uint32_t)(v[r] >> 32));
-            up = max(up, (uint32_t)(v[r] >> 32));
+        for (int r = 0; r < KPT; ++r)
+            if (t + r * TPG < n) {
+                lo = min(lo, word(v[r]));
+                up = max(up, word(v[r]));
+            }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        up = __reduce_max_sync(0xffffffffu, up);
+        if (W > 1) {
+            if (lane == 0) {
+                red[w] = lo;
+                red[W + w] = up;
+            }
+            group_bar(bar, TPG);
+            lo = __reduce_min_sync(0xffffffffu, lane < W ? red[lane] : ~0u);
+            up = __reduce_max_sync(0xffffffffu, lane < W ? red[W + lane] : 0u);
+        } else {
+            __syncwarp();
         }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    up = __reduce_max_sync(0xffffffffu, up);
-    if (W > 1) {
-        if (lane == 0) {
-            red[w] = lo;
-            red[W + w] = up;
-        }
+    };
+    range();
+    if (up == lo) {  // (group-uniform)
+        ids = true;
         group_bar(bar, TPG);
-        lo = __reduce_min_sync(0xffffffffu, lane < W ? red[lane] : ~0u);
-        up = __reduce_max_sync(0xffffffffu, lane < W ? red[W + lane] : 0u);
-    } else {
-        __syncwarp();
+        range();
     }
     const int sh = max(0, 32 - __clz(up - lo) - LOGM);  // (up - lo) >> sh < M
 #pragma unroll
     for (int r = 0; r < KPT; ++r)
-        if (t + r * TPG < n) atomicAdd(bin + (((uint32_t)(v[r] >> 32) - lo) >> sh), 1u);
+        if (t + r * TPG < n) atomicAdd(bin + ((word(v[r]) - lo) >> sh), 1u);
     group_bar(bar, TPG);
     // exclusive scan of the counts, 8 consecutive bins a thread
     uint4 b0 = reinterpret_cast<const uint4*>(bin)[2 * t], b1 = reinterpret_cast<const uint4*>(bin)[2 * t + 1];
@@ -729,12 +743,12 @@ __device__ __forceinline__ void dist_sort_group(const u64* src, u64* key, uint32
     group_bar(bar, TPG);
 #pragma unroll
     for (int r = 0; r < KPT; ++r)
-        if (t + r * TPG < n) buf[atomicAdd(bin + (((uint32_t)(v[r] >> 32) - lo) >> sh), 1u)] = v[r];
+        if (t + r * TPG < n) buf[atomicAdd(bin + ((word(v[r]) - lo) >> sh), 1u)] = v[r];
     group_bar(bar, TPG);
     // bin[c] now ends bin c, so bin c starts at bin[c - 1]
     for (int p = t; p < n; p += TPG) {
         const u64 k = buf[p];
-        const uint32_t c = ((uint32_t)(k >> 32) - lo) >> sh;
+        const uint32_t c = (word(k) - lo) >> sh;
         const int q0 = c ? (int)bin[c - 1] : 0, q1 = (int)bin[c];
         int pos = q0;
         for (int q = q0; q < q1; ++q) pos += buf[q] < k ? 1 : 0;
@@ -796,30 +810,39 @@ __device__ __forceinline__ void tile_sort_body(const uint32_t* __restrict__ rang
     if (per == 2) return dist_sort_group<256>(key, key, val, n, hi, buf, bin, red, t, 1 + g);
     if (n <= TS_KEYS) return dist_sort_group<512>(key, key, val, n, hi, buf, bin, red, t, 1);
     // Longer buckets: the keys are first placed bin by bin in tmp (4096 bins
-    // over the depth range), then slabs of whole bins, each starting in its
+    // over the range of the depths, or the ids of one depth), then slabs of whole bins, each starting in its
     // own 2048 places (so at most 2048 keys and one bin), are sorted alone.
     if (n <= TS_DIST_KEYS) {
-        uint32_t lo = ~0u, up = 0u;
         for (int i = tid; i < TS_KEYS; i += TS_THREADS) bins[i] = 0u;
-        for (int i = tid; i < n; i += TS_THREADS) {
-            const uint32_t d = (uint32_t)(__ldcg(key + i) >> 32);
-            lo = min(lo, d);
-            up = max(up, d);
-        }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        up = __reduce_max_sync(0xffffffffu, up);
         constexpr int W = TS_THREADS / 32;
         const int lane = tid & 31, w = tid >> 5;
-        if (lane == 0) {
-            s_red[w] = lo;
-            s_red[W + w] = up;
+        uint32_t lo, up;
+        bool ids = false;  // as in dist_sort_group
+        auto word = [&](u64 k) { return ids ? (uint32_t)k : (uint32_t)(k >> 32); };
+        for (;;) {
+            lo = ~0u;
+            up = 0u;
+            for (int i = tid; i < n; i += TS_THREADS) {
+                const uint32_t d = word(__ldcg(key + i));
+                lo = min(lo, d);
+                up = max(up, d);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            up = __reduce_max_sync(0xffffffffu, up);
+            if (lane == 0) {
+                s_red[w] = lo;
+                s_red[W + w] = up;
+            }
+            __syncthreads();
+            lo = __reduce_min_sync(0xffffffffu, lane < W ? s_red[lane] : ~0u);
+            up = __reduce_max_sync(0xffffffffu, lane < W ? s_red[W + lane] : 0u);
+            if (up != lo) break;  // (CTA-uniform; ids differ)
+            ids = true;
+            __syncthreads();
         }
-        __syncthreads();
-        lo = __reduce_min_sync(0xffffffffu, lane < W ? s_red[lane] : ~0u);
-        up = __reduce_max_sync(0xffffffffu, lane < W ? s_red[W + lane] : 0u);
         const int sh = max(0, 32 - __clz(up - lo) - 12);
         for (int i = tid; i < n; i += TS_THREADS)
-            atomicAdd(bins + (((uint32_t)(__ldcg(key + i) >> 32) - lo) >> sh), 1u);
+            atomicAdd(bins + ((word(__ldcg(key + i)) - lo) >> sh), 1u);
         __syncthreads();
         uint32_t c[8], sum = 0u, big = 0u;
 #pragma unroll
@@ -861,7 +884,7 @@ __device__ __forceinline__ void tile_sort_body(const uint32_t* __restrict__ rang
             u64* const place = tmp + b;
             for (int i = tid; i < n; i += TS_THREADS) {
                 const u64 k = __ldcg(key + i);
-                place[atomicAdd(bins + (((uint32_t)(k >> 32) - lo) >> sh), 1u)] = k;
+                place[atomicAdd(bins + ((word(k) - lo) >> sh), 1u)] = k;
             }
             __threadfence_block();
             __syncthreads();
