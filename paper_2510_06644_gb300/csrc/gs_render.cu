@@ -1924,18 +1924,18 @@ static gs_status smem_once(const void* fn, int id, int bytes) {
 // 100k Gaussians, 300 tiles 117 against 38 us, 1200 62 / 62, 3225 44 / 146 --
 // but its products and sums round differently, which moves stops and the
 // signs of L1 residuals.)
-// Backward with masks, for which both kernels give the same sums to float32
-// rounding: the one-warp CTAs do less work, the entry-parallel kernel's 8 or
-// 16 warps a tile finish it sooner, which counts while the tiles do not fill
-// the chip.  One-warp against entry-parallel, us (100k Gaussians):
-//   stride 2x2  300 tiles 67 / 55, 1200 41 / 67, 3225 40 / 162
-//   stride 4x2  300 tiles 77 / 57, 1200 44 / 35, 3225 38 / 70
-//   stride 4x4  300 tiles 64 / 36, 1200 39 / 24, 3225 36 / 46
-// (measured before the entry-parallel kernel read a batch's mask words at once:
-// it gained 2 to 20 % since, most on few tiles)
+// Backward with masks, for which both kernels form the same float32 terms: the
+// one-warp CTAs do less work, the entry-parallel kernel's 8 or 16 warps a tile
+// finish it sooner, which counts while the tiles do not fill the chip.
+// One-warp against entry-parallel, us (200k Gaussians; 50k and 600k cross at the
+// same numbers of tiles):
+//   stride 2x2   384 tiles 72 / 49,  638 63 / 50,  800 62 / 56, 1000 57 / 66
+//   stride 4x2  1200 tiles 56 / 44, 1600 58 / 50, 1920 55 / 59, 2160 51 / 63
+//   stride 4x4  1200 tiles 49 / 29, 1920 47 / 38, 2160 46 / 41, 2640 45 / 47
 static bool fwd_entry_parallel(const Grid& g) { return g.tw * g.th <= 64; }
 static bool bwd_entry_parallel(const Grid& g, bool masks, int tiles) {  // tiles: of the launch
-    return g.tw * g.th <= 64 && (!masks || tiles < (g.tw * g.th == 64 ? 512 : 2048));
+    const int pixels = g.tw * g.th;
+    return pixels <= 64 && (!masks || tiles < (pixels == 64 ? 896 : pixels == 32 ? 1792 : 2560));
 }
 
 template <int DT>
