@@ -66,7 +66,9 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_count(gs_camera cam, float
 //   k_tile_scatter_rows  CTA c starts tile t's slots at start[t] +
 //                    hist[c][t] and deals them out with shared-memory atomics.
 #define AGG_MAX_TILES 8192
-#define AGG_ROWS 912         // one wave of six counting CTAs on 152 SMs
+// (A constant, not the device's count: it shapes the workspace, whose size is
+// asked for before the device that runs the call may be current.)
+#define AGG_ROWS 912         // rows of a large map: one wave of six counting CTAs on 152 SMs
 
 template <int DT>
 __global__ void __launch_bounds__(BIN_THREADS) k_tile_hist(gs_camera cam, float alpha_min, const void* __restrict__ splats, int64_t n,
@@ -88,9 +90,9 @@ __global__ void __launch_bounds__(BIN_THREADS) k_tile_hist(gs_camera cam, float 
     for (int t = threadIdx.x; t < ntiles; t += blockDim.x) row[t] = h[t];
 }
 
-// Column scan of the per-CTA rows: CTA b takes 32 tiles; its 32 warps split
-// the rows into 32 consecutive ranges, sum them, scan the 32 partial sums in
-// shared memory and write each row's exclusive prefix in place.
+// Column scan of the per-CTA rows: CTA b takes CS_TILES tiles; its threads
+// split the rows into CS_GROUPS consecutive ranges, sum them, scan the partial
+// sums in shared memory and write each row's exclusive prefix in place.
 __device__ __forceinline__ void col_scan_body(uint32_t* __restrict__ hist, int nrows, int ntiles,
                                               uint32_t* __restrict__ total, int blk) {
     // CTA: CS_TILES tiles x (1024 / CS_TILES) row groups of consecutive rows
@@ -992,8 +994,10 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // Gaussians per CTA of the aggregated passes: two per thread (half the
 // rows of one per thread for the column scan, and 782 -> 391 CTAs fit one
 // wave: projection + binning + sort 63.6-64.6 -> 61.6-62.5 us on the
-// tracking frame; four per thread 72.8-74.8), or more when the per-CTA rows
-// would pass 2^24 entries (64 MB).
+// tracking frame; four per thread 72.8-74.8).  On larger maps as many as make
+// the rows one wave (AGG_ROWS; figures at k_project_hist): rows beyond it cost
+// the column scan a pass each (3M Gaussians / 8160 tiles, 1824 rows 41.6 us, 912
+// 26.5).  More when the rows would pass 2^24 entries (64 MB).
 static int64_t agg_per_cta(int64_t n, int ntiles) {
     const int64_t lim = (int64_t)1 << 24;
     int64_t want = (n * (int64_t)ntiles + lim - 1) / lim;

@@ -251,9 +251,10 @@ __device__ __forceinline__ Geom load_geom(const void* base, uint32_t k) {
 // 0.  (Three divisions and a root made the fused map step issue-bound, 3485
 // instructions a warp of Gaussians, zeros through the slow paths: 1.5M
 // Gaussians of which 40 % have gradients 246 -> 172 us; the fewer divisions
-// without the test for 0: 280.)  As many roundings as the first form, every
-// operation on its own (no contraction), so gs_adam and the Adam step fused
-// into the backward projection give the same bits.
+// without the test for 0: 280.)  An element has as many roundings as before,
+// and its two factors one or two of their own.  No operation is contracted, so
+// gs_adam and the Adam step fused into the backward projection give the same
+// bits from the same gradients.
 struct AdamStep {
     float lr_c1, rs_c2;  // lr / c1, 1 / sqrt(c2)
 };

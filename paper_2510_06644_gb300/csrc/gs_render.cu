@@ -40,8 +40,7 @@
 namespace gs {
 
 #define R_THREADS 256            // largest CTA (16x16 tile)
-#define R_BATCH 1024             // largest batch of entries a tile stages at a time
-#define R_MASKW (R_BATCH / 32)   // mask words of a batch (at most 32: lane q holds word q)
+#define R_BATCH 1024             // largest batch of entries a tile stages at a time (32 mask words: lane q holds word q)
 #define R_BWD_SMEM (70 * 1024)          // backward staging budget per CTA (512 entries: 51 KB, 4 CTAs per SM)
 
 #define EP_B 256     // entries an entry-parallel tile stages per batch (64-pixel
@@ -297,7 +296,7 @@ __device__ __forceinline__ void stage_batch(const void* __restrict__ splats, con
 // is set when entry 32q + e (below `limit`) meets the block.  Lane q returns
 // word q (words at or beyond `words` are zero), so a word is one shuffle away
 // and the masks stay in registers.  Only the words that hold entries are
-// built (a loop to the batch's last word rather than over all R_MASKW:
+// built (a loop to the batch's last word rather than over all 32:
 // tracking step 236.6 -> 231.5 us).
 __device__ __forceinline__ unsigned warp_masks(const StagedSplat* sp, int limit, int words, const PixelMap& m) {
     const int lane = threadIdx.x & 31;
@@ -759,12 +758,15 @@ struct FragGeo {
 };
 
 // The geometry of a staged entry at the pixel, with the forward's arithmetic
-// (so the same alpha); `blended` says whether the forward blended it.
-__device__ __forceinline__ FragGeo frag_geo_at(const StagedSplat& s, float pxc, float pyc, const gs_config& cfg,
-                                               bool blended) {
+// (so the same alpha).  Without blend masks the decision is re-derived: inside
+// the box, exponent <= 0, alpha >= alpha_min, before the pixel's last blended
+// position.
+__device__ __forceinline__ FragGeo frag_geo(const StagedSplat& s, const PixelMap& m, float pxc, float pyc,
+                                            const gs_config& cfg, bool before_last) {
     FragGeo f;
     const float4 A = s.a;
     const float4 Bv = s.b;
+    const int4 box = s.box;
     f.dep = Bv.z;
     f.dx = pxc - A.x;
     f.dy = pyc - A.y;
@@ -774,16 +776,6 @@ __device__ __forceinline__ FragGeo frag_geo_at(const StagedSplat& s, float pxc, 
     f.q = Qd.q;
     f.raw = raw_alpha(Qd.q, Bv.w);
     f.alpha = fminf(cfg.alpha_max, f.raw);
-    f.contrib = blended;
-    return f;
-}
-
-// Without blend masks the decision is re-derived: inside the box, exponent
-// <= 0, alpha >= alpha_min, before the pixel's last blended position.
-__device__ __forceinline__ FragGeo frag_geo(const StagedSplat& s, const PixelMap& m, float pxc, float pyc,
-                                            const gs_config& cfg, bool before_last) {
-    FragGeo f = frag_geo_at(s, pxc, pyc, cfg, false);
-    const int4 box = s.box;
     f.contrib = before_last && (unsigned)(m.px - box.x) <= (unsigned)box.y &&
                 (unsigned)(m.py - box.z) <= (unsigned)box.w && !(f.q < 0.f) && !(f.alpha < cfg.alpha_min);
     return f;
@@ -1315,9 +1307,9 @@ __global__ void __launch_bounds__(32, PW_CTAS)
 // ---------------------------------------------------------------------------
 // Entry-parallel compositing for the small tiles of downsampled frames
 // ---------------------------------------------------------------------------
-// With both strides >= 2 a tile holds at most 8x8 sampled pixels but covers
-// the same full-resolution area, hence the same list length, as a 16x16
-// tile: pixel-parallel warps would walk long lists with few (and far apart)
+// With a stride of 2 in both axes or of 4 in one a tile holds at most 64
+// sampled pixels but covers the same full-resolution area, hence the same
+// list length, as a 16x16 tile: pixel-parallel warps would walk long lists with few (and far apart)
 // pixels.  Here one CTA of W warps serves a tile (W = 8 for up to 32
 // pixels, else 16) and warp w takes PPW = ceil(pixels / W) of its pixels
 // (2 to 4), one at a time.  For its pixel the warp first compacts the staged
@@ -1342,7 +1334,6 @@ struct EpStageN {
     float4 c[NB];    // r, g, b, -
     int4 box[NB];    // pixel box
 };
-typedef EpStageN<EP_B> EpStage;
 
 template <int W>
 struct EpFwdBatch {
@@ -1385,14 +1376,14 @@ __device__ __forceinline__ bool ep_may_blend(const EpStageN<NB>& S, int e, int p
 // outside the image have h = 0.  perm[w * ppw + j] is warp w's j-th pixel.
 // Any h gives a valid permutation; it only changes which warp does what.
 template <int W>
-__device__ __forceinline__ void ep_pair(const Grid& g, int tile, int q0, int npix, const uint32_t* hint,
+__device__ __forceinline__ void ep_pair(const Grid& g, int tile, int npix, const uint32_t* hint,
                                         uint32_t* s_h, uint8_t* perm) {
     const int ppw = (npix + W - 1) / W;
     const int q = (int)threadIdx.x;
     if (q < npix) {
         int i, j;
         uint32_t h = 0;
-        if (hint && ep_pixel(g, tile, q0 + q, i, j)) h = hint[(size_t)j * g.Ws + i];
+        if (hint && ep_pixel(g, tile, q, i, j)) h = hint[(size_t)j * g.Ws + i];
         s_h[q] = h;
     }
     __syncthreads();
@@ -1410,24 +1401,24 @@ __device__ __forceinline__ void ep_pair(const Grid& g, int tile, int q0, int npi
     __syncthreads();
 }
 
-// Forward compositing of pixels q0 .. q0 + npix - 1 of `tile` by the CTA's W
-// warps, entry-parallel (S: staging; cbuf_all: W compaction buffers).
+// Forward compositing of the pixels of `tile` by the CTA's W warps,
+// entry-parallel (S: staging; cbuf_all: W compaction buffers).
 template <int DT, int W, int NB>
 __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
-                                       const FwdOut& O, int tile, int q0, int npix, EpStageN<NB>& S,
+                                       const FwdOut& O, int tile, EpStageN<NB>& S,
                                        int (*cbuf_all)[64], uint32_t* s_h, uint8_t* perm,
                                        uint32_t (*bm_all)[NB / 32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
     int* cbuf = cbuf_all[warp];
-    const int ppw = (npix + W - 1) / W;
+    const int npix = g.tw * g.th, ppw = (npix + W - 1) / W;
     const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
     // out_last still holds the previous iteration's positions (read before any write)
-    ep_pair<W>(g, tile, q0, npix, cfg.balance ? O.last : nullptr, s_h, perm);
+    ep_pair<W>(g, tile, npix, cfg.balance ? O.last : nullptr, s_h, perm);
     // lane j < ppw holds the state of the warp's pixel j
     int mi, mj;
-    const bool mine = lane < ppw && warp * ppw + lane < npix && ep_pixel(g, tile, q0 + perm[warp * ppw + lane], mi, mj);
+    const bool mine = lane < ppw && warp * ppw + lane < npix && ep_pixel(g, tile, perm[warp * ppw + lane], mi, mj);
     float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, D = 0.f;
     uint32_t last = 0, nb = 0;
     bool done = !mine;
@@ -1441,7 +1432,7 @@ __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, cons
         for (int j = 0; j < ppw; ++j) {
             if (__shfl_sync(0xffffffffu, done, j)) continue;
             int pi, pj;
-            ep_pixel(g, tile, q0 + perm[warp * ppw + j], pi, pj);
+            ep_pixel(g, tile, perm[warp * ppw + j], pi, pj);
             const int px = pi * g.sx, py = pj * g.sy;
             const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
             float Tj = __shfl_sync(0xffffffffu, T, j);
@@ -1519,7 +1510,7 @@ __device__ __forceinline__ void fwd_ep(const gs_config& cfg, const Grid& g, cons
             if (!stopped && cnt > 0) composite(cnt);
             __syncwarp();
             if (O.bmask && lane < ((n_in + 31) >> 5))
-                O.bmask[bm_tile + 64 * (size_t)(((b - start) >> 5) + lane) + (q0 + perm[warp * ppw + j])] = bmw[lane];
+                O.bmask[bm_tile + 64 * (size_t)(((b - start) >> 5) + lane) + perm[warp * ppw + j]] = bmw[lane];
             p0 = warp_sum(p0);
             p1 = warp_sum(p1);
             p2 = warp_sum(p2);
@@ -1559,7 +1550,7 @@ __device__ __forceinline__ void fwd_ep_cta(const gs_config& cfg, const Grid& g, 
     extern __shared__ __align__(16) unsigned char r_smem[];
     EpFwdSmem<W, NB>& M = *reinterpret_cast<EpFwdSmem<W, NB>*>(r_smem);
     const int tile = order ? (int)__ldg(order + blk) : blk;
-    fwd_ep<DT, W, NB>(cfg, g, splats, vals, ranges, O, tile, 0, g.tw * g.th, M.S, M.cbuf, M.s_h, M.perm, M.bm);
+    fwd_ep<DT, W, NB>(cfg, g, splats, vals, ranges, O, tile, M.S, M.cbuf, M.s_h, M.perm, M.bm);
 }
 
 template <int DT, int W>
@@ -1594,7 +1585,7 @@ struct EpBwdSmem {
     uint32_t s_max;
 };
 
-// Backward compositing of pixels q0 .. q0 + npix - 1 of `tile` by the CTA's
+// Backward compositing of the pixels of `tile` by the CTA's
 // W warps, entry-parallel.
 template <int DT, int MODE, int W>
 __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
@@ -1602,7 +1593,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
                                        const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
                                        const float* __restrict__ d_rgb, const float* __restrict__ d_depth,
                                        float* __restrict__ grad2d, const uint32_t* __restrict__ bmask, int tile,
-                                       int q0, int npix, EpBwdSmem<MODE, W>& M) {
+                                       EpBwdSmem<MODE, W>& M) {
     constexpr int NF = EpFields<MODE>::N;
     constexpr int NB = EpFwdBatch<W>::N;
     EpStageN<NB>& S = M.S;
@@ -1612,12 +1603,12 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned gt_mask = lane == 31 ? 0u : ~0u << (lane + 1);
     int* cbuf = M.cbuf[warp];
-    const int ppw = (npix + W - 1) / W;
+    const int npix = g.tw * g.th, ppw = (npix + W - 1) / W;
     const uint32_t start = ranges[2 * tile], end = ranges[2 * tile + 1];
     uint8_t* perm = M.perm;
-    ep_pair<W>(g, tile, q0, npix, last_idx, M.s_h, perm);
+    ep_pair<W>(g, tile, npix, last_idx, M.s_h, perm);
     int mi, mj;
-    const bool mine = lane < ppw && warp * ppw + lane < npix && ep_pixel(g, tile, q0 + perm[warp * ppw + lane], mi, mj);
+    const bool mine = lane < ppw && warp * ppw + lane < npix && ep_pixel(g, tile, perm[warp * ppw + lane], mi, mj);
     // state of pixel `lane`: T after the part already walked, the colour
     // behind it dotted with g, last blended position, image gradient g
     float T = 1.f, sdot = 0.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, gd = 0.f;
@@ -1655,7 +1646,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
             const uint32_t lastj = __shfl_sync(0xffffffffu, last, j);
             if (lastj <= base_pos) continue;  // nothing blended in this batch
             const int nj = (int)min((uint32_t)n_in, lastj - base_pos);
-            const int qj = q0 + perm[warp * ppw + j];  // the pixel's index in the tile
+            const int qj = perm[warp * ppw + j];  // the pixel's index in the tile
             int pi, pj;
             ep_pixel(g, tile, qj, pi, pj);
             const int px = pi * g.sx, py = pj * g.sy;
@@ -1789,8 +1780,7 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 4 : 2)
     extern __shared__ __align__(16) unsigned char r_smem[];
     EpBwdSmem<MODE, W>& M = *reinterpret_cast<EpBwdSmem<MODE, W>*>(r_smem);
     const int tile = order ? (int)__ldg(order + blockIdx.x) : (int)blockIdx.x;
-    bwd_ep<DT, MODE, W>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, 0,
-                        g.tw * g.th, M);
+    bwd_ep<DT, MODE, W>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, M);
 }
 
 // ---------------------------------------------------------------------------
@@ -1890,7 +1880,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 2)
     const int blk = (int)blockIdx.x - W.start[j];
     const int tile = J.order ? (int)__ldg(J.order + blk) : blk;
     bwd_ep<GS_F32, GS_TRACK, NW>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb, J.d_depth,
-                                 J.grad2d, J.bmask, tile, 0, J.g.tw * J.g.th, M);
+                                 J.grad2d, J.bmask, tile, M);
 }
 
 }  // namespace gs
