@@ -307,10 +307,11 @@ gs_status gs_render_fwd_loss(const gs_config* cfg, const gs_camera* cam, int rec
  * (Eq. 3 differentiated; the printed Eq. 4 omits T_k and the normalisation);
  * then through alpha = opacity exp(power) to opacity, conic and 2D mean
  * unless alpha was clamped.  Per-fragment gradients are summed per Gaussian
- * inside each warp; with blend_masks (pixel-parallel frames) each warp's
- * sums go to grad2d with one global atomic per (Gaussian, warp, field),
- * otherwise they are summed per tile in shared memory first (one atomic per
- * (Gaussian, tile, field)).
+ * inside each warp; with blend_masks each warp's sums go to grad2d with one
+ * global atomic per (Gaussian, warp, field), without them -- and in strided
+ * frames of few tiles of at most 64 sampled pixels -- they are summed per tile
+ * in shared memory first (one atomic per (Gaussian, tile, field)).  Every
+ * path forms the same float32 terms.
  * grad2d [n][12] float (GS_GRAD2D_STRIDE layout): zeroed by this call.
  * mode GS_TRACK skips dL/dopacity and dL/drgb (not needed for the pose).
  * If grads, pose_grad6 or score_terms is non-NULL, gs_project_bwd runs as

@@ -1109,8 +1109,8 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 // of sum (Q d) h is three times as far from 64 bits on a needle.
 //
 // They go straight to grad2d, one atomic per (entry, field, warp): the warps
-// of a tile share nothing and run as one-warp CTAs
-// that the hardware schedules as they free up, heavy tiles first.
+// of a tile share nothing and run as one-warp CTAs that the hardware schedules
+// as they free up, heavy tiles first.
 template <int DT, int MODE>
 __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
@@ -1280,10 +1280,10 @@ __device__ __forceinline__ void bwd_pw(const gs_config& cfg, const Grid& g, cons
     }
 }
 
-// One-warp CTAs of the masked backward per SM: 24 (78 registers).  us of the
-// kernel, tracking 640x480 / 200k, 1200x680 / 458k at 2x2, mapping 1200x680 /
-// 1M and 1920x1080 / 1M f16: 20 a SM 69, 63, 239 and 491; 24 69, 65, 229 and
-// 464; 28 72, 67, 228 and 460.  (One float32 butterfly per two to four entries
+// One-warp CTAs of the masked backward per SM: 24 (75 registers, mapping 80).
+// us of the kernel, tracking 640x480 / 200k, 1200x680 / 458k at 2x2, mapping
+// 1200x680 / 1M and 1920x1080 / 1M f16: 20 a SM 69, 63, 235 and 483; 24 69, 65,
+// 224 and 457; 28 72, 67, 227 and 457.  (One float32 butterfly per two to four entries
 // instead of the sums through shared memory: 85, 79, 260 and 535.)
 #define PW_CTAS 24
 
