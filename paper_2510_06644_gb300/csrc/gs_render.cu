@@ -407,10 +407,10 @@ __device__ __forceinline__ void add_loss(const FwdOut& O, float part) {
 // scalar operation), the alpha test, transmittance and blending entry by entry, each
 // lane's box test one bit of the slot's mask.
 //
-// Issue-bound (68 % issue-active, then barriers and fixed latencies): box tests
+// Issue-bound (64 % issue-active, then barriers and fixed latencies): box tests
 // of four words in every lane, scalar geometry and steps of three entries
 // padded with dummies took 74 instructions a (warp, entry) visit, 65.9 M for
-// the tracking frame, against 43.3 M now.  Forward + loss 640x480 / 200k 84 ->
+// the tracking frame, against 41.4 M now.  Forward + loss 640x480 / 200k 84 ->
 // 61.4 us, forward 1200x680 / 1M 180 -> 100, 1296x968 / 750k bf16 232 -> 144.
 // Measured and not kept: records by cp.async a batch ahead (raw records
 // in shared memory cost each warp their unpacking: 61.4 / 105.8 / 152.7), the
@@ -1107,6 +1107,12 @@ __device__ __forceinline__ void back_pair(BackState& S, const PwRing& R, int pai
 // the block's centre (block / Gaussian)^2 of them (a Gaussian of 0.55 px: 1.6e-6
 // relative at stride 1, 2e-5 at 4x4, against 1e-7), and Q sum h d in place
 // of sum (Q d) h is three times as far from 64 bits on a needle.
+//
+// Shared memory bounds it: 107 k wavefronts an SM in 142 k cycles on the
+// tracking frame, 275 k in 346 k mapping 1200x680 / 1M, at 57 and 62 %
+// issue-active (48.9 M and 129 M warp instructions).  All ten mapping terms
+// as eight-byte words, without the weights' part, took 257 us at 1M against
+// 229.
 //
 // They go straight to grad2d, one atomic per (entry, field, warp): the warps
 // of a tile share nothing and run as one-warp CTAs that the hardware schedules
