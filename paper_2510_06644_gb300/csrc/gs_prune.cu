@@ -358,11 +358,14 @@ __global__ void __launch_bounds__(PR_THREADS) k_change(gs_camera cam, float alph
     }
 }
 
+__host__ __device__ constexpr int compact_rows(int w) { return w == 1 ? 1024 : w == 2 ? 512 : 256; }
+
 // Rows of a parameter array to their places in the compacted one; W floats a
-// row (1 to 4 as constants: 0 takes any width).  A block moves 256 rows, so the
+// row (1 to 4 as constants: 0 takes any width).  A block moves ROWS rows, so the
 // row of an element is a 32-bit division by a constant and every load of the
-// block is in flight at once.  One 64-bit division an element made it
-// instruction-bound: 1M rows of 3 floats 11.3 us, now 6.3 (29 MB moved).
+// block is in flight at once, three or four elements a thread (1M rows of 3
+// floats, a 64-bit division an element 8.5 us, now 5.5; 3M rows of 1, 256 rows a
+// block 10.9, now 5.4).
 template <int W>
 __global__ void __launch_bounds__(256) k_compact(const float* __restrict__ src, int64_t n, int width,
                                                  const uint32_t* __restrict__ map, float* __restrict__ dst) {
@@ -376,20 +379,20 @@ __global__ void __launch_bounds__(256) k_compact(const float* __restrict__ src, 
         }
         return;
     }
-    constexpr int WC = W > 0 ? W : 1;
-    for (int64_t r0 = (int64_t)blockIdx.x * 256; r0 < n; r0 += (int64_t)gridDim.x * 256) {
-        const unsigned int rows = (unsigned int)(n - r0 < 256 ? n - r0 : 256);
-        uint32_t to[WC];
-        float v[WC];
+    constexpr int WC = W > 0 ? W : 1, ROWS = compact_rows(W), E = WC * ROWS / 256;
+    for (int64_t r0 = (int64_t)blockIdx.x * ROWS; r0 < n; r0 += (int64_t)gridDim.x * ROWS) {
+        const unsigned int rows = (unsigned int)(n - r0 < ROWS ? n - r0 : ROWS);
+        uint32_t to[E];
+        float v[E];
 #pragma unroll
-        for (int j = 0; j < WC; ++j) {
+        for (int j = 0; j < E; ++j) {
             const unsigned int e = threadIdx.x + 256u * j;
             const bool in = e < rows * WC;
             to[j] = in ? __ldg(map + r0 + e / WC) : 0xFFFFFFFFu;
             v[j] = in ? __ldg(src + r0 * WC + e) : 0.f;
         }
 #pragma unroll
-        for (int j = 0; j < WC; ++j)
+        for (int j = 0; j < E; ++j)
             if (to[j] != 0xFFFFFFFFu) dst[(int64_t)to[j] * WC + (threadIdx.x + 256u * j) % WC] = v[j];
     }
 }
@@ -525,7 +528,8 @@ extern "C" gs_status gs_compact(const float* src, int64_t n, int32_t width, cons
     if (n == 0) return GS_OK;
     if (!src || !compact_map || !dst) return set_error(GS_ERR_INVALID_ARG, "NULL pointer");
     const int sms = num_sms();
-    const int64_t want = width <= 4 ? (n + 255) / 256 : (n * width + 255) / 256;
+    const int rows = compact_rows(width);
+    const int64_t want = width <= 4 ? (n + rows - 1) / rows : (n * width + 255) / 256;
     const int64_t cap = (int64_t)(width <= 4 ? 64 : 8) * sms;
     const unsigned nb = (unsigned)(want < cap ? want : cap);
     cudaStream_t st = (cudaStream_t)stream;
