@@ -1064,8 +1064,17 @@ static gs_status set_agg_smem_attrs() {
     return GS_OK;
 }
 
+// Most CTAs of the bucket sort that lists of up to cap keys in all can fill
+// (tile_sort_body's classes: one, two, four or 16 tiles a CTA).  A CTA a tile left
+// a grid of 47 k tiles and 28 k keys with 44 k CTAs that only look their 
+// up (88 us, now 17).
+static int64_t sort_blocks(int ntiles, int64_t cap) {
+    const int64_t most = cap / 2049 + (cap / 1025 + 1) / 2 + (cap / 257 + 3) / 4 + (ntiles + 15) / 16;
+    return std::min<int64_t>(ntiles, most);
+}
+
 // The bucket sort of the scattered keys, heavy tiles first.
-static gs_status launch_tile_sort(int ntiles, const uint32_t* tile_ranges, const uint32_t* order,
+static gs_status launch_tile_sort(int ntiles, int64_t cap, const uint32_t* tile_ranges, const uint32_t* order,
                                   const uint32_t* n_big, uint64_t* keys_out, uint32_t* vals_out, u64* tmp,
                                   cudaStream_t st) {
     // once per device (not repeated while a graph is being captured)
@@ -1078,7 +1087,7 @@ static gs_status launch_tile_sort(int ntiles, const uint32_t* tile_ranges, const
             return set_error(GS_ERR_CUDA, "cudaFuncSetAttribute(k_tile_sort)");
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
-    k_tile_sort<<<(unsigned)ntiles, TS_THREADS, TS_SMEM, st>>>(
+    k_tile_sort<<<(unsigned)sort_blocks(ntiles, cap), TS_THREADS, TS_SMEM, st>>>(
         tile_ranges, order, n_big, ntiles, (u64*)keys_out, vals_out, tmp);
     return check_launch("k_tile_sort");
 }
@@ -1216,7 +1225,7 @@ extern "C" gs_status gs_bin_sort(const gs_config* cfg, const gs_camera* cam, int
             k_tile_scatter<GS_F16><<<nb, BIN_THREADS, 0, st>>>(*cam, alpha_min, splats, n, start, fill, keys_capacity, (u64*)keys_out);
         if ((s = check_launch("k_tile_scatter")) != GS_OK) return s;
     }
-    return launch_tile_sort(ntiles, tile_ranges, order, n_big, keys_out, vals_out, tmp, st);
+    return launch_tile_sort(ntiles, keys_capacity, tile_ranges, order, n_big, keys_out, vals_out, tmp, st);
 }
 
 // Projection and binning in one call: gs_project, then gs_bin_sort with
@@ -1281,7 +1290,7 @@ extern "C" gs_status gs_project_bin_sort(const gs_config* cfg, const gs_camera* 
     else if (rec_dtype == GS_BF16) k_tile_scatter_rects<GS_BF16><<<blocks, BIN_THREADS, sm, st>>>(A);
     else k_tile_scatter_rects<GS_F16><<<blocks, BIN_THREADS, sm, st>>>(A);
     if ((s = check_launch("k_tile_scatter_rects")) != GS_OK) return s;
-    return launch_tile_sort(ntiles, tile_ranges, order, n_big, keys_out, vals_out, tmp, st);
+    return launch_tile_sort(ntiles, keys_capacity, tile_ranges, order, n_big, keys_out, vals_out, tmp, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1373,7 +1382,7 @@ gs_status wave_bin_sort(const gs_track_job* jobs, const WaveBin* bins, int n, cu
             const gs_track_job& t = jobs[j];
             const WaveBin& b = bins[j];
             W.start[j] = blocks;
-            blocks += b.ntiles;
+            blocks += (int)sort_blocks(b.ntiles, t.keys_capacity);
             W.job[j] = WaveSortJob{t.tile_ranges, t.tile_order, b.n_big, b.ntiles, (u64*)t.keys, t.vals, (u64*)b.tmp};
         }
         W.start[n] = blocks;
