@@ -1929,9 +1929,18 @@ static gs_status smem_once(const void* fn, int id, int bytes) {
 //   stride 4x2  1200 tiles 56 / 44, 1600 58 / 50, 1920 55 / 59, 2160 51 / 63
 //   stride 4x4  1200 tiles 49 / 29, 1920 47 / 38, 2160 46 / 41, 2640 45 / 47
 static bool fwd_entry_parallel(const Grid& g) { return g.tw * g.th <= 64; }
-static bool bwd_entry_parallel(const Grid& g, bool masks, int tiles) {  // tiles: of the launch
+// On tiles of 64 pixels, lists of a few dozen entries leave the entry-parallel
+// kernel's 16 warps a tile without work, and its CTAs, two an SM, go in rounds
+// (300 tiles: 1000 Gaussians 4.7 / 10.5, 4000 8.1 / 11.6, 8000 14.1 / 12.9, 16000 26.5
+// / 18.3; 638 tiles: 16000 18.5 / 29.0, 50k 41 / 37): it takes 24 Gaussians a tile
+// and round.
+// tiles, n: of the launch
+static bool bwd_entry_parallel(const Grid& g, bool masks, int tiles, int64_t n) {
     const int pixels = g.tw * g.th;
-    return pixels <= 64 && (!masks || tiles < (pixels == 64 ? 896 : pixels == 32 ? 1792 : 2560));
+    if (pixels > 64 || !masks) return pixels <= 64;
+    if (pixels < 64) return tiles < (pixels == 32 ? 1792 : 2560);
+    const int round = 2 * num_sms();
+    return tiles < 896 && n >= (int64_t)24 * tiles * ((tiles + round - 1) / round);
 }
 
 template <int DT>
@@ -1968,14 +1977,14 @@ template <int DT, int MD>
 static gs_status launch_bwd(const gs_config& cfg, const Grid& g, const void* splats, const uint32_t* vals,
                             const uint32_t* ranges, const uint32_t* order, const float* t_final,
                             const uint32_t* last_idx, const float* d_rgb, const float* d_depth, float* grad2d,
-                            const uint32_t* bmask, cudaStream_t st) {
+                            const uint32_t* bmask, int64_t n, cudaStream_t st) {
     const int ntiles = g.TX * g.TY;
-    if (bmask && !bwd_entry_parallel(g, true, ntiles)) {  // one-warp CTAs
+    if (bmask && !bwd_entry_parallel(g, true, ntiles, n)) {  // one-warp CTAs
         k_render_bwd_pw<DT, MD><<<(unsigned)ntiles * (unsigned)pw_warps(g), 32, 0, st>>>(
             cfg, g, splats, vals, ranges, order, t_final, last_idx, d_rgb, d_depth, grad2d, bmask);
         return check_launch("k_render_bwd_pw");
     }
-    if (bwd_entry_parallel(g, bmask != nullptr, ntiles)) {
+    if (bwd_entry_parallel(g, bmask != nullptr, ntiles, n)) {
         gs_status s;
         const int id = 18 + 4 * (MD == GS_MAP) + DT;  // + 0 or 8 below: W
         if (g.tw * g.th <= 32) {
@@ -2118,7 +2127,7 @@ extern "C" gs_status gs_render_bwd(const gs_config* cfg, const gs_camera* cam, c
     if (n > 0) {
 #define GS_LB(DT, MD) \
     launch_bwd<DT, MD>(*cfg, g, splats, vals, tile_ranges, tile_order, t_final, last_idx, d_rgb, d_depth, grad2d, \
-                       blend_masks, st)
+                       blend_masks, n, st)
         if (mode == GS_MAP)
             s = rec_dtype == GS_F32 ? GS_LB(GS_F32, GS_MAP) : rec_dtype == GS_BF16 ? GS_LB(GS_BF16, GS_MAP)
                                                                                    : GS_LB(GS_F16, GS_MAP);
@@ -2192,13 +2201,17 @@ gs_status wave_render(const gs_config& cfg, const gs_track_job* jobs, int n, cud
     // launches by each session's own tiles); both kernels form the same float32
     // terms, so a session's gradients move by their rounding alone.
     int masked = 0;
+    int64_t masked_n = 0;
     for (int j = 0; j < n; ++j) {
         const Grid g = make_grid(jobs[j].cam);
-        if (jobs[j].blend_masks) masked += g.TX * g.TY;
+        if (jobs[j].blend_masks) {
+            masked += g.TX * g.TY;
+            masked_n += jobs[j].g.n;
+        }
     }
-    auto bwd_kind = [masked](const gs_track_job& t) {
+    auto bwd_kind = [masked, masked_n](const gs_track_job& t) {
         const Grid g = make_grid(t.cam);
-        if (bwd_entry_parallel(g, t.blend_masks != nullptr, masked)) return g.tw * g.th <= 32 ? 2 : 3;
+        if (bwd_entry_parallel(g, t.blend_masks != nullptr, masked, masked_n)) return g.tw * g.th <= 32 ? 2 : 3;
         return t.blend_masks ? 4 : (R_THREADS / tile_threads(g) == 1 ? 0 : 1);
     };
     int kinds = 0;

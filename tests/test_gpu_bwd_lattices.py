@@ -58,3 +58,25 @@ def test_small_tiles_at_step_edges(G, n, sx, sy, mode):
             assert not g2[1][:, cols].any()
         else:
             assert rel_l2(g2[1][:, cols], g2[0][:, cols]) <= TOL, (cols, rel_l2(g2[1][:, cols], g2[0][:, cols]))
+
+
+@pytest.mark.parametrize("n", [7199, 7200])
+def test_either_side_of_the_line_between_the_kernels(G, n):
+    """300 tiles of 64 pixels: with 24 Gaussians a tile the entry-parallel
+    kernel takes over from the one-warp CTAs."""
+    W, H = 320, 240
+    cam = S.camera(W, H, 100.0, sx=2, sy=2)
+    s = S.splats(n, W, H, seed=n, opaque_frac=0.02)
+    rec, cs, cfg = pack_splats(s), G.camera(cam), G.default_config()
+    cap = int(G.gs_bin_count(cs, rec, n, cfg=cfg).item())
+    _, vals, _, ranges, order = G.gs_bin_sort(cs, rec, n, cap)
+    bm = torch.zeros(G.gs_blend_mask_words(cs, cap), dtype=torch.int32, device="cuda")
+    out = G.gs_render_fwd(cfg, cs, rec, n, vals, ranges, order=order, masks=bm)
+    d_rgb, d_dep = (torch.from_numpy(x).cuda() for x in S.image_grads(W // 2, H // 2, n))
+    z = dev({"means": np.zeros((n, 3), np.float32), "log_scales": np.zeros((n, 3), np.float32),
+             "quats": np.zeros((n, 4), np.float32), "opacity_logit": np.zeros(n, np.float32),
+             "rgb": np.zeros((n, 3), np.float32)})
+    g2 = [np_of(G.gs_render_bwd(cfg, cs, z, rec, vals, ranges, out["t_final"], out["last_idx"], d_rgb, d_dep,
+                                mode=G.GS_MAP, order=order, masks=k)) for k in (None, bm)]
+    for cols in ([0, 1], [2, 3, 4], [5], [6], [8, 9, 10]):
+        assert rel_l2(g2[1][:, cols], g2[0][:, cols]) <= TOL, (cols, rel_l2(g2[1][:, cols], g2[0][:, cols]))
