@@ -1591,9 +1591,10 @@ struct EpBwdSmem {
     uint32_t s_max;
 };
 
-// Backward compositing of the pixels of `tile` by the CTA's
-// W warps, entry-parallel.
-template <int DT, int MODE, int W>
+// Backward compositing of the pixels of `tile` by the CTA's W warps,
+// entry-parallel.  MASKED: from the forward's blend masks (a test inside the
+// loops cost the other form 1 to 5 %).
+template <int DT, int MODE, int W, bool MASKED>
 __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, const void* __restrict__ splats,
                                        const uint32_t* __restrict__ vals, const uint32_t* __restrict__ ranges,
                                        const float* __restrict__ t_final, const uint32_t* __restrict__ last_idx,
@@ -1638,7 +1639,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
     if (lane == 0) atomicMax(&s_max, wl);
     __syncthreads();
     const uint32_t tile_last = s_max;
-    const uint32_t* bm_tile = bmask ? bmask + blend_mask_base_ep(tile, start) : nullptr;
+    const uint32_t* bm_tile = MASKED ? bmask + blend_mask_base_ep(tile, start) : nullptr;
     // batches [start + k NB, start + (k + 1) NB) from the last one holding a
     // blended entry back to the first
     for (int kb = (int)((tile_last + NB - 1) / NB) - 1; kb >= 0; --kb) {
@@ -1659,11 +1660,11 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
             const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
             // the pixel's blend mask from the forward (entries it blended),
             // else its pixel box, selects the entries to compact
-            const uint32_t* bmj = bm_tile ? bm_tile + 64 * (size_t)(base_pos >> 5) + qj : nullptr;
+            const uint32_t* bmj = MASKED ? bm_tile + 64 * (size_t)(base_pos >> 5) + qj : nullptr;
             // (lane r takes run r's word, at most 32 a batch: a load a run in
             // the loop below waits for each; 300 tiles of 32 pixels, 50k / 200k
             // Gaussians 47.8 / 68.7 us, now 35.0 / 52.3)
-            const uint32_t mw = bmj && lane < ((nj + 31) >> 5) ? __ldg(bmj + 64 * lane) : 0u;
+            const uint32_t mw = MASKED && lane < ((nj + 31) >> 5) ? __ldg(bmj + 64 * lane) : 0u;
             float Tj = __shfl_sync(0xffffffffu, T, j);
             float sj = __shfl_sync(0xffffffffu, sdot, j);
             // the pixel's image gradient
@@ -1740,8 +1741,8 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
             int cnt = 0;
             for (int c = (nj - 1) & ~31; c >= 0; c -= 32) {
                 const int e = c + lane;
-                const uint32_t word = __shfl_sync(0xffffffffu, mw, c >> 5);
-                const bool in = e < nj && (bmj ? ((word >> lane) & 1u) != 0u : ep_may_blend(S, e, px, py));
+                const uint32_t word = MASKED ? __shfl_sync(0xffffffffu, mw, c >> 5) : 0u;
+                const bool in = e < nj && (MASKED ? ((word >> lane) & 1u) != 0u : ep_may_blend(S, e, px, py));
                 const unsigned m = __ballot_sync(0xffffffffu, in);
                 if (in) cbuf[cnt + __popc(m & gt_mask)] = e;
                 cnt += __popc(m);
@@ -1776,7 +1777,7 @@ __device__ __forceinline__ void bwd_ep(const gs_config& cfg, const Grid& g, cons
     }
 }
 
-template <int DT, int MODE, int W>
+template <int DT, int MODE, int W, bool MASKED>
 __global__ void __launch_bounds__(W * 32, W == 8 ? 4 : 2)
     k_render_bwd_ep(gs_config cfg, Grid g, const void* __restrict__ splats, const uint32_t* __restrict__ vals,
                     const uint32_t* __restrict__ ranges, const uint32_t* __restrict__ order,
@@ -1786,7 +1787,8 @@ __global__ void __launch_bounds__(W * 32, W == 8 ? 4 : 2)
     extern __shared__ __align__(16) unsigned char r_smem[];
     EpBwdSmem<MODE, W>& M = *reinterpret_cast<EpBwdSmem<MODE, W>*>(r_smem);
     const int tile = order ? (int)__ldg(order + blockIdx.x) : (int)blockIdx.x;
-    bwd_ep<DT, MODE, W>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile, M);
+    bwd_ep<DT, MODE, W, MASKED>(cfg, g, splats, vals, ranges, t_final, last_idx, d_rgb, d_depth, grad2d, bmask, tile,
+                                M);
 }
 
 // ---------------------------------------------------------------------------
@@ -1885,8 +1887,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 2)
     const WaveBwdJob& J = W.job[j];
     const int blk = (int)blockIdx.x - W.start[j];
     const int tile = J.order ? (int)__ldg(J.order + blk) : blk;
-    bwd_ep<GS_F32, GS_TRACK, NW>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb, J.d_depth,
-                                 J.grad2d, J.bmask, tile, M);
+    if (J.bmask)
+        bwd_ep<GS_F32, GS_TRACK, NW, true>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb,
+                                           J.d_depth, J.grad2d, J.bmask, tile, M);
+    else
+        bwd_ep<GS_F32, GS_TRACK, NW, false>(cfg, J.g, J.splats, J.vals, J.ranges, J.t_final, J.last_idx, J.d_rgb,
+                                            J.d_depth, J.grad2d, nullptr, tile, M);
 }
 
 }  // namespace gs
@@ -1904,7 +1910,7 @@ static int group_batch(int gpc, int bytes_per_entry, int budget) {
 // Raises a kernel's dynamic shared-memory limit once per device and
 // instantiation (not repeated while a graph is being captured).
 static gs_status smem_once(const void* fn, int id, int bytes) {
-    static bool done[64][48] = {};  // ids: bwd 6-17, entry-parallel bwd 18-33, waves 42-45
+    static bool done[64][64] = {};  // ids: bwd 6-17, entry-parallel bwd 18-33 (masked 46-61), waves 42-45
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && done[dev][id]) return GS_OK;
@@ -1986,19 +1992,18 @@ static gs_status launch_bwd(const gs_config& cfg, const Grid& g, const void* spl
     }
     if (bwd_entry_parallel(g, bmask != nullptr, ntiles, n)) {
         gs_status s;
-        const int id = 18 + 4 * (MD == GS_MAP) + DT;  // + 0 or 8 below: W
-        if (g.tw * g.th <= 32) {
-            const int sm = (int)sizeof(EpBwdSmem<MD, 8>);
-            if ((s = smem_once((const void*)k_render_bwd_ep<DT, MD, 8>, id, sm)) != GS_OK) return s;
-            k_render_bwd_ep<DT, MD, 8><<<ntiles, 8 * 32, sm, st>>>(cfg, g, splats, vals, ranges, order, t_final,
-                                                                    last_idx, d_rgb, d_depth, grad2d, bmask);
-        } else {
-            const int sm = (int)sizeof(EpBwdSmem<MD, 16>);
-            if ((s = smem_once((const void*)k_render_bwd_ep<DT, MD, 16>, id + 8, sm)) != GS_OK) return s;
-            k_render_bwd_ep<DT, MD, 16><<<ntiles, 16 * 32, sm, st>>>(cfg, g, splats, vals, ranges, order,
-                                                                      t_final, last_idx, d_rgb, d_depth, grad2d,
-                                                                      bmask);
-        }
+        const int id = (bmask ? 46 : 18) + 4 * (MD == GS_MAP) + DT;  // + 0 or 8 below: W
+#define GS_EP(W, M)                                                                                             \
+    {                                                                                                           \
+        const int sm = (int)sizeof(EpBwdSmem<MD, W>);                                                           \
+        if ((s = smem_once((const void*)k_render_bwd_ep<DT, MD, W, M>, W == 8 ? id : id + 8, sm)) != GS_OK)     \
+            return s;                                                                                           \
+        k_render_bwd_ep<DT, MD, W, M><<<ntiles, W * 32, sm, st>>>(cfg, g, splats, vals, ranges, order, t_final, \
+                                                                   last_idx, d_rgb, d_depth, grad2d, bmask);    \
+    }
+        if (g.tw * g.th <= 32) { if (bmask) GS_EP(8, true) else GS_EP(8, false) }
+        else { if (bmask) GS_EP(16, true) else GS_EP(16, false) }
+#undef GS_EP
         return check_launch("k_render_bwd_ep");
     }
     const int gpc = R_THREADS / tile_threads(g);
