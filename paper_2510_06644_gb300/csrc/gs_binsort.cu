@@ -1066,8 +1066,8 @@ static gs_status set_agg_smem_attrs() {
 
 // Most CTAs of the bucket sort that lists of up to cap keys in all can fill
 // (tile_sort_body's classes: one, two, four or 16 tiles a CTA).  A CTA a tile left
-// a grid of 47 k tiles and 28 k keys with 44 k CTAs that only look their 
-// up (88 us, now 17).
+// a grid of 47 k tiles and 28 k keys with 44 k CTAs that only look for their
+// class (88 us, now 17).
 static int64_t sort_blocks(int ntiles, int64_t cap) {
     const int64_t most = cap / 2049 + (cap / 1025 + 1) / 2 + (cap / 257 + 3) / 4 + (ntiles + 15) / 16;
     return std::min<int64_t>(ntiles, most);
