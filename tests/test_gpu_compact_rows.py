@@ -14,8 +14,7 @@ def test_compact_keeps_the_unmasked_rows(n, width):
     from paper_2510_06644_gb300 import build
     build.build()
     from paper_2510_06644_gb300 import gs as G
-    if n * width > 40_000_000:
-        pytest.skip("one and three floats a row are enough at this size")
+    n = min(n, 36_000_000 // width)
     gen = torch.Generator(device="cuda").manual_seed(n)
     src = torch.rand(n, width, generator=gen, device="cuda")
     keep = torch.rand(n, generator=gen, device="cuda") < 0.7
